@@ -270,8 +270,12 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   with the full 1-D stiffness K = D^T W D (3 (N+1) multiply-adds per
  *   node).  Without it, for odd N <= 9, they use the even-odd form of the
  *   centrosymmetric W^-1 K (Solomonoff's decomposition; half-length
- *   contractions, about a quarter fewer operations per node); results
- *   differ by rounding only.
+ *   contractions, about a quarter fewer operations per node), and the FP64
+ *   kernels of degrees 4..7 (except the batched solver's) evaluate the
+ *   contractions exactly in 58-bit fixed point relative to each element's
+ *   largest value, on the tensor cores (an element whose values are not
+ *   finite, lie outside [2^-900, 2^900] or differ too much in size takes
+ *   the direct FP64 sums); results differ by rounding only.
  * Problems with geometric factors (bs_problem_create_geo) always use their
  * own unfused FP64 kernel.  Returns the previous mode; a negative value only
  * queries it.  Not thread-safe against solves in flight. */

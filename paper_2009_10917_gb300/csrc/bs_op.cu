@@ -88,6 +88,143 @@ static void stiffness_1d(int N, const double *w, const double *D, double *K) {
     }
 }
 
+// A double-double value (hi + lo), for the tables that need more than 53 bits
+// (Dekker's and Knuth's error-free transformations, std::fma for products).
+struct DD {
+  double h, l;
+  DD(double a = 0.0, double b = 0.0) : h(a), l(b) {}
+};
+static DD dd_fast(double a, double b) {
+  const double s = a + b;
+  return DD(s, b - (s - a));
+}
+static DD operator+(DD a, DD b) {
+  const double s = a.h + b.h, t = s - a.h;
+  const double e = (a.h - (s - t)) + (b.h - t);
+  return dd_fast(s, e + (a.l + b.l));
+}
+static DD operator-(DD a) { return DD(-a.h, -a.l); }
+static DD operator-(DD a, DD b) { return a + (-b); }
+static DD operator*(DD a, DD b) {
+  const double p = a.h * b.h;
+  return dd_fast(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+static DD operator/(DD a, DD b) {
+  const double q = a.h / b.h;
+  const DD r = a - b * DD(q);
+  return dd_fast(q, (r.h + r.l) / b.h);
+}
+
+// The digits of Kh = W^-1 K (bs_op_fx.cuh), from GLL nodes, weights and
+// derivative matrix redone in double-double (Newton on the nodes x, as
+// gll_tables): a 58-bit entry holds more than a double, and an error common to
+// every element would shift the operator's low modes coherently.  Each entry
+// becomes an integer of at most 58 bits, the diagonal minus the rest of its
+// row (the rows sum to zero, as K's do), then signed 10-bit digits by the bias of 512
+// per digit that the kernel uses for its values, as the bits of a half.
+static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t) {
+  const int Nq = N + 1;
+  DD x[kMaxNq], w[kMaxNq], D[kMaxNq][kMaxNq], Kh[kMaxNq][kMaxNq];
+  auto legendre = [&](DD z, DD *pn, DD *pm) {  // P_N, P_{N-1}
+    DD p0(1.0), p1 = z;
+    for (int k = 2; k <= N; ++k) {
+      const DD p2 = (DD(2.0 * k - 1.0) * z * p1 - DD(k - 1.0) * p0) / DD(k);
+      p0 = p1;
+      p1 = p2;
+    }
+    *pn = p1;
+    *pm = p0;
+  };
+  for (int i = 0; i < Nq; ++i) {
+    DD pn, pm;
+    x[i] = DD(x0[i]);
+    for (int it = 0; it < 3; ++it) {
+      legendre(x[i], &pn, &pm);
+      x[i] = x[i] - (x[i] * pn - pm) / (DD(Nq) * pn);
+    }
+    legendre(x[i], &pn, &pm);
+    w[i] = DD(2.0) / (DD((double)N * Nq) * pn * pn);
+  }
+  DD b[kMaxNq];
+  for (int j = 0; j < Nq; ++j) {
+    DD p(1.0);
+    for (int k = 0; k < Nq; ++k)
+      if (k != j) p = p * (x[j] - x[k]);
+    b[j] = DD(1.0) / p;
+  }
+  for (int a = 0; a < Nq; ++a) {
+    DD diag;
+    for (int i = 0; i < Nq; ++i)
+      if (i != a) {
+        D[a][i] = (b[i] / b[a]) / (x[a] - x[i]);
+        diag = diag - D[a][i];
+      }
+    D[a][a] = diag;
+  }
+  double big = 0.0;
+  for (int i = 0; i < Nq; ++i)
+    for (int m = 0; m < Nq; ++m) {
+      DD s;
+      for (int a = 0; a < Nq; ++a) s = s + D[a][i] * w[a] * D[a][m];
+      Kh[i][m] = s / w[i];
+      big = std::fmax(big, std::fabs(Kh[i][m].h));
+    }
+  int e = 0;
+  std::frexp(big, &e);  // big < 2^e
+  t->q = 58 - e;
+  int64_t Ki[kMaxNq][kMaxNq];
+  for (int i = 0; i < Nq; ++i) {
+    int64_t rest = 0;
+    for (int m = 0; m < Nq; ++m) {
+      const double hi = std::ldexp(Kh[i][m].h, t->q), n = std::rint(hi);
+      Ki[i][m] = (int64_t)n + (int64_t)std::rint((hi - n) + std::ldexp(Kh[i][m].l, t->q));
+      if (m != i) rest += Ki[i][m];
+    }
+    Ki[i][i] = -rest;
+  }
+  int64_t bias = 0;
+  for (int d = 0; d < kFxDigits; ++d) bias += (int64_t)512 << (10 * d);
+  auto digit = [&](int i, int m, int d) {
+    return (int)(((bias + Ki[i][m]) >> (10 * (kFxDigits - 1 - d))) & 0x3ff) - 512;
+  };
+  // the largest sum an accumulator can meet: digits of a value up to 257
+  // (the first) or 512 in magnitude, products a + b = o of one row
+  for (int o = 0; o < kFxDigits; ++o)
+    for (int i = 0; i < Nq; ++i) {
+      int64_t s = 0;
+      for (int a = 0; a <= o; ++a)
+        for (int m = 0; m < Nq; ++m) s += (a ? 512 : 257) * std::abs(digit(i, m, o - a));
+      if (s > (o == kFxDigits - 1 ? 1 << 23 : 1 << 22)) return false;
+    }
+  auto half_bits = [](int v) -> uint32_t {  // |v| <= 512
+    if (v == 0) return 0;
+    const uint32_t sign = v < 0 ? 0x8000u : 0u, a = (uint32_t)(v < 0 ? -v : v);
+    int p = 31;
+    while (!(a >> p)) --p;
+    return sign | ((uint32_t)(p + 15) << 10) | ((a << (10 - p)) & 0x3ffu);
+  };
+  for (int d = 0; d < kFxDigits; ++d)
+    for (int lane = 0; lane < 32; ++lane) {
+      uint32_t word = 0;
+      for (int hf = 0; hf < 2; ++hf) {
+        const int i = lane >> 2, m = 2 * (lane & 3) + hf;
+        if (i < Nq && m < Nq) word |= half_bits(digit(i, m, d)) << (16 * hf);
+      }
+      t->w[d][lane] = word;
+    }
+  const DD g(0.5 * h), ml = DD(lambda) * g * g * g;
+  for (int k = 0; k < Nq; ++k)
+    for (int lane = 0; lane < 32; ++lane)
+      for (int hf = 0; hf < 2; ++hf) {
+        const int i = 2 * (lane & 3) + hf, j = lane >> 2;
+        if (i >= Nq || j >= Nq) continue;
+        const DD w3 = w[i] * w[j] * w[k];
+        t->wg[(k * 32 + lane) * 2 + hf] = (w3 * g).h;
+        t->wm[(k * 32 + lane) * 2 + hf] = (w3 * ml).h;
+      }
+  return true;
+}
+
 // diag(A_L) per local node: c_e (h/2) (K_ii w_j w_k + w_i K_jj w_k + w_i w_j K_kk)
 // + lambda (h/2)^3 w_i w_j w_k.
 template <typename T>
@@ -225,6 +362,10 @@ int bs_problem_create(const bs_map *map, double h, double lambda, const double *
         split(e, tabff.Eeh[a * hq + m], tabff.Eel[a * hq + m]);
         split(o, tabff.Eoh[a * hq + m], tabff.Eol[a * hq + m]);
       }
+  }
+  if (Nq >= kFxMinNq && Nq <= kFxMaxNq && !fx_table(N, x, h, lambda, &tab.fx)) {
+    free(p);
+    return fail(BS_ERR_ARG, "bs_problem_create: digit tables of degree %d out of range", N);
   }
   for (int i = 0; i < Nq; ++i) {
     tab.w[i] = w[i];

@@ -35,6 +35,20 @@ namespace bs {
 
 constexpr int kMaxNq = 16;  // degrees 1..15
 
+// Digit tables of the fixed-point contractions (bs_op_fx.cuh), degrees
+// kFxMinNq - 1 .. kFxMaxNq - 1: w[b][lane] = digit b of Kh[g][2t] and
+// Kh[g][2t + 1] (g = lane / 4, t = lane % 4; Kh = W^-1 K, zero past Nq) as a
+// pair of halves; Kh = sum_b digit_b 2^(10 (5 - b)) 2^-q.
+constexpr int kFxDigits = 6;  // digits per operand, 10 bits each
+constexpr int kFxMinNq = 5, kFxMaxNq = 8;
+// wg, wm [k][lane][h]: (h/2) w_i w_j w_k and lambda (h/2)^3 w_i w_j w_k of the
+// node (2t + h, g, k), rounded once.
+struct __align__(16) FxTab {
+  uint32_t w[kFxDigits][32];
+  double wg[kFxMaxNq * 64], wm[kFxMaxNq * 64];
+  int q;
+};
+
 // Per-problem constant tables, in device memory.
 template <typename T>
 struct OpTab {
@@ -45,6 +59,7 @@ struct OpTab {
   // Ee[a*h + m] = (Kh_am + Kh_a,Nq-1-m) / 2, Eo[a*h + m] = (Kh_am - Kh_a,Nq-1-m) / 2.
   T Ee[(kMaxNq / 2) * (kMaxNq / 2)];
   T Eo[(kMaxNq / 2) * (kMaxNq / 2)];
+  FxTab fx;        // FP64 tables only
   int64_t ne, ng;  // the problem's E and N_G (index checks of the checked build)
 };
 
@@ -362,12 +377,21 @@ __global__ void __launch_bounds__(OpShape<NQ>::THREADS)
   }
 }
 
+}  // namespace bs
+
+#include "bs_op_fx.cuh"
+
+namespace bs {
+
 // Blocks of the element kernels for E elements of degree N (the fused
-// operator's partials hold one double per block).
-inline int64_t ax_blocks(int N, int64_t E) {
+// operator's partials hold one double per block); fx: the FP64 kernels, which
+// may take the fixed-point form.
+inline int64_t ax_blocks(int N, int64_t E, bool fx) {
   switch (N + 1) {
 #define BS_AXB(NQ)                                                      \
   case NQ:                                                              \
+    if (fx && use_fx<NQ>() && g_op_evenodd)                             \
+      return (E + FxShape<NQ>::EPB - 1) / FxShape<NQ>::EPB;             \
     return use_eo<NQ>() && g_op_evenodd                                 \
                ? (E + EoShape<NQ>::EPB - 1) / EoShape<NQ>::EPB          \
                : (E + OpShape<NQ>::EPB - 1) / OpShape<NQ>::EPB;
@@ -390,7 +414,16 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
   if (E == 0) return BS_OK;
 #define BS_AX_CASE(NQ)                                                                   \
   case NQ: {                                                                             \
-    if constexpr (use_eo<NQ>()) {                                                        \
+    if constexpr (use_fx<NQ>() && sizeof(T) == 8) {                                      \
+      if (g_op_evenodd) {                                                                \
+        const int vec = ((uintptr_t)out % 16 == 0) && (GATHER_IN || (uintptr_t)in % 16 == 0); \
+        using Sf = FxShape<NQ>;                                                          \
+        k_ax_fx<NQ, GATHER_IN, FUSED>                                                    \
+            <<<(unsigned)((E + Sf::EPB - 1) / Sf::EPB), Sf::THREADS, Sf::SMEM, s>>>(     \
+                E, order, ids, in, out, tab, coef, st, outG, partials, vec);             \
+        break;                                                                           \
+      }                                                                                  \
+    } else if constexpr (use_eo<NQ>()) {                                                 \
       if (g_op_evenodd) {                                                                \
         using Se = EoShape<NQ>;                                                          \
         const int64_t grid = (E + Se::EPB - 1) / Se::EPB;                                \

@@ -680,7 +680,7 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
     return launch_gather<T, DOT, Ep>(m, ApL, Ap, DOT ? p : nullptr, P->d_partials, P->d_counter,
                                      ep, st, s);
   return launch_gather_rows<T, DOT, Ep>(m, fused, ApL, Ap, DOT ? p : nullptr, P->d_partials,
-                                        P->d_counter, opp, opp ? ax_blocks(P->N, m->E) : 0, ep,
+                                        P->d_counter, opp, opp ? ax_blocks(P->N, m->E, sizeof(T) == 8 && !ff) : 0, ep,
                                         st, s);
 }
 

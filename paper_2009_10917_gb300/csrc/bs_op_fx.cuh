@@ -1,0 +1,525 @@
+// bs_op_fx.cuh -- the FP64 element operator of bs_op.cuh with its 1-D
+// contractions on the tensor cores, in exact fixed-point pieces.
+//
+// GB300 executes FP64 at 1/64 of its FP32 rate (about 2 DFMA per clock and
+// SM, tensor-core FP64 included), so the element operator, 24 FP64
+// operations per node even in its even-odd form, ran at 88% of that pipe
+// while HBM idled.  Here the contractions sum_m Kh_im u_m (Kh = W^-1 D^T W D)
+// are integer arithmetic (an error-free splitting of the kind of Ozaki,
+// Ogita, Oishi & Rump, Numer. Algorithms 59, 2012):
+//  - an element's values are taken as 58-bit integers relative to its largest
+//    exponent and cut into six signed 10-bit digits; so is Kh, on the host
+//    (FxTab);
+//  - a digit fits a half exactly, and mma.sync m16n8k16 sums the products of
+//    equal weight (order o = a + b, 48 at most) into an FP32 accumulator that
+//    starts at 1.5 * 2^23: with the actual digits of Kh every partial sum is
+//    an integer in [2^23, 2^24) (below 0.95 of the 2^22 either way for
+//    degrees up to 7, checked where the table is made), so nothing rounds and
+//    the accumulator's bits ARE the integer: no conversion instructions,
+//    which share the FP64 pipe.  Order 5, the last, would reach 1.22 and
+//    starts at 1.5 * 2^24 instead, counting by two; its low ten bits are
+//    dropped anyway;
+//  - orders 0..5 are joined into one 64-bit integer per node, the three
+//    directions summed there, and only then is there a double, put together
+//    by integer operations: two FP64 operations per node (the weighted sum
+//    and the mass term), three with a coefficient.
+// Dropped: u below 2^-58 of the element's largest power of two, orders >= 6
+// and the last ten bits, together about 2^-57 of the element's max|u| times
+// sum|Kh| per node.  The FP64 forms round relative to each line's own values,
+// up to (2 Nq + 4) 2^-53 of sum|Kh||u|; an element in which some column along
+// t (so some line of every node) stays more than 2^-8 below the element's
+// largest value therefore takes the FP64 sums.
+//
+// One or two warps per element, each with its own layers k (and planes j of
+// the t direction).  With g = lane / 4 and t = lane % 4, a lane owns the nodes
+// i = 2t, 2t + 1, j = g of its layers; its digit pairs are at once the A fragment of the contraction
+// along r (rows j of two layers, columns m; Kh^T as B), the transposed 8 x 8
+// layers the B fragment along s and the transposed (k, i) planes the one along
+// t, both by ldmatrix.trans from the digit planes in shared memory (row chunks
+// XOR-swizzled by k: stores and loads without bank conflicts).  Results along
+// r and s arrive in the owner's layout; those along t go through shared
+// memory.  Nq < 8 runs in the same 8 x 8 tiles, padded with zero digits.
+// The small tiles (K = 8 per digit) are why this is mma.sync and not tcgen05:
+// the tensor pipe is not what bounds it, and the accumulators are wanted in
+// registers at once.
+//
+// Measured (N = 7 on 36^3, 23.9M local nodes): A_L Z p 176 us, the even-odd
+// FP64 kernel 1047 us; HBM alone would allow 60 us.  What bounds it now is
+// spread out: issue slots 61%, integer pipe 55%, FP64 pipe 46%, L1 65%, HBM 26%.
+// Conversions by two FP64 additions per node (instead of fx_double) and the
+// weights multiplied node by node took 312 us with the FP64 pipe at 82%.
+// Error against extended precision on uniform inputs 1.4e-16 normwise (the
+// even-odd kernel 8.3e-16), after 64 CG iterations 1.7e-15 (2.8e-14).
+//
+// The FP64 sums (fx_direct) also serve an element whose largest value is not
+// finite or outside [2^-900, 2^900].
+#pragma once
+
+#include <type_traits>
+
+#include "bs_gather.cuh"
+
+namespace bs {
+
+constexpr int kFxRange = 8;          // log2 of the column range the digits serve
+constexpr uint32_t kFxMagicBits = 0x4B400000u;   // 1.5 * 2^23: counts by one
+constexpr uint32_t kFxMagic2Bits = 0x4BC00000u;  // 1.5 * 2^24: counts by two
+
+template <int NQ>
+constexpr bool use_fx() {
+  return NQ >= kFxMinNq && NQ <= kFxMaxNq;
+}
+
+// Two warps of four layers per element at Nq = 8 (72 registers, 14 elements per
+// SM: 176 us for 46656 elements, A_L Z p alone, against 180 with 80 registers,
+// 190 for one warp of eight layers, 196 for four of two), one warp below (the
+// last warp would idle: Nq = 5, 112 us against 147 for two layers per warp,
+// Nq = 6 139 against 150).
+template <int NQ>
+struct FxShape {
+  static constexpr int L = NQ == 8 ? 4 : (NQ + 1) / 2 * 2;  // layers per warp
+  static constexpr int WPE = (NQ + L - 1) / L;              // warps per element
+  static constexpr int EPB = 1;                             // elements per block
+  static constexpr int THREADS = 32 * WPE * EPB;
+  static constexpr int BLOCKS = NQ == 8 ? 14 : (NQ == 7 ? 20 : 24);  // resident per SM
+  static constexpr int PLANE = NQ * 8 * 16;       // bytes of one digit plane
+  static constexpr int DIG = kFxDigits * PLANE;
+  static constexpr int XCH = NQ * NQ * 64;        // [j][k][8 i] uint64
+  static constexpr int ELEM = DIG + XCH + (WPE > 1 ? WPE * 256 : 0);  // + columns' maxima
+  static constexpr int SMEM = EPB * ELEM;
+};
+
+// c += A B on a 16 x 8 tile, 16 digit products per entry, all exact.
+__device__ __forceinline__ void fx_mma(float *c, uint32_t a0, uint32_t a1, uint32_t a2,
+                                       uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// Start values of a tile's four sums (rows 0-7 twice, rows 8-15 twice) in
+// registers of their own, opaque to the compiler, which otherwise moves the
+// constants into place for every sum (3% of all instructions).
+struct FxStart {
+  float v[4];
+  __device__ __forceinline__ FxStart(uint32_t lo, uint32_t hi) {
+    asm volatile("mov.b32 %0, %1;\n" : "=f"(v[0]) : "r"(lo));
+    asm volatile("mov.b32 %0, %1;\n" : "=f"(v[1]) : "r"(lo));
+    asm volatile("mov.b32 %0, %1;\n" : "=f"(v[2]) : "r"(hi));
+    asm volatile("mov.b32 %0, %1;\n" : "=f"(v[3]) : "r"(hi));
+  }
+};
+// The first product of a sum: c = A B + start.
+__device__ __forceinline__ void fx_mma0(float *c, uint32_t a0, uint32_t a1, uint32_t a2,
+                                        uint32_t a3, uint32_t b0, uint32_t b1,
+                                        const FxStart &s) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%10,%11,%12,%13};\n"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(s.v[0]), "f"(s.v[1]),
+        "f"(s.v[2]), "f"(s.v[3]));
+}
+__device__ __forceinline__ void fx_ldsm4(uint32_t *r, uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void fx_ldsm4t(uint32_t *r, uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void fx_ldsm2t(uint32_t *r, uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
+               : "=r"(r[0]), "=r"(r[1])
+               : "r"(addr)
+               : "memory");
+}
+
+// x as an integer of 58 bits in units of 2^(emax - 1080), rounded to nearest,
+// plus 512 in every 10-bit digit (each digit of the result, less 512, is x's),
+// shifted left by one: the significand << 6, shifted down to emax with one
+// more bit, and for rounding 1 added (x >= 0) or its ones' complement taken.
+// Values whose exponent field is 0 (zero, subnormal) shift out entirely.
+__device__ __forceinline__ uint64_t fx_fixed(double x, int emax) {
+  const uint32_t hw = (uint32_t)__double2hiint(x), lw = (uint32_t)__double2loint(x);
+  const int d = min(emax - (int)((hw >> 20) & 0x7ffu), 63);
+  const uint64_t m = ((uint64_t)((hw & 0xfffffu) | 0x100000u) << 32 | lw) << 6;
+  const uint32_t sg = (uint32_t)((int32_t)hw >> 31);
+  constexpr uint64_t bias = 1024ull * (1ull + (1ull << 10) + (1ull << 20) + (1ull << 30) +
+                                       (1ull << 40) + (1ull << 50));
+  return ((m >> d) ^ ((uint64_t)sg << 32 | sg)) + (bias + 1ull);
+}
+
+// Digit A (0 = most significant) of two values of fx_fixed as a pair of halves.
+template <int A>
+__device__ __forceinline__ uint32_t fx_digit2(uint64_t x, uint64_t y) {
+  constexpr int S = 10 * (kFxDigits - 1 - A) + 1;
+  const uint32_t h =
+      (__byte_perm((uint32_t)(x >> S), (uint32_t)(y >> S), 0x5410) & 0x03ff03ffu) | 0x64006400u;
+  uint32_t r;  // halves 1024 + digit + 512, less 1536
+  asm("sub.f16x2 %0, %1, %2;\n" : "=r"(r) : "r"(h), "r"(0x66006600u));
+  return r;
+}
+
+// The orders' integer sums as one 64-bit integer in units of 2^10 of order 5
+// (whose accumulators count by two), rounded to nearest: a floor would bias
+// every node the same way.
+// Unsigned: the start values' bits may still be in the sums, modulo 2^64.
+__device__ __forceinline__ uint64_t fx_join(const uint32_t *s) {
+  uint64_t v = (uint64_t)(int64_t)((int)s[4] + ((int)(s[5] + 256u) >> 9));
+  v += (uint64_t)((int64_t)(int)s[3] * 1024);
+  v += (uint64_t)((int64_t)(int)s[2] * (1 << 20));
+  v += (uint64_t)((int64_t)(int)s[1] * (1 << 30));
+  v += (uint64_t)s[0] << 40;
+  return v;
+}
+
+// v 2^p as a double, rounded once (|v| < 2^62, the result normal or zero), by
+// integer operations alone: conversions and additions of doubles share the
+// FP64 pipe.  The significand's implicit bit adds one to the exponent field,
+// and so does a carry out of its rounding.
+__device__ __forceinline__ double fx_double(int64_t v, int p) {
+  const uint64_t a = (uint64_t)(v < 0 ? -v : v);
+  const uint32_t hi = (uint32_t)(a >> 32), lo = (uint32_t)a;
+  const int lz = __clz((int)(hi ? hi : lo)) + (hi ? 0 : 32);
+  const uint64_t m = ((a << ((lz - 1) & 63)) + 512u) >> 10;  // leading bit at 52
+  uint64_t b = m + ((uint64_t)(uint32_t)(p + 1085 - lz) << 52);
+  b = a ? b : 0;
+  return __longlong_as_double((int64_t)(b | ((uint64_t)v & 0x8000000000000000ull)));
+}
+
+// Direct FP64 sums of one element (values in x[], node order as in memory)
+// for the node (i, j, k): (W^-1 D^T W D applied along r, s and t).
+template <int NQ>
+__device__ __noinline__ double fx_direct(const double *x, const OpTab<double> *tab, int i, int j,
+                                         int k) {
+  const double *K = tab->K, *w = tab->w;
+  double ar = 0.0, as = 0.0, at = 0.0;
+  for (int m = 0; m < NQ; ++m) {
+    ar = fma(K[i * NQ + m], x[m + NQ * (j + NQ * k)], ar);
+    as = fma(K[j * NQ + m], x[i + NQ * (m + NQ * k)], as);
+    at = fma(K[k * NQ + m], x[i + NQ * (j + NQ * m)], at);
+  }
+  return (ar / w[i] + as / w[j]) + at / w[k];
+}
+
+// out = A_L in; arguments as k_ax_local (FUSED likewise).  vec: out (and,
+// without GATHER_IN, in) is 16-byte aligned.
+template <int NQ, bool GATHER_IN, bool FUSED>
+__global__ void __launch_bounds__(FxShape<NQ>::THREADS, FxShape<NQ>::BLOCKS)
+    k_ax_fx(int64_t E, const int32_t *__restrict__ order, const int32_t *__restrict__ ids,
+            const double *__restrict__ in, double *__restrict__ out,
+            const OpTab<double> *__restrict__ tab, const double *__restrict__ coef,
+            const CgState *st, double *__restrict__ outG, double *__restrict__ partials,
+            int vec) {
+  static_assert(!FUSED || GATHER_IN, "the fused operator reads its input through the map");
+  using S = FxShape<NQ>;
+  constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2, D = kFxDigits, L = S::L;
+  constexpr bool EVEN = NQ % 2 == 0;
+  extern __shared__ __align__(128) unsigned char fx_smem[];
+  if (cg_halted(st)) return;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int le = (int)threadIdx.x / (32 * S::WPE);  // the element's slot in the block
+  const int k0 = ((int)threadIdx.x / 32 - le * S::WPE) * L;  // this warp's first layer
+  unsigned char *dig = fx_smem + le * S::ELEM, *xch = dig + S::DIG;
+  uint32_t *col = reinterpret_cast<uint32_t *>(xch + S::XCH);
+  const uint32_t dig_s = (uint32_t)__cvta_generic_to_shared(dig);
+  auto sync = [&]() {  // the element's warps
+    if (S::WPE == 1)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;\n" ::"r"(1 + le), "n"(32 * S::WPE) : "memory");
+  };
+  Acc<double> acc;
+  const int64_t slot = (int64_t)blockIdx.x * S::EPB + le;
+  int64_t e = slot < E ? (order ? (int64_t)order[slot] : slot) : -1;
+  if (e >= 0 && !chk(bs_pred_index(e, tab->ne), BS_CHK_OP_ENTRY)) e = -1;
+  if (e >= 0) {
+    const bool on0 = g < NQ && 2 * t < NQ, on1 = g < NQ && 2 * t + 1 < NQ;
+    const int64_t base = e * NP + (int64_t)k0 * NQ2 + g * NQ + 2 * t;
+    auto layer = [&](int l) { return NQ % L == 0 || k0 + l < NQ; };
+    // ---- the values of nodes (2t, g, k0 + l), (2t + 1, g, k0 + l), l < L
+    double u0[L], u1[L];
+    int32_t id0[GATHER_IN ? L : 1], id1[GATHER_IN ? L : 1];
+    if (GATHER_IN) {
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        id0[l] = id1[l] = -1;
+        if (EVEN) {
+          if (on0 && layer(l)) {
+            const int2 q = __ldcs(reinterpret_cast<const int2 *>(ids + base + l * NQ2));
+            id0[l] = q.x;
+            id1[l] = q.y;
+          }
+        } else {
+          if (on0 && layer(l)) id0[l] = __ldcs(ids + base + l * NQ2);
+          if (on1 && layer(l)) id1[l] = __ldcs(ids + base + l * NQ2 + 1);
+        }
+        if (!chk(FUSED ? bs_pred_fused_entry(id0[l], tab->ng) : bs_pred_map_entry(id0[l], tab->ng),
+                 BS_CHK_OP_ENTRY))
+          id0[l] = -1;
+        if (!chk(FUSED ? bs_pred_fused_entry(id1[l], tab->ng) : bs_pred_map_entry(id1[l], tab->ng),
+                 BS_CHK_OP_ENTRY))
+          id1[l] = -1;
+      }
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        if (FUSED) {
+          u0[l] = id0[l] != -1 ? in[id0[l] >= 0 ? id0[l] : -2 - id0[l]] : 0.0;
+          u1[l] = id1[l] != -1 ? in[id1[l] >= 0 ? id1[l] : -2 - id1[l]] : 0.0;
+        } else {
+          u0[l] = id0[l] >= 0 ? in[id0[l]] : 0.0;
+          u1[l] = id1[l] >= 0 ? in[id1[l]] : 0.0;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        u0[l] = u1[l] = 0.0;
+        if (EVEN && vec) {
+          if (on0 && layer(l)) {
+            const double2 q = __ldcs(reinterpret_cast<const double2 *>(in + base + l * NQ2));
+            u0[l] = q.x;
+            u1[l] = q.y;
+          }
+        } else {
+          if (on0 && layer(l)) u0[l] = __ldcs(in + base + l * NQ2);
+          if (on1 && layer(l)) u1[l] = __ldcs(in + base + l * NQ2 + 1);
+        }
+      }
+    }
+    // ---- the columns' largest values (high words; 1 for a value whose high
+    // word is zero but which is not), the largest exponent, and whether the
+    // digits serve
+    uint32_t big0 = 0, big1 = 0;
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      big0 = max(big0, ((uint32_t)__double2hiint(u0[l]) & 0x7fffffffu) |
+                           min((uint32_t)__double2loint(u0[l]), 1u));
+      big1 = max(big1, ((uint32_t)__double2hiint(u1[l]) & 0x7fffffffu) |
+                           min((uint32_t)__double2loint(u1[l]), 1u));
+    }
+    if (S::WPE > 1) {
+      reinterpret_cast<uint2 *>(col)[k0 / L * 32 + lane] = make_uint2(big0, big1);
+      sync();
+#pragma unroll
+      for (int w = 0; w < S::WPE; ++w) {
+        const uint2 c = reinterpret_cast<const uint2 *>(col)[w * 32 + lane];
+        big0 = max(big0, c.x);
+        big1 = max(big1, c.y);
+      }
+    }
+    const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0, big1));
+    const uint32_t low = __reduce_min_sync(  // columns of zeros left out
+        0xffffffffu, min(big0 ? big0 : 0x7fffffffu, big1 ? big1 : 0x7fffffffu));
+    const int emax = big ? (int)(big >> 20) : 1023;  // an element of zeros has zero digits
+    const bool direct = emax < 123 || emax > 1923 ||  // outside [2^-900, 2^900]
+                        (big && emax - (int)(low >> 20) > kFxRange);
+    const double ce = coef ? coef[e] : 1.0;
+    auto store = [&](int l, double r0, double r1, int32_t i0, int32_t i1, double v0, double v1) {
+      if (FUSED) {
+        auto one = [&](double r, int32_t id, double u, int h) {
+          if (id >= 0) {
+            __stcs(out + base + l * NQ2 + h, r);
+          } else if (id != -1) {
+            const double v = plus_zero(r);
+            __stcs(outG + (-2 - id), v);
+            acc.add(u, v);
+          }
+        };
+        if (on0) one(r0, i0, v0, 0);
+        if (on1) one(r1, i1, v1, 1);
+      } else if (EVEN && vec) {
+        if (on0) __stcs(reinterpret_cast<double2 *>(out + base + l * NQ2), make_double2(r0, r1));
+      } else {
+        if (on0) __stcs(out + base + l * NQ2, r0);
+        if (on1) __stcs(out + base + l * NQ2 + 1, r1);
+      }
+    };
+    if (!direct) {
+      // ---- digits into shared memory: word (a, k, g ^ k, t)
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        if (!layer(l)) break;
+        const int k = k0 + l;
+        const uint64_t x = fx_fixed(u0[l], emax), y = fx_fixed(u1[l], emax);
+        uint32_t *p = reinterpret_cast<uint32_t *>(dig) + (k * 8 + (g ^ k)) * 4 + t;
+        constexpr int PW = S::PLANE / 4;
+        p[0 * PW] = fx_digit2<0>(x, y);
+        p[1 * PW] = fx_digit2<1>(x, y);
+        p[2 * PW] = fx_digit2<2>(x, y);
+        p[3 * PW] = fx_digit2<3>(x, y);
+        p[4 * PW] = fx_digit2<4>(x, y);
+        p[5 * PW] = fx_digit2<5>(x, y);
+      }
+      const FxStart start1(kFxMagicBits, kFxMagicBits), start2(kFxMagic2Bits, kFxMagic2Bits),
+          start12(kFxMagicBits, kFxMagic2Bits);
+      uint32_t kw[D];
+#pragma unroll
+      for (int b = 0; b < D; ++b) kw[b] = __ldg(&tab->fx.w[b][lane]);
+      sync();
+      // A fragments of Kh for the orders o (rows 0-7) and o + 1 (rows 8-15)
+      // against digits a, a + 1: digits o - a, o + 1 - a, o - a - 1, o - a
+      auto kd = [&](int b) { return b >= 0 ? kw[b < D ? b : 0] : 0u; };
+      const int mrow = lane & 7, mmat = lane >> 3;  // ldmatrix: row, matrix of this lane
+      // ---- along t, planes j = k0 + l: rows k of the digit planes, transposed
+      // (rows past Nq repeat the last one; their Kh digits are zero)
+      const int krow = mrow < NQ ? mrow : NQ - 1;
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        if (!layer(l)) break;
+        const int j = k0 + l;
+        uint32_t f[D];
+        const uint32_t row = dig_s + (krow * 8 + (j ^ krow)) * 16;
+        fx_ldsm4t(f, row + mmat * S::PLANE);
+        fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * S::PLANE);
+        uint32_t s0[D], s1[D];  // with the start values' bits: removed along r and s
+#pragma unroll
+        for (int o = 0; o < D; o += 2) {
+          float c[4];
+          fx_mma0(c, kd(o), kd(o + 1), kd(o - 1), kd(o), f[0], f[1],
+                  o + 2 == D ? start12 : start1);
+#pragma unroll
+          for (int a = 2; a <= o; a += 2)
+            fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
+          s0[o] = __float_as_uint(c[0]);
+          s1[o] = __float_as_uint(c[1]);
+          s0[o + 1] = __float_as_uint(c[2]);
+          s1[o + 1] = __float_as_uint(c[3]);
+        }
+        // the lane holds nodes (2t, j, k = g), (2t + 1, j, g)
+        if (NQ == 8 || g < NQ) {
+          // 64-byte rows (j, k), in an order that lets the owner's reads
+          // (fixed k, all j) and these writes (fixed j, all k) miss no bank
+          const int kk = NQ == 8 ? (g ^ j) : g;
+          *reinterpret_cast<ulonglong2 *>(xch + (j * NQ + kk) * 64 + t * 16) =
+              make_ulonglong2(fx_join(s0), fx_join(s1));
+        }
+      }
+      // ---- along r and s, two layers at a time
+      uint64_t T0[L], T1[L];
+#pragma unroll
+      for (int l = 0; l < L; l += 2) {
+        if (!layer(l)) break;
+        const int ka = k0 + l, kb = ka + 1 < NQ ? ka + 1 : ka;  // odd Nq: the last layer twice
+        uint32_t s[4][D];  // (ka, 2t), (ka, 2t + 1), (kb, 2t), (kb, 2t + 1)
+        // r: A = digits a, a + 1 of layers ka (rows 0-7) and kb, B = Kh^T
+        uint32_t fr[D / 2][4];  // (a, ka), (a, kb), (a + 1, ka), (a + 1, kb)
+        const int kk = (mmat & 1) ? kb : ka;
+#pragma unroll
+        for (int a = 0; a < D; a += 2)
+          fx_ldsm4(fr[a / 2], dig_s + (a + (mmat >> 1)) * S::PLANE + (kk * 8 + (mrow ^ kk)) * 16);
+#pragma unroll
+        for (int o = 0; o < D; ++o) {
+          float c[4];
+          fx_mma0(c, fr[0][0], fr[0][1], fr[0][2], fr[0][3], kd(o), kd(o - 1),
+                  o + 1 == D ? start2 : start1);
+#pragma unroll
+          for (int a = 2; a <= o; a += 2)
+            fx_mma(c, fr[a / 2][0], fr[a / 2][1], fr[a / 2][2], fr[a / 2][3], kd(o - a),
+                   kd(o - a - 1));
+#pragma unroll
+          for (int n = 0; n < 4; ++n) s[n][o] = __float_as_uint(c[n]);
+        }
+        // s: A = Kh, B = the transposed layer; the start values of all three
+        // directions come off here
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int k = h ? kb : ka;
+          uint32_t f[D];
+          const uint32_t row = dig_s + (k * 8 + (mrow ^ k)) * 16;
+          fx_ldsm4t(f, row + mmat * S::PLANE);
+          fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * S::PLANE);
+#pragma unroll
+          for (int o = 0; o < D; o += 2) {
+            float c[4];
+            fx_mma0(c, kd(o), kd(o + 1), kd(o - 1), kd(o), f[0], f[1],
+                    o + 2 == D ? start12 : start1);
+#pragma unroll
+            for (int a = 2; a <= o; a += 2)
+              fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
+            const uint32_t off = 3u * kFxMagicBits;
+            const uint32_t off1 = 3u * (o + 1 == D - 1 ? kFxMagic2Bits : kFxMagicBits);
+            s[2 * h][o] += __float_as_uint(c[0]) - off;
+            s[2 * h + 1][o] += __float_as_uint(c[1]) - off;
+            s[2 * h][o + 1] += __float_as_uint(c[2]) - off1;
+            s[2 * h + 1][o + 1] += __float_as_uint(c[3]) - off1;
+          }
+          T0[l + h] = fx_join(s[2 * h]);
+          T1[l + h] = fx_join(s[2 * h + 1]);
+        }
+      }
+      sync();
+      // ---- results: w_i w_j w_k (c h/2 sum + lambda (h/2)^3 u), the weights'
+      // products from tables; sum = T 2^60 2^-q 2^(emax - 1080)
+      const int p2 = emax - 1020 - tab->fx.q;
+      // (two loops, not a select per node: a product by 1 costs the FP64 pipe
+      // as much as any)
+      auto results = [&](auto with_coef) {
+#pragma unroll
+        for (int l = 0; l < L; ++l) {
+          if (!layer(l)) break;
+          const int k = k0 + l;
+          ulonglong2 v = make_ulonglong2(0, 0);
+          if (NQ == 8 || g < NQ) {
+            const int kk = NQ == 8 ? (k ^ g) : k;
+            v = *reinterpret_cast<const ulonglong2 *>(xch + (g * NQ + kk) * 64 + t * 16);
+          }
+          double d0 = fx_double((int64_t)(T0[l] + v.x), p2);
+          double d1 = fx_double((int64_t)(T1[l] + v.y), p2);
+          const double2 wg = __ldg(reinterpret_cast<const double2 *>(tab->fx.wg) + k * 32 + lane);
+          const double2 wm = __ldg(reinterpret_cast<const double2 *>(tab->fx.wm) + k * 32 + lane);
+          if (decltype(with_coef)::value) {
+            d0 = ce * d0;
+            d1 = ce * d1;
+          }
+          store(l, fma(wg.x, d0, wm.x * u0[l]), fma(wg.y, d1, wm.y * u1[l]),
+                id0[GATHER_IN ? l : 0], id1[GATHER_IN ? l : 0], u0[l], u1[l]);
+        }
+      };
+      if (coef)
+        results(std::true_type{});
+      else
+        results(std::false_type{});
+    } else {  // ---- the direct sums, from the element's values in memory order
+      double *x = reinterpret_cast<double *>(dig);
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        if (!layer(l)) break;
+        if (on0) x[2 * t + NQ * (g + NQ * (k0 + l))] = u0[l];
+        if (on1) x[2 * t + 1 + NQ * (g + NQ * (k0 + l))] = u1[l];
+      }
+      sync();
+#pragma unroll 1
+      for (int l = 0; l < L; ++l) {
+        if (!layer(l)) break;
+        const int k = k0 + l;
+        double r[2] = {0.0, 0.0}, u[2] = {0.0, 0.0};
+        int32_t id[2] = {-1, -1};
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          if (!(h ? on1 : on0)) continue;
+          const int i = 2 * t + h;
+          u[h] = x[i + NQ * (g + NQ * k)];
+          const double d = fx_direct<NQ>(x, tab, i, g, k);
+          r[h] = fma(tab->fx.wg[(k * 32 + lane) * 2 + h], coef ? ce * d : d,
+                     tab->fx.wm[(k * 32 + lane) * 2 + h] * u[h]);
+          if (FUSED) {
+            id[h] = ids[base + l * NQ2 + h];
+            if (!chk(bs_pred_fused_entry(id[h], tab->ng), BS_CHK_OP_ENTRY)) id[h] = -1;
+          }
+        }
+        store(l, r[0], r[1], id[0], id[1], u[0], u[1]);
+      }
+    }
+  }
+  if (FUSED && partials) {
+    const double part = block_sum<S::THREADS>(acc.value());
+    if (threadIdx.x == 0) partials[blockIdx.x] = part;
+  }
+}
+
+}  // namespace bs
