@@ -43,7 +43,8 @@ __device__ long long g_barrier_budget = kBarrierBudget;
 
 struct BDesc {
   int NQ;
-  int eo;      // 1: even-odd element operator for even NQ (bs_operator_mode at setup)
+  int eo;      // 1: not BS_OP_DIRECT (bs_operator_mode at setup)
+  int epb;     // elements per A item
   int active;  // 1: participates in the current inner/outer step
   int64_t E, NG;
   int64_t NL, nnz, ntiles;  // bounds of the checked build's index tests
@@ -152,6 +153,34 @@ __device__ __noinline__ void ax_call_eo(int64_t slot0, int64_t slot1, const int3
                                                      g, mlam, smem, nullptr, nullptr);
 }
 
+// The fixed-point element operator (bs_op_fx.cuh) on elements [slot0, slot1),
+// on one warp each (two at Nq = 8): no block barriers between elements, and
+// the FP64 pipe, which a batch of small FP64 solves kept 46% busy over a whole
+// iteration, is left to the reductions.
+template <int NQ>
+__device__ __noinline__ void ax_call_fx(int64_t slot0, int64_t slot1, const int32_t *order,
+                                        const int32_t *ids, const double *in, double *out,
+                                        const OpTab<double> *tab, const double *coef,
+                                        unsigned char *smem) {
+  using S = FxShape<NQ>;
+  const int warp = threadIdx.x / 32, group = warp / S::WPE;
+  Acc<double> none;
+  auto sync = [group] {  // the element's warps
+    if (S::WPE == 1)
+      __syncwarp();
+    else
+      asm volatile("bar.sync %0, %1;\n" ::"r"(1 + group), "n"(32 * S::WPE) : "memory");
+  };
+  __syncthreads();  // the previous item may still read the shared memory in another layout
+  for (int64_t s = slot0 + group; s < slot1; s += kBBlock / S::THREADS) {
+    const int64_t e = order[s];
+    if (!chk(bs_pred_index(e, tab->ne), BS_CHK_OP_ENTRY)) continue;
+    sync();  // the last element's exchange buffer has been read
+    fx_element<NQ, S::L, true, false>(e, (warp - group * S::WPE) * S::L, ids, in, out, tab, coef,
+                                      nullptr, none, 1, smem + group * S::SMEM, sync);
+  }
+}
+
 // The float-float element operator (bs_op_ff.cuh) as a real call.
 template <int NQ>
 __device__ __noinline__ void ax_call_ff(int64_t slot0, int64_t E, const int32_t *order,
@@ -169,17 +198,24 @@ __device__ __noinline__ void ax_call_ff(int64_t slot0, int64_t E, const int32_t 
 template <typename T, bool GATHER_IN, bool FF = false>
 __device__ void item_ax(const BDesc &d, int64_t slot0, const T *in, T *out, T *smem) {
   // elements of this item: [slot0, slot1)
-  const int nq2 = d.NQ * d.NQ;
-  const int64_t slot1 = slot0 + (nq2 >= 128 ? 1 : 256 / nq2) < d.E
-                            ? slot0 + (nq2 >= 128 ? 1 : 256 / nq2)
-                            : d.E;
+  const int64_t slot1 = slot0 + d.epb < d.E ? slot0 + d.epb : d.E;
   if constexpr (GATHER_IN && !FF && sizeof(T) == 8) {
-    if (d.eo && (d.NQ == 2 || d.NQ == 4 || d.NQ == 6 || d.NQ == 8)) {
+    if (d.eo && (d.NQ == 2 || (d.NQ >= 4 && d.NQ <= kFxMaxNq))) {
 #define BS_EO_CASE(NQ)                                                                         \
   case NQ:                                                                                     \
     ax_call_eo<NQ>(slot0, slot1, d.order, d.ids, in, out, d.tab, d.coef, d.g, d.mlam, smem);   \
     return;
-      switch (d.NQ) { BS_EO_CASE(2) BS_EO_CASE(4) BS_EO_CASE(6) BS_EO_CASE(8) default: return; }
+#define BS_FX_CASE(NQ)                                                                         \
+  case NQ:                                                                                     \
+    ax_call_fx<NQ>(slot0, slot1, d.order, d.ids, in, out, d.tab, d.coef,                       \
+                   reinterpret_cast<unsigned char *>(smem));                                   \
+    return;
+      switch (d.NQ) {
+        BS_EO_CASE(2) BS_EO_CASE(4)
+        BS_FX_CASE(5) BS_FX_CASE(6) BS_FX_CASE(7) BS_FX_CASE(8)
+        default: return;
+      }
+#undef BS_FX_CASE
 #undef BS_EO_CASE
     }
   }
@@ -303,13 +339,15 @@ __device__ void finish_iteration(const BLists &L, int s, CgState *st, double rr_
 // (FP64 / FP32 operator), or, viewed as floats, the float pairs of the
 // values, the four split tables and the split weights (float-float
 // operator); in the FP64 form also the largest even-odd element group at
-// this block width (Nq = 8: four elements of 4 x 512 values plus tables).
-// Dynamic: 64 KB in the FP64 form, 19 KB float-float, 9 KB FP32.
+// this block width and the block's elements of the fixed-point form (Nq = 7:
+// eight of 8.5 KB).  Dynamic: 68 KB in the FP64 form, 19 KB float-float, 9 KB
+// FP32.
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
 constexpr int kBSmemDirect = kBSmem + 2 * kBMaxNq * kBMaxNq + 32;  // doubles
 constexpr int kBSmemD =
     cmax(kBSmemDirect, cmax(cmax(EoShape<2, kBBlock>::SMEM, EoShape<4, kBBlock>::SMEM),
-                            cmax(EoShape<6, kBBlock>::SMEM, EoShape<8, kBBlock>::SMEM)));
+                            cmax(kBBlock / FxShape<7>::THREADS * FxShape<7>::SMEM / 8,
+                                 kBBlock / FxShape<8>::THREADS * FxShape<8>::SMEM / 8)));
 constexpr int kBSmemF = kBSmem + kBMaxNq * kBMaxNq + 16;  // floats
 template <typename T, bool FF>
 constexpr int iter_smem_bytes() {
@@ -731,9 +769,11 @@ static int build_batch(Batch &B, int ns, const bs_problem *const *P, const doubl
       d.ApLf = reinterpret_cast<float *>(p->d_ApL);
     }
     d.st = p->d_state;
+    // a multiple of a block's warps where each takes an element of its own
     const int nq2 = d.NQ * d.NQ;
-    const int epb = nq2 >= 128 ? 1 : 256 / nq2;
-    for (int64_t e = 0; e < m->E; e += epb) B.hA[(size_t)s].push_back(make_int2(s, (int)e));
+    const bool fx = !f32 && !B.ff && d.eo && d.NQ >= kFxMinNq && d.NQ <= kFxMaxNq;
+    d.epb = fx ? kBBlock / 32 / (d.NQ == 8 ? FxShape<8>::WPE : 1) : (nq2 >= 128 ? 1 : 256 / nq2);
+    for (int64_t e = 0; e < m->E; e += d.epb) B.hA[(size_t)s].push_back(make_int2(s, (int)e));
     for (int64_t t = 0; t < m->ntiles; ++t) B.hB[(size_t)s].push_back(make_int2(s, (int)t));
     const int64_t nch = (m->NG + B.chunk - 1) / B.chunk;
     for (int64_t c = 0; c < (nch > 0 ? nch : 1); ++c)

@@ -391,7 +391,7 @@ inline int64_t ax_blocks(int N, int64_t E, bool fx) {
 #define BS_AXB(NQ)                                                      \
   case NQ:                                                              \
     if (fx && use_fx<NQ>() && g_op_evenodd)                             \
-      return (E + FxShape<NQ>::EPB - 1) / FxShape<NQ>::EPB;             \
+      return E;                                                         \
     return use_eo<NQ>() && g_op_evenodd                                 \
                ? (E + EoShape<NQ>::EPB - 1) / EoShape<NQ>::EPB          \
                : (E + OpShape<NQ>::EPB - 1) / OpShape<NQ>::EPB;
@@ -419,8 +419,8 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
         const int vec = ((uintptr_t)out % 16 == 0) && (GATHER_IN || (uintptr_t)in % 16 == 0); \
         using Sf = FxShape<NQ>;                                                          \
         k_ax_fx<NQ, GATHER_IN, FUSED>                                                    \
-            <<<(unsigned)((E + Sf::EPB - 1) / Sf::EPB), Sf::THREADS, Sf::SMEM, s>>>(     \
-                E, order, ids, in, out, tab, coef, st, outG, partials, vec);             \
+            <<<(unsigned)E, Sf::THREADS, Sf::SMEM, s>>>(E, order, ids, in, out, tab, coef, \
+                                                        st, outG, partials, vec);        \
         break;                                                                           \
       }                                                                                  \
     } else if constexpr (use_eo<NQ>()) {                                                 \

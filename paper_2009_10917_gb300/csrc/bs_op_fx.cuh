@@ -79,14 +79,13 @@ template <int NQ>
 struct FxShape {
   static constexpr int L = NQ == 8 ? 4 : (NQ + 1) / 2 * 2;  // layers per warp
   static constexpr int WPE = (NQ + L - 1) / L;              // warps per element
-  static constexpr int EPB = 1;                             // elements per block
-  static constexpr int THREADS = 32 * WPE * EPB;
+  static constexpr int THREADS = 32 * WPE;                  // one element per block
   static constexpr int BLOCKS = NQ == 8 ? 14 : (NQ == 7 ? 20 : 24);  // resident per SM
   static constexpr int PLANE = NQ * 8 * 16;       // bytes of one digit plane
   static constexpr int DIG = kFxDigits * PLANE;
   static constexpr int XCH = NQ * NQ * 64;        // [j][k][8 i] uint64
-  static constexpr int ELEM = DIG + XCH + (WPE > 1 ? WPE * 256 : 0);  // + columns' maxima
-  static constexpr int SMEM = EPB * ELEM;
+  static constexpr int WARP = DIG + XCH;          // bytes an element takes on one warp
+  static constexpr int SMEM = WARP + (WPE > 1 ? WPE * 256 : 0);  // + columns' maxima
 };
 
 // c += A B on a 16 x 8 tile, 16 digit products per entry, all exact.
@@ -206,177 +205,221 @@ __device__ __noinline__ double fx_direct(const double *x, const OpTab<double> *t
   return (ar / w[i] + as / w[j]) + at / w[k];
 }
 
-// out = A_L in; arguments as k_ax_local (FUSED likewise).  vec: out (and,
-// without GATHER_IN, in) is 16-byte aligned.
-template <int NQ, bool GATHER_IN, bool FUSED>
-__global__ void __launch_bounds__(FxShape<NQ>::THREADS, FxShape<NQ>::BLOCKS)
-    k_ax_fx(int64_t E, const int32_t *__restrict__ order, const int32_t *__restrict__ ids,
-            const double *__restrict__ in, double *__restrict__ out,
-            const OpTab<double> *__restrict__ tab, const double *__restrict__ coef,
-            const CgState *st, double *__restrict__ outG, double *__restrict__ partials,
-            int vec) {
+// out = A_L in on one element e, by the WPE warps that call it with their own
+// first layer k0 (of L) and the same shared memory (dig; see FxShape); sync()
+// is a barrier of these warps.  Other arguments as k_ax_local (FUSED
+// likewise); vec: out (and, without GATHER_IN, in) is 16-byte aligned.
+template <int NQ, int L, bool GATHER_IN, bool FUSED, class Sync>
+__device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__restrict__ ids,
+                                           const double *__restrict__ in,
+                                           double *__restrict__ out,
+                                           const OpTab<double> *__restrict__ tab,
+                                           const double *__restrict__ coef,
+                                           double *__restrict__ outG, Acc<double> &acc, int vec,
+                                           unsigned char *dig, Sync sync) {
   static_assert(!FUSED || GATHER_IN, "the fused operator reads its input through the map");
   using S = FxShape<NQ>;
-  constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2, D = kFxDigits, L = S::L;
+  constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2, D = kFxDigits, WPE = (NQ + L - 1) / L;
   constexpr bool EVEN = NQ % 2 == 0;
-  extern __shared__ __align__(128) unsigned char fx_smem[];
-  if (cg_halted(st)) return;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int le = (int)threadIdx.x / (32 * S::WPE);  // the element's slot in the block
-  const int k0 = ((int)threadIdx.x / 32 - le * S::WPE) * L;  // this warp's first layer
-  unsigned char *dig = fx_smem + le * S::ELEM, *xch = dig + S::DIG;
+  unsigned char *xch = dig + S::DIG;
   uint32_t *col = reinterpret_cast<uint32_t *>(xch + S::XCH);
   const uint32_t dig_s = (uint32_t)__cvta_generic_to_shared(dig);
-  auto sync = [&]() {  // the element's warps
-    if (S::WPE == 1)
-      __syncwarp();
-    else
-      asm volatile("bar.sync %0, %1;\n" ::"r"(1 + le), "n"(32 * S::WPE) : "memory");
-  };
-  Acc<double> acc;
-  const int64_t slot = (int64_t)blockIdx.x * S::EPB + le;
-  int64_t e = slot < E ? (order ? (int64_t)order[slot] : slot) : -1;
-  if (e >= 0 && !chk(bs_pred_index(e, tab->ne), BS_CHK_OP_ENTRY)) e = -1;
-  if (e >= 0) {
-    const bool on0 = g < NQ && 2 * t < NQ, on1 = g < NQ && 2 * t + 1 < NQ;
-    const int64_t base = e * NP + (int64_t)k0 * NQ2 + g * NQ + 2 * t;
-    auto layer = [&](int l) { return NQ % L == 0 || k0 + l < NQ; };
-    // ---- the values of nodes (2t, g, k0 + l), (2t + 1, g, k0 + l), l < L
-    double u0[L], u1[L];
-    int32_t id0[GATHER_IN ? L : 1], id1[GATHER_IN ? L : 1];
-    if (GATHER_IN) {
-#pragma unroll
-      for (int l = 0; l < L; ++l) {
-        id0[l] = id1[l] = -1;
-        if (EVEN) {
-          if (on0 && layer(l)) {
-            const int2 q = __ldcs(reinterpret_cast<const int2 *>(ids + base + l * NQ2));
-            id0[l] = q.x;
-            id1[l] = q.y;
-          }
-        } else {
-          if (on0 && layer(l)) id0[l] = __ldcs(ids + base + l * NQ2);
-          if (on1 && layer(l)) id1[l] = __ldcs(ids + base + l * NQ2 + 1);
-        }
-        if (!chk(FUSED ? bs_pred_fused_entry(id0[l], tab->ng) : bs_pred_map_entry(id0[l], tab->ng),
-                 BS_CHK_OP_ENTRY))
-          id0[l] = -1;
-        if (!chk(FUSED ? bs_pred_fused_entry(id1[l], tab->ng) : bs_pred_map_entry(id1[l], tab->ng),
-                 BS_CHK_OP_ENTRY))
-          id1[l] = -1;
-      }
-#pragma unroll
-      for (int l = 0; l < L; ++l) {
-        if (FUSED) {
-          u0[l] = id0[l] != -1 ? in[id0[l] >= 0 ? id0[l] : -2 - id0[l]] : 0.0;
-          u1[l] = id1[l] != -1 ? in[id1[l] >= 0 ? id1[l] : -2 - id1[l]] : 0.0;
-        } else {
-          u0[l] = id0[l] >= 0 ? in[id0[l]] : 0.0;
-          u1[l] = id1[l] >= 0 ? in[id1[l]] : 0.0;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int l = 0; l < L; ++l) {
-        u0[l] = u1[l] = 0.0;
-        if (EVEN && vec) {
-          if (on0 && layer(l)) {
-            const double2 q = __ldcs(reinterpret_cast<const double2 *>(in + base + l * NQ2));
-            u0[l] = q.x;
-            u1[l] = q.y;
-          }
-        } else {
-          if (on0 && layer(l)) u0[l] = __ldcs(in + base + l * NQ2);
-          if (on1 && layer(l)) u1[l] = __ldcs(in + base + l * NQ2 + 1);
-        }
-      }
-    }
-    // ---- the columns' largest values (high words; 1 for a value whose high
-    // word is zero but which is not), the largest exponent, and whether the
-    // digits serve
-    uint32_t big0 = 0, big1 = 0;
+  const bool on0 = g < NQ && 2 * t < NQ, on1 = g < NQ && 2 * t + 1 < NQ;
+  const int64_t base = e * NP + (int64_t)k0 * NQ2 + g * NQ + 2 * t;
+  auto layer = [&](int l) { return NQ % L == 0 || k0 + l < NQ; };
+  // ---- the values of nodes (2t, g, k0 + l), (2t + 1, g, k0 + l), l < L
+  double u0[L], u1[L];
+  int32_t id0[GATHER_IN ? L : 1], id1[GATHER_IN ? L : 1];
+  if (GATHER_IN) {
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-      big0 = max(big0, ((uint32_t)__double2hiint(u0[l]) & 0x7fffffffu) |
-                           min((uint32_t)__double2loint(u0[l]), 1u));
-      big1 = max(big1, ((uint32_t)__double2hiint(u1[l]) & 0x7fffffffu) |
-                           min((uint32_t)__double2loint(u1[l]), 1u));
-    }
-    if (S::WPE > 1) {
-      reinterpret_cast<uint2 *>(col)[k0 / L * 32 + lane] = make_uint2(big0, big1);
-      sync();
-#pragma unroll
-      for (int w = 0; w < S::WPE; ++w) {
-        const uint2 c = reinterpret_cast<const uint2 *>(col)[w * 32 + lane];
-        big0 = max(big0, c.x);
-        big1 = max(big1, c.y);
-      }
-    }
-    const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0, big1));
-    const uint32_t low = __reduce_min_sync(  // columns of zeros left out
-        0xffffffffu, min(big0 ? big0 : 0x7fffffffu, big1 ? big1 : 0x7fffffffu));
-    const int emax = big ? (int)(big >> 20) : 1023;  // an element of zeros has zero digits
-    const bool direct = emax < 123 || emax > 1923 ||  // outside [2^-900, 2^900]
-                        (big && emax - (int)(low >> 20) > kFxRange);
-    const double ce = coef ? coef[e] : 1.0;
-    auto store = [&](int l, double r0, double r1, int32_t i0, int32_t i1, double v0, double v1) {
-      if (FUSED) {
-        auto one = [&](double r, int32_t id, double u, int h) {
-          if (id >= 0) {
-            __stcs(out + base + l * NQ2 + h, r);
-          } else if (id != -1) {
-            const double v = plus_zero(r);
-            __stcs(outG + (-2 - id), v);
-            acc.add(u, v);
-          }
-        };
-        if (on0) one(r0, i0, v0, 0);
-        if (on1) one(r1, i1, v1, 1);
-      } else if (EVEN && vec) {
-        if (on0) __stcs(reinterpret_cast<double2 *>(out + base + l * NQ2), make_double2(r0, r1));
+      id0[l] = id1[l] = -1;
+      if (EVEN) {
+        if (on0 && layer(l)) {
+          const int2 q = __ldcs(reinterpret_cast<const int2 *>(ids + base + l * NQ2));
+          id0[l] = q.x;
+          id1[l] = q.y;
+        }
       } else {
-        if (on0) __stcs(out + base + l * NQ2, r0);
-        if (on1) __stcs(out + base + l * NQ2 + 1, r1);
+        if (on0 && layer(l)) id0[l] = __ldcs(ids + base + l * NQ2);
+        if (on1 && layer(l)) id1[l] = __ldcs(ids + base + l * NQ2 + 1);
       }
-    };
-    if (!direct) {
-      // ---- digits into shared memory: word (a, k, g ^ k, t)
+      if (!chk(FUSED ? bs_pred_fused_entry(id0[l], tab->ng) : bs_pred_map_entry(id0[l], tab->ng),
+               BS_CHK_OP_ENTRY))
+        id0[l] = -1;
+      if (!chk(FUSED ? bs_pred_fused_entry(id1[l], tab->ng) : bs_pred_map_entry(id1[l], tab->ng),
+               BS_CHK_OP_ENTRY))
+        id1[l] = -1;
+    }
 #pragma unroll
-      for (int l = 0; l < L; ++l) {
-        if (!layer(l)) break;
-        const int k = k0 + l;
-        const uint64_t x = fx_fixed(u0[l], emax), y = fx_fixed(u1[l], emax);
-        uint32_t *p = reinterpret_cast<uint32_t *>(dig) + (k * 8 + (g ^ k)) * 4 + t;
-        constexpr int PW = S::PLANE / 4;
-        p[0 * PW] = fx_digit2<0>(x, y);
-        p[1 * PW] = fx_digit2<1>(x, y);
-        p[2 * PW] = fx_digit2<2>(x, y);
-        p[3 * PW] = fx_digit2<3>(x, y);
-        p[4 * PW] = fx_digit2<4>(x, y);
-        p[5 * PW] = fx_digit2<5>(x, y);
+    for (int l = 0; l < L; ++l) {
+      if (FUSED) {
+        u0[l] = id0[l] != -1 ? in[id0[l] >= 0 ? id0[l] : -2 - id0[l]] : 0.0;
+        u1[l] = id1[l] != -1 ? in[id1[l] >= 0 ? id1[l] : -2 - id1[l]] : 0.0;
+      } else {
+        u0[l] = id0[l] >= 0 ? in[id0[l]] : 0.0;
+        u1[l] = id1[l] >= 0 ? in[id1[l]] : 0.0;
       }
-      const FxStart start1(kFxMagicBits, kFxMagicBits), start2(kFxMagic2Bits, kFxMagic2Bits),
-          start12(kFxMagicBits, kFxMagic2Bits);
-      uint32_t kw[D];
+    }
+  } else {
 #pragma unroll
-      for (int b = 0; b < D; ++b) kw[b] = __ldg(&tab->fx.w[b][lane]);
-      sync();
-      // A fragments of Kh for the orders o (rows 0-7) and o + 1 (rows 8-15)
-      // against digits a, a + 1: digits o - a, o + 1 - a, o - a - 1, o - a
-      auto kd = [&](int b) { return b >= 0 ? kw[b < D ? b : 0] : 0u; };
-      const int mrow = lane & 7, mmat = lane >> 3;  // ldmatrix: row, matrix of this lane
-      // ---- along t, planes j = k0 + l: rows k of the digit planes, transposed
-      // (rows past Nq repeat the last one; their Kh digits are zero)
-      const int krow = mrow < NQ ? mrow : NQ - 1;
+    for (int l = 0; l < L; ++l) {
+      u0[l] = u1[l] = 0.0;
+      if (EVEN && vec) {
+        if (on0 && layer(l)) {
+          const double2 q = __ldcs(reinterpret_cast<const double2 *>(in + base + l * NQ2));
+          u0[l] = q.x;
+          u1[l] = q.y;
+        }
+      } else {
+        if (on0 && layer(l)) u0[l] = __ldcs(in + base + l * NQ2);
+        if (on1 && layer(l)) u1[l] = __ldcs(in + base + l * NQ2 + 1);
+      }
+    }
+  }
+  // ---- the columns' largest values (high words; 1 for a value whose high
+  // word is zero but which is not), the largest exponent, and whether the
+  // digits serve
+  uint32_t big0 = 0, big1 = 0;
 #pragma unroll
-      for (int l = 0; l < L; ++l) {
-        if (!layer(l)) break;
-        const int j = k0 + l;
+  for (int l = 0; l < L; ++l) {
+    big0 = max(big0, ((uint32_t)__double2hiint(u0[l]) & 0x7fffffffu) |
+                         min((uint32_t)__double2loint(u0[l]), 1u));
+    big1 = max(big1, ((uint32_t)__double2hiint(u1[l]) & 0x7fffffffu) |
+                         min((uint32_t)__double2loint(u1[l]), 1u));
+  }
+  if (WPE > 1) {
+    reinterpret_cast<uint2 *>(col)[k0 / L * 32 + lane] = make_uint2(big0, big1);
+    sync();
+#pragma unroll
+    for (int w = 0; w < WPE; ++w) {
+      const uint2 c = reinterpret_cast<const uint2 *>(col)[w * 32 + lane];
+      big0 = max(big0, c.x);
+      big1 = max(big1, c.y);
+    }
+  }
+  const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0, big1));
+  const uint32_t low = __reduce_min_sync(  // columns of zeros left out
+      0xffffffffu, min(big0 ? big0 : 0x7fffffffu, big1 ? big1 : 0x7fffffffu));
+  const int emax = big ? (int)(big >> 20) : 1023;  // an element of zeros has zero digits
+  const bool direct = emax < 123 || emax > 1923 ||  // outside [2^-900, 2^900]
+                      (big && emax - (int)(low >> 20) > kFxRange);
+  const double ce = coef ? coef[e] : 1.0;
+  auto store = [&](int l, double r0, double r1, int32_t i0, int32_t i1, double v0, double v1) {
+    if (FUSED) {
+      auto one = [&](double r, int32_t id, double u, int h) {
+        if (id >= 0) {
+          __stcs(out + base + l * NQ2 + h, r);
+        } else if (id != -1) {
+          const double v = plus_zero(r);
+          __stcs(outG + (-2 - id), v);
+          acc.add(u, v);
+        }
+      };
+      if (on0) one(r0, i0, v0, 0);
+      if (on1) one(r1, i1, v1, 1);
+    } else if (EVEN && vec) {
+      if (on0) __stcs(reinterpret_cast<double2 *>(out + base + l * NQ2), make_double2(r0, r1));
+    } else {
+      if (on0) __stcs(out + base + l * NQ2, r0);
+      if (on1) __stcs(out + base + l * NQ2 + 1, r1);
+    }
+  };
+  if (!direct) {
+    // ---- digits into shared memory: word (a, k, g ^ k, t)
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      if (!layer(l)) break;
+      const int k = k0 + l;
+      const uint64_t x = fx_fixed(u0[l], emax), y = fx_fixed(u1[l], emax);
+      uint32_t *p = reinterpret_cast<uint32_t *>(dig) + (k * 8 + (g ^ k)) * 4 + t;
+      constexpr int PW = S::PLANE / 4;
+      p[0 * PW] = fx_digit2<0>(x, y);
+      p[1 * PW] = fx_digit2<1>(x, y);
+      p[2 * PW] = fx_digit2<2>(x, y);
+      p[3 * PW] = fx_digit2<3>(x, y);
+      p[4 * PW] = fx_digit2<4>(x, y);
+      p[5 * PW] = fx_digit2<5>(x, y);
+    }
+    const FxStart start1(kFxMagicBits, kFxMagicBits), start2(kFxMagic2Bits, kFxMagic2Bits),
+        start12(kFxMagicBits, kFxMagic2Bits);
+    uint32_t kw[D];
+#pragma unroll
+    for (int b = 0; b < D; ++b) kw[b] = __ldg(&tab->fx.w[b][lane]);
+    sync();
+    // A fragments of Kh for the orders o (rows 0-7) and o + 1 (rows 8-15)
+    // against digits a, a + 1: digits o - a, o + 1 - a, o - a - 1, o - a
+    auto kd = [&](int b) { return b >= 0 ? kw[b < D ? b : 0] : 0u; };
+    const int mrow = lane & 7, mmat = lane >> 3;  // ldmatrix: row, matrix of this lane
+    // ---- along t, planes j = k0 + l: rows k of the digit planes, transposed
+    // (rows past Nq repeat the last one; their Kh digits are zero)
+    const int krow = mrow < NQ ? mrow : NQ - 1;
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      if (!layer(l)) break;
+      const int j = k0 + l;
+      uint32_t f[D];
+      const uint32_t row = dig_s + (krow * 8 + (j ^ krow)) * 16;
+      fx_ldsm4t(f, row + mmat * S::PLANE);
+      fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * S::PLANE);
+      uint32_t s0[D], s1[D];  // with the start values' bits: removed along r and s
+#pragma unroll
+      for (int o = 0; o < D; o += 2) {
+        float c[4];
+        fx_mma0(c, kd(o), kd(o + 1), kd(o - 1), kd(o), f[0], f[1],
+                o + 2 == D ? start12 : start1);
+#pragma unroll
+        for (int a = 2; a <= o; a += 2)
+          fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
+        s0[o] = __float_as_uint(c[0]);
+        s1[o] = __float_as_uint(c[1]);
+        s0[o + 1] = __float_as_uint(c[2]);
+        s1[o + 1] = __float_as_uint(c[3]);
+      }
+      // the lane holds nodes (2t, j, k = g), (2t + 1, j, g)
+      if (NQ == 8 || g < NQ) {
+        // 64-byte rows (j, k), in an order that lets the owner's reads
+        // (fixed k, all j) and these writes (fixed j, all k) miss no bank
+        const int kk = NQ == 8 ? (g ^ j) : g;
+        *reinterpret_cast<ulonglong2 *>(xch + (j * NQ + kk) * 64 + t * 16) =
+            make_ulonglong2(fx_join(s0), fx_join(s1));
+      }
+    }
+    // ---- along r and s, two layers at a time
+    uint64_t T0[L], T1[L];
+#pragma unroll
+    for (int l = 0; l < L; l += 2) {
+      if (!layer(l)) break;
+      const int ka = k0 + l, kb = ka + 1 < NQ ? ka + 1 : ka;  // odd Nq: the last layer twice
+      uint32_t s[4][D];  // (ka, 2t), (ka, 2t + 1), (kb, 2t), (kb, 2t + 1)
+      // r: A = digits a, a + 1 of layers ka (rows 0-7) and kb, B = Kh^T
+      uint32_t fr[D / 2][4];  // (a, ka), (a, kb), (a + 1, ka), (a + 1, kb)
+      const int kk = (mmat & 1) ? kb : ka;
+#pragma unroll
+      for (int a = 0; a < D; a += 2)
+        fx_ldsm4(fr[a / 2], dig_s + (a + (mmat >> 1)) * S::PLANE + (kk * 8 + (mrow ^ kk)) * 16);
+#pragma unroll
+      for (int o = 0; o < D; ++o) {
+        float c[4];
+        fx_mma0(c, fr[0][0], fr[0][1], fr[0][2], fr[0][3], kd(o), kd(o - 1),
+                o + 1 == D ? start2 : start1);
+#pragma unroll
+        for (int a = 2; a <= o; a += 2)
+          fx_mma(c, fr[a / 2][0], fr[a / 2][1], fr[a / 2][2], fr[a / 2][3], kd(o - a),
+                 kd(o - a - 1));
+#pragma unroll
+        for (int n = 0; n < 4; ++n) s[n][o] = __float_as_uint(c[n]);
+      }
+      // s: A = Kh, B = the transposed layer; the start values of all three
+      // directions come off here
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = h ? kb : ka;
         uint32_t f[D];
-        const uint32_t row = dig_s + (krow * 8 + (j ^ krow)) * 16;
+        const uint32_t row = dig_s + (k * 8 + (mrow ^ k)) * 16;
         fx_ldsm4t(f, row + mmat * S::PLANE);
         fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * S::PLANE);
-        uint32_t s0[D], s1[D];  // with the start values' bits: removed along r and s
 #pragma unroll
         for (int o = 0; o < D; o += 2) {
           float c[4];
@@ -385,137 +428,104 @@ __global__ void __launch_bounds__(FxShape<NQ>::THREADS, FxShape<NQ>::BLOCKS)
 #pragma unroll
           for (int a = 2; a <= o; a += 2)
             fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
-          s0[o] = __float_as_uint(c[0]);
-          s1[o] = __float_as_uint(c[1]);
-          s0[o + 1] = __float_as_uint(c[2]);
-          s1[o + 1] = __float_as_uint(c[3]);
+          const uint32_t off = 3u * kFxMagicBits;
+          const uint32_t off1 = 3u * (o + 1 == D - 1 ? kFxMagic2Bits : kFxMagicBits);
+          s[2 * h][o] += __float_as_uint(c[0]) - off;
+          s[2 * h + 1][o] += __float_as_uint(c[1]) - off;
+          s[2 * h][o + 1] += __float_as_uint(c[2]) - off1;
+          s[2 * h + 1][o + 1] += __float_as_uint(c[3]) - off1;
         }
-        // the lane holds nodes (2t, j, k = g), (2t + 1, j, g)
-        if (NQ == 8 || g < NQ) {
-          // 64-byte rows (j, k), in an order that lets the owner's reads
-          // (fixed k, all j) and these writes (fixed j, all k) miss no bank
-          const int kk = NQ == 8 ? (g ^ j) : g;
-          *reinterpret_cast<ulonglong2 *>(xch + (j * NQ + kk) * 64 + t * 16) =
-              make_ulonglong2(fx_join(s0), fx_join(s1));
-        }
+        T0[l + h] = fx_join(s[2 * h]);
+        T1[l + h] = fx_join(s[2 * h + 1]);
       }
-      // ---- along r and s, two layers at a time
-      uint64_t T0[L], T1[L];
+    }
+    sync();
+    // ---- results: w_i w_j w_k (c h/2 sum + lambda (h/2)^3 u), the weights'
+    // products from tables; sum = T 2^60 2^-q 2^(emax - 1080)
+    const int p2 = emax - 1020 - tab->fx.q;
+    // (two loops, not a select per node: a product by 1 costs the FP64 pipe
+    // as much as any)
+    auto results = [&](auto with_coef) {
 #pragma unroll
-      for (int l = 0; l < L; l += 2) {
-        if (!layer(l)) break;
-        const int ka = k0 + l, kb = ka + 1 < NQ ? ka + 1 : ka;  // odd Nq: the last layer twice
-        uint32_t s[4][D];  // (ka, 2t), (ka, 2t + 1), (kb, 2t), (kb, 2t + 1)
-        // r: A = digits a, a + 1 of layers ka (rows 0-7) and kb, B = Kh^T
-        uint32_t fr[D / 2][4];  // (a, ka), (a, kb), (a + 1, ka), (a + 1, kb)
-        const int kk = (mmat & 1) ? kb : ka;
-#pragma unroll
-        for (int a = 0; a < D; a += 2)
-          fx_ldsm4(fr[a / 2], dig_s + (a + (mmat >> 1)) * S::PLANE + (kk * 8 + (mrow ^ kk)) * 16);
-#pragma unroll
-        for (int o = 0; o < D; ++o) {
-          float c[4];
-          fx_mma0(c, fr[0][0], fr[0][1], fr[0][2], fr[0][3], kd(o), kd(o - 1),
-                  o + 1 == D ? start2 : start1);
-#pragma unroll
-          for (int a = 2; a <= o; a += 2)
-            fx_mma(c, fr[a / 2][0], fr[a / 2][1], fr[a / 2][2], fr[a / 2][3], kd(o - a),
-                   kd(o - a - 1));
-#pragma unroll
-          for (int n = 0; n < 4; ++n) s[n][o] = __float_as_uint(c[n]);
-        }
-        // s: A = Kh, B = the transposed layer; the start values of all three
-        // directions come off here
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int k = h ? kb : ka;
-          uint32_t f[D];
-          const uint32_t row = dig_s + (k * 8 + (mrow ^ k)) * 16;
-          fx_ldsm4t(f, row + mmat * S::PLANE);
-          fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * S::PLANE);
-#pragma unroll
-          for (int o = 0; o < D; o += 2) {
-            float c[4];
-            fx_mma0(c, kd(o), kd(o + 1), kd(o - 1), kd(o), f[0], f[1],
-                    o + 2 == D ? start12 : start1);
-#pragma unroll
-            for (int a = 2; a <= o; a += 2)
-              fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
-            const uint32_t off = 3u * kFxMagicBits;
-            const uint32_t off1 = 3u * (o + 1 == D - 1 ? kFxMagic2Bits : kFxMagicBits);
-            s[2 * h][o] += __float_as_uint(c[0]) - off;
-            s[2 * h + 1][o] += __float_as_uint(c[1]) - off;
-            s[2 * h][o + 1] += __float_as_uint(c[2]) - off1;
-            s[2 * h + 1][o + 1] += __float_as_uint(c[3]) - off1;
-          }
-          T0[l + h] = fx_join(s[2 * h]);
-          T1[l + h] = fx_join(s[2 * h + 1]);
-        }
-      }
-      sync();
-      // ---- results: w_i w_j w_k (c h/2 sum + lambda (h/2)^3 u), the weights'
-      // products from tables; sum = T 2^60 2^-q 2^(emax - 1080)
-      const int p2 = emax - 1020 - tab->fx.q;
-      // (two loops, not a select per node: a product by 1 costs the FP64 pipe
-      // as much as any)
-      auto results = [&](auto with_coef) {
-#pragma unroll
-        for (int l = 0; l < L; ++l) {
-          if (!layer(l)) break;
-          const int k = k0 + l;
-          ulonglong2 v = make_ulonglong2(0, 0);
-          if (NQ == 8 || g < NQ) {
-            const int kk = NQ == 8 ? (k ^ g) : k;
-            v = *reinterpret_cast<const ulonglong2 *>(xch + (g * NQ + kk) * 64 + t * 16);
-          }
-          double d0 = fx_double((int64_t)(T0[l] + v.x), p2);
-          double d1 = fx_double((int64_t)(T1[l] + v.y), p2);
-          const double2 wg = __ldg(reinterpret_cast<const double2 *>(tab->fx.wg) + k * 32 + lane);
-          const double2 wm = __ldg(reinterpret_cast<const double2 *>(tab->fx.wm) + k * 32 + lane);
-          if (decltype(with_coef)::value) {
-            d0 = ce * d0;
-            d1 = ce * d1;
-          }
-          store(l, fma(wg.x, d0, wm.x * u0[l]), fma(wg.y, d1, wm.y * u1[l]),
-                id0[GATHER_IN ? l : 0], id1[GATHER_IN ? l : 0], u0[l], u1[l]);
-        }
-      };
-      if (coef)
-        results(std::true_type{});
-      else
-        results(std::false_type{});
-    } else {  // ---- the direct sums, from the element's values in memory order
-      double *x = reinterpret_cast<double *>(dig);
-#pragma unroll
-      for (int l = 0; l < L; ++l) {
-        if (!layer(l)) break;
-        if (on0) x[2 * t + NQ * (g + NQ * (k0 + l))] = u0[l];
-        if (on1) x[2 * t + 1 + NQ * (g + NQ * (k0 + l))] = u1[l];
-      }
-      sync();
-#pragma unroll 1
       for (int l = 0; l < L; ++l) {
         if (!layer(l)) break;
         const int k = k0 + l;
-        double r[2] = {0.0, 0.0}, u[2] = {0.0, 0.0};
-        int32_t id[2] = {-1, -1};
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          if (!(h ? on1 : on0)) continue;
-          const int i = 2 * t + h;
-          u[h] = x[i + NQ * (g + NQ * k)];
-          const double d = fx_direct<NQ>(x, tab, i, g, k);
-          r[h] = fma(tab->fx.wg[(k * 32 + lane) * 2 + h], coef ? ce * d : d,
-                     tab->fx.wm[(k * 32 + lane) * 2 + h] * u[h]);
-          if (FUSED) {
-            id[h] = ids[base + l * NQ2 + h];
-            if (!chk(bs_pred_fused_entry(id[h], tab->ng), BS_CHK_OP_ENTRY)) id[h] = -1;
-          }
+        ulonglong2 v = make_ulonglong2(0, 0);
+        if (NQ == 8 || g < NQ) {
+          const int kk = NQ == 8 ? (k ^ g) : k;
+          v = *reinterpret_cast<const ulonglong2 *>(xch + (g * NQ + kk) * 64 + t * 16);
         }
-        store(l, r[0], r[1], id[0], id[1], u[0], u[1]);
+        double d0 = fx_double((int64_t)(T0[l] + v.x), p2);
+        double d1 = fx_double((int64_t)(T1[l] + v.y), p2);
+        const double2 wg = __ldg(reinterpret_cast<const double2 *>(tab->fx.wg) + k * 32 + lane);
+        const double2 wm = __ldg(reinterpret_cast<const double2 *>(tab->fx.wm) + k * 32 + lane);
+        if (decltype(with_coef)::value) {
+          d0 = ce * d0;
+          d1 = ce * d1;
+        }
+        store(l, fma(wg.x, d0, wm.x * u0[l]), fma(wg.y, d1, wm.y * u1[l]),
+              id0[GATHER_IN ? l : 0], id1[GATHER_IN ? l : 0], u0[l], u1[l]);
       }
+    };
+    if (coef)
+      results(std::true_type{});
+    else
+      results(std::false_type{});
+  } else {  // ---- the direct sums, from the element's values in memory order
+    double *x = reinterpret_cast<double *>(dig);
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      if (!layer(l)) break;
+      if (on0) x[2 * t + NQ * (g + NQ * (k0 + l))] = u0[l];
+      if (on1) x[2 * t + 1 + NQ * (g + NQ * (k0 + l))] = u1[l];
+    }
+    sync();
+#pragma unroll 1
+    for (int l = 0; l < L; ++l) {
+      if (!layer(l)) break;
+      const int k = k0 + l;
+      double r[2] = {0.0, 0.0}, u[2] = {0.0, 0.0};
+      int32_t id[2] = {-1, -1};
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        if (!(h ? on1 : on0)) continue;
+        const int i = 2 * t + h;
+        u[h] = x[i + NQ * (g + NQ * k)];
+        const double d = fx_direct<NQ>(x, tab, i, g, k);
+        r[h] = fma(tab->fx.wg[(k * 32 + lane) * 2 + h], coef ? ce * d : d,
+                   tab->fx.wm[(k * 32 + lane) * 2 + h] * u[h]);
+        if (FUSED) {
+          id[h] = ids[base + l * NQ2 + h];
+          if (!chk(bs_pred_fused_entry(id[h], tab->ng), BS_CHK_OP_ENTRY)) id[h] = -1;
+        }
+      }
+      store(l, r[0], r[1], id[0], id[1], u[0], u[1]);
     }
   }
+}
+
+template <int NQ, bool GATHER_IN, bool FUSED>
+__global__ void __launch_bounds__(FxShape<NQ>::THREADS, FxShape<NQ>::BLOCKS)
+    k_ax_fx(int64_t E, const int32_t *__restrict__ order, const int32_t *__restrict__ ids,
+            const double *__restrict__ in, double *__restrict__ out,
+            const OpTab<double> *__restrict__ tab, const double *__restrict__ coef,
+            const CgState *st, double *__restrict__ outG, double *__restrict__ partials,
+            int vec) {
+  using S = FxShape<NQ>;
+  extern __shared__ __align__(128) unsigned char fx_smem[];
+  if (cg_halted(st)) return;
+  Acc<double> acc;
+  const int64_t slot = blockIdx.x;
+  int64_t e = slot < E ? (order ? (int64_t)order[slot] : slot) : -1;
+  if (e >= 0 && !chk(bs_pred_index(e, tab->ne), BS_CHK_OP_ENTRY)) e = -1;
+  if (e >= 0)
+    fx_element<NQ, S::L, GATHER_IN, FUSED>(e, (int)(threadIdx.x / 32) * S::L, ids, in, out, tab,
+                                           coef, outG, acc, vec, fx_smem, [] {
+                                             if (S::WPE == 1)
+                                               __syncwarp();
+                                             else
+                                               __syncthreads();
+                                           });
   if (FUSED && partials) {
     const double part = block_sum<S::THREADS>(acc.value());
     if (threadIdx.x == 0) partials[blockIdx.x] = part;
