@@ -469,8 +469,9 @@ enum {
  * GEMM on mma.sync (bf16 -> fp32); 1 runs them on the tcgen05 tensor cores
  * (accumulator in tensor memory, operands staged by cp.async in the
  * canonical K-major layout) wherever the shape allows -- K a multiple of 8,
- * 16-byte aligned operands, any epilogue but the relu' mask of the backward
- * pass.  Both give bitwise identical results; at the learned
+ * 16-byte aligned operands -- except a training step's products after the
+ * hidden layer, whose epilogues (loss, relu' mask, Adam) and transposed
+ * operands only the mma.sync kernels have.  Both give bitwise identical results; at the learned
  * preconditioner's shapes the mma.sync kernel is measured faster (97 vs
  * 137 us for the interior GEMM at N = 5 on 48^3).  Returns the previous
  * engine; any other value only queries it. */

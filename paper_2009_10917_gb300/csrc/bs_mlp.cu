@@ -1,11 +1,14 @@
 // bs_mlp.cu -- BF16 tensor-core GEMM and the MLP's forward pass, MSE loss and
-// gradients, and Adam (see bs_mlp.cuh).  Training runs entirely in these
-// kernels: forward (2 GEMMs), loss, backward (3 GEMMs), Adam, bf16 refresh.
+// gradients, and Adam (see bs_mlp.cuh).  A training step is five launches: the
+// input's packing, then the small-tile GEMM of bs_gemm_s.cuh for the hidden
+// layer, the output layer with the loss, dZ, and both weight gradients with
+// Adam (256 rows, D = 216, H = 256: 136 us a step as 14 launches of the large
+// tiles, transposes and element-wise kernels, about 40 us now).
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
 
-#include "bs_mlp.cuh"
+#include "bs_gemm_s.cuh"
 
 namespace bs {
 
@@ -146,10 +149,21 @@ int launch_gemm(int epi, const GemmArgs &a, cudaStream_t s) {
   if (gemm_tc_supported(epi, a)) return launch_gemm_tc(epi, a, a.err, s);
   const int64_t gy = (a.M + GBM - 1) / GBM;
   if (gy > 65535) return fail(BS_ERR_ARG, "gemm: M too large");
+  // Too few 128-row tiles for half the SMs: the small tiles (a 256-row batch
+  // at D = 216, H = 256: hidden layer 35 us on four blocks, 4 us on 64).
+  DeviceInfo di;
+  if (int rc = device_info(&di)) return rc;
+  if (gy * (a.N <= 64 ? 1 : (a.N + 127) / 128) < di.sms / 2) {
+    switch (epi) {
+      case EPI_F32: return launch_gemm_s<EPI_F32, false, false>(a, TrainArgs{}, s);
+      case EPI_HIDDEN: return launch_gemm_s<EPI_HIDDEN, false, false>(a, TrainArgs{}, s);
+      case EPI_SCATTER_F64: return launch_gemm_s<EPI_SCATTER_F64, false, false>(a, TrainArgs{}, s);
+      default: break;
+    }
+  }
   switch (epi) {
     case EPI_F32: launch_epi<EPI_F32>(a, gy, s); break;
     case EPI_HIDDEN: launch_epi<EPI_HIDDEN>(a, gy, s); break;
-    case EPI_MASK_BF16: launch_epi<EPI_MASK_BF16>(a, gy, s); break;
     case EPI_SCALE_F64: launch_epi<EPI_SCALE_F64>(a, gy, s); break;
     case EPI_SCATTER_F64: launch_epi<EPI_SCATTER_F64>(a, gy, s); break;
     default: return fail(BS_ERR_ARG, "gemm: unknown epilogue");
@@ -180,30 +194,6 @@ __global__ void k_pack_bf16(int64_t R, int C, int Cp, int split, const float *__
   }
 }
 
-// out[c * R + r] = in[r * ldi + c] for r < R, c < C (bf16 transpose by tiles).
-__global__ void k_transpose_bf16(int R, int C, int ldi, const __nv_bfloat16 *__restrict__ in,
-                                 __nv_bfloat16 *__restrict__ out) {
-  __shared__ __nv_bfloat16 t[32][33];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int r = r0 + k, c = c0 + threadIdx.x;
-    if (r < R && c < C) t[k][threadIdx.x] = in[(int64_t)r * ldi + c];
-  }
-  __syncthreads();
-  for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-    const int c = c0 + k, r = r0 + threadIdx.x;
-    if (r < R && c < C) out[(int64_t)c * R + r] = t[threadIdx.x][k];
-  }
-}
-
-static int transpose(int R, int C, int ldi, const __nv_bfloat16 *in, __nv_bfloat16 *out,
-                     cudaStream_t s) {
-  dim3 grid((C + 31) / 32, (R + 31) / 32), block(32, 8);
-  k_transpose_bf16<<<grid, block, 0, s>>>(R, C, ldi, in, out);
-  BS_LAUNCH_CHECK();
-  return BS_OK;
-}
-
 // dY = 2 (Y - T) / (B D) as bf16 [B x Dp] (zero padding); loss = mean (Y - T)^2.
 __global__ void __launch_bounds__(kReduceBlock)
     k_mse(int64_t B, int D, int Dp, const float *__restrict__ Y, const float *__restrict__ T,
@@ -230,53 +220,16 @@ __global__ void __launch_bounds__(kReduceBlock)
     *loss = total / ((double)B * D);
 }
 
-// Adam (Kingma & Ba 2015) on float weights; c1 = 1 - b1^t, c2 = 1 - b2^t.
-__global__ void k_adam(int64_t n, float *__restrict__ w, const float *__restrict__ g,
-                       float *__restrict__ m, float *__restrict__ v, float lr, float b1, float b2,
-                       float eps, float c1, float c2) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nth = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = tid; i < n; i += nth) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  }
-}
-
 // Weight operands from the FP32 masters: W1b rows [hi] or [hi | lo | hi]
-// (row length K1 = Dp or 3 Dp), W2b likewise (K2 = H or 3 H), and
-// W2tb = hi(W2)^T [H x Dp].
+// (row length K1 = Dp or 3 Dp) and W2b likewise (K2 = H or 3 H).
 __global__ void k_refresh(int H, int Dp, int split, const float *__restrict__ W1,
-                          const float *__restrict__ W2, __nv_bfloat16 *W1b, __nv_bfloat16 *W2b,
-                          __nv_bfloat16 *W2tb) {
+                          const float *__restrict__ W2, __nv_bfloat16 *W1b, __nv_bfloat16 *W2b) {
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nth = (int64_t)gridDim.x * blockDim.x;
   const int64_t n = (int64_t)H * Dp;
-  const int64_t K1 = split ? 3 * Dp : Dp, K2 = split ? 3 * H : H;
   for (int64_t i = tid; i < n; i += nth) {
-    __nv_bfloat16 hi, lo;
-    {  // W1 [H x Dp]
-      const int64_t j = i / Dp, c = i - j * Dp;
-      bf16_split(W1[i], hi, lo);
-      W1b[j * K1 + c] = hi;
-      if (split) {
-        W1b[j * K1 + Dp + c] = lo;
-        W1b[j * K1 + 2 * Dp + c] = hi;
-      }
-    }
-    {  // W2 [Dp x H]
-      const int64_t r = i / H, c = i - r * H;
-      bf16_split(W2[i], hi, lo);
-      W2b[r * K2 + c] = hi;
-      if (split) {
-        W2b[r * K2 + H + c] = lo;
-        W2b[r * K2 + 2 * H + c] = hi;
-      }
-      W2tb[c * Dp + r] = hi;
-    }
+    store_weight(W1b, i / Dp, (int)(i % Dp), Dp, split, W1[i]);  // [H x Dp]
+    store_weight(W2b, i / H, (int)(i % H), H, split, W2[i]);     // [Dp x H]
   }
 }
 
@@ -366,14 +319,11 @@ int mlp_odd_matrix(bs_mlp *m, cudaStream_t s) {
 
 static void free_scratch(bs_mlp *m) {
   cudaFree(m->Xb);
-  cudaFree(m->Xtb);
   cudaFree(m->Hb);
-  cudaFree(m->Htb);
   cudaFree(m->dYb);
-  cudaFree(m->dYtb);
-  cudaFree(m->dZtb);
+  cudaFree(m->dZb);
   cudaFree(m->Y);
-  m->Xb = m->Xtb = m->Hb = m->Htb = m->dYb = m->dYtb = m->dZtb = nullptr;
+  m->Xb = m->Hb = m->dYb = m->dZb = nullptr;
   m->Y = nullptr;
   m->Bcap = 0;
 }
@@ -388,12 +338,9 @@ int mlp_ensure(bs_mlp *m, int64_t B) {
   };
   const int64_t k3 = m->split ? 3 : 1;
   A((void **)&m->Xb, 2 * B * Dp * k3);
-  A((void **)&m->Xtb, 2 * B * Dp);
   A((void **)&m->Hb, 2 * B * H * k3);
-  A((void **)&m->Htb, 2 * B * H);
   A((void **)&m->dYb, 2 * B * Dp);
-  A((void **)&m->dYtb, 2 * B * Dp);
-  A((void **)&m->dZtb, 2 * B * H);
+  A((void **)&m->dZb, 2 * B * H);
   A((void **)&m->Y, 4 * B * Dp);
   if (e != cudaSuccess) {
     free_scratch(m);
@@ -411,94 +358,120 @@ static int check_mlp(const bs_mlp *m, const char *fn) {
   return BS_OK;
 }
 
-int mlp_forward_packed(bs_mlp *m, int64_t B, int relu, GemmArgs b, int out_epi, cudaStream_t s) {
-  const int K1 = m->split ? 3 * m->Dp : m->Dp, K2 = m->split ? 3 * m->H : m->H;
+// The layers' products on the packed input Xb: Hb = act(Xb W1^T), Hb W2^T.
+static GemmArgs hidden_args(const bs_mlp *m, int64_t B, int relu) {
+  const int K1 = m->split ? 3 * m->Dp : m->Dp;
   GemmArgs a{};
   a.A = m->Xb;
   a.B = m->W1b;
   a.M = B;
   a.N = m->H;
-  a.K = K1;
-  a.lda = K1;
-  a.ldb = K1;
-  a.ldc = K2;
+  a.K = a.lda = a.ldb = K1;
+  a.ldc = m->split ? 3 * m->H : m->H;
   a.out_b16 = m->Hb;
   a.relu = relu;
   a.split = m->split ? m->H : 0;
-  a.st = b.st;
-  if (int rc = launch_gemm(EPI_HIDDEN, a, s)) return rc;
+  return a;
+}
+static GemmArgs output_args(const bs_mlp *m, int64_t B, GemmArgs b = GemmArgs{}) {
   b.A = m->Hb;
   b.B = m->W2b;
   b.M = B;
   b.N = m->Dp;
-  b.K = K2;
-  b.lda = K2;
-  b.ldb = K2;
-  return launch_gemm(out_epi, b, s);
+  b.K = b.lda = b.ldb = m->split ? 3 * m->H : m->H;
+  return b;
 }
 
-// Forward of f on Xb: Y [B x Dp] (float).
-static int forward_packed(bs_mlp *m, int64_t B, cudaStream_t s) {
-  GemmArgs b{};
-  b.ldc = m->Dp;
-  b.out_f32 = m->Y;
-  return mlp_forward_packed(m, B, 1, b, EPI_F32, s);
+int mlp_forward_packed(bs_mlp *m, int64_t B, int relu, GemmArgs b, int out_epi, cudaStream_t s) {
+  GemmArgs a = hidden_args(m, B, relu);
+  a.st = b.st;
+  if (int rc = launch_gemm(EPI_HIDDEN, a, s)) return rc;
+  return launch_gemm(out_epi, output_args(m, B, b), s);
 }
 
-// Forward + MSE + backward into m->g1 (H x Dp), m->g2 (Dp x H) (float).
+// Forward + MSE + backward: the gradients into m->g1 (H x Dp) and m->g2 (Dp x H)
+// (float), or, with adam, straight into an Adam step on the weights.
 static int loss_grad(bs_mlp *m, int64_t B, const float *X, const float *T, double *d_loss,
-                     cudaStream_t s) {
+                     const TrainArgs *adam, cudaStream_t s) {
   const int Dp = m->Dp, H = m->H, D = m->D;
   const int K1 = m->split ? 3 * Dp : Dp, K2 = m->split ? 3 * H : H;
   const int grid = stream_grid(B * Dp, 1, 256, 8);
   k_pack_bf16<<<grid, 256, 0, s>>>(B, D, Dp, m->split, X, m->Xb);
   BS_LAUNCH_CHECK();
-  if (int rc = forward_packed(m, B, s)) return rc;
-  k_mse<<<stream_grid(B * Dp, 1, kReduceBlock, 4), kReduceBlock, 0, s>>>(
-      B, D, Dp, m->Y, T, m->dYb, m->lossp, m->cnt, d_loss);
-  BS_LAUNCH_CHECK();
-  if (int rc = transpose((int)B, Dp, K1, m->Xb, m->Xtb, s)) return rc;   // hi(X)^T [Dp x B]
-  if (int rc = transpose((int)B, H, K2, m->Hb, m->Htb, s)) return rc;    // hi(H)^T [H x B]
-  if (int rc = transpose((int)B, Dp, Dp, m->dYb, m->dYtb, s)) return rc; // dY^T [Dp x B]
-  // gW2 [Dp x H] = dY^T H
-  GemmArgs g2{};
-  g2.A = m->dYtb;
-  g2.B = m->Htb;
-  g2.M = Dp;
-  g2.N = H;
-  g2.K = (int)B;
-  g2.lda = (int)B;
-  g2.ldb = (int)B;
-  g2.ldc = H;
-  g2.out_f32 = m->g2;
-  if (int rc = launch_gemm(EPI_F32, g2, s)) return rc;
-  // dZ [B x H] = (dY W2) * relu'(hidden); W2 as B operand is W2^T [H x Dp]
+  DeviceInfo di;
+  if (int rc = device_info(&di)) return rc;
+  if (gs_blocks(B, Dp, gs_tile(B, Dp, di.sms)) <= kMaxPartials) {
+    if (int rc = launch_gemm(EPI_HIDDEN, hidden_args(m, B, 1), s)) return rc;
+    GemmArgs b = output_args(m, B);
+    b.ldc = Dp;
+    b.out_b16 = m->dYb;
+    TrainArgs ta{};
+    ta.target = T;
+    ta.D = D;
+    ta.partials = m->lossp;
+    ta.counter = m->cnt;
+    ta.loss = d_loss;
+    if (int rc = launch_gemm_s<EPI_MSE, false, false>(b, ta, s)) return rc;
+  } else {  // more blocks than the loss has partials
+    GemmArgs b{};
+    b.ldc = Dp;
+    b.out_f32 = m->Y;
+    if (int rc = mlp_forward_packed(m, B, 1, b, EPI_F32, s)) return rc;
+    k_mse<<<stream_grid(B * Dp, 1, kReduceBlock, 4), kReduceBlock, 0, s>>>(
+        B, D, Dp, m->Y, T, m->dYb, m->lossp, m->cnt, d_loss);
+    BS_LAUNCH_CHECK();
+  }
+  // dZ [B x H] = (dY W2) * relu'(hidden), before W2 changes; W2's hi part is
+  // the first H columns of W2b [Dp x K2]
   GemmArgs dz{};
   dz.A = m->dYb;
-  dz.B = m->W2tb;
+  dz.B = m->W2b;
   dz.M = B;
   dz.N = H;
   dz.K = Dp;
   dz.lda = Dp;
-  dz.ldb = Dp;
+  dz.ldb = K2;
   dz.ldc = H;
-  dz.out_b16 = m->Htb;  // reuse: H^T already consumed by gW2 above (same stream)
+  dz.out_b16 = m->dZb;
   dz.mask = m->Hb;
   dz.ldmask = K2;
-  if (int rc = launch_gemm(EPI_MASK_BF16, dz, s)) return rc;
-  if (int rc = transpose((int)B, H, H, m->Htb, m->dZtb, s)) return rc;   // dZ^T [H x B]
-  // gW1 [H x Dp] = dZ^T X
+  if (int rc = launch_gemm_s<EPI_MASK_BF16, false, true>(dz, TrainArgs{}, s)) return rc;
+  // gW2 [Dp x H] = dY^T H and gW1 [H x Dp] = dZ^T X (hi parts)
+  GemmArgs g2{};
+  g2.A = m->dYb;
+  g2.B = m->Hb;
+  g2.M = Dp;
+  g2.N = H;
+  g2.K = (int)B;
+  g2.lda = Dp;
+  g2.ldb = K2;
+  g2.ldc = H;
+  g2.out_f32 = m->g2;
   GemmArgs g1{};
-  g1.A = m->dZtb;
-  g1.B = m->Xtb;
+  g1.A = m->dZb;
+  g1.B = m->Xb;
   g1.M = H;
   g1.N = Dp;
   g1.K = (int)B;
-  g1.lda = (int)B;
-  g1.ldb = (int)B;
+  g1.lda = H;
+  g1.ldb = K1;
   g1.ldc = Dp;
   g1.out_f32 = m->g1;
-  return launch_gemm(EPI_F32, g1, s);
+  GsArgs a{};
+  a.g[0] = g2;
+  a.g[1] = g1;
+  if (!adam) return launch_gemm_s<EPI_F32, true, true>(a, 1, s);
+  a.t[0] = a.t[1] = *adam;
+  a.t[0].w = m->W2;
+  a.t[0].m1 = m->m2;
+  a.t[0].m2 = m->v2;
+  a.t[0].wb = m->W2b;
+  a.t[1].w = m->W1;
+  a.t[1].m1 = m->m1;
+  a.t[1].m2 = m->v1;
+  a.t[1].wb = m->W1b;
+  a.t[0].split = a.t[1].split = m->split;
+  return launch_gemm_s<EPI_ADAM, true, true>(a, 1, s);
 }
 
 static void free_mlp(bs_mlp *m) {
@@ -533,11 +506,11 @@ int bs_mlp_create(int32_t D, int32_t H, const float *h_W1, const float *h_W2, in
   m->split = (flags & BS_MLP_BF16X3) ? 1 : 0;
   const size_t n = (size_t)H * m->Dp;
   // one allocation: W1, W2, m1, v1, m2, v2, g1, g2 (float) + bf16 operands
-  // W1b (3n), W2b (3n), W2tb (n)
+  // W1b (3n), W2b (3n)
   cudaError_t e = cudaGetDevice(&m->device);
   char *base = nullptr;
-  if (e == cudaSuccess) e = cudaMalloc(&base, n * (8 * sizeof(float) + 7 * 2) + 256);
-  if (e == cudaSuccess) e = cudaMemset(base, 0, n * (8 * sizeof(float) + 7 * 2) + 256);
+  if (e == cudaSuccess) e = cudaMalloc(&base, n * (8 * sizeof(float) + 6 * 2) + 256);
+  if (e == cudaSuccess) e = cudaMemset(base, 0, n * (8 * sizeof(float) + 6 * 2) + 256);
   {  // L (float Dp x Dp) then Lb (bf16 Dp x 3 Dp)
     const size_t nl = (size_t)m->Dp * m->Dp;
     if (e == cudaSuccess) e = cudaMalloc(&m->L, nl * (sizeof(float) + 3 * 2) + 256);
@@ -586,7 +559,6 @@ int bs_mlp_create(int32_t D, int32_t H, const float *h_W1, const float *h_W2, in
   __nv_bfloat16 *bb = reinterpret_cast<__nv_bfloat16 *>(f + 8 * n);
   m->W1b = bb;
   m->W2b = bb + 3 * n;
-  m->W2tb = bb + 6 * n;
   m->cnt = reinterpret_cast<unsigned int *>(m->lossp + kMaxPartials);
   // padded host copies -> device
   float *p1 = (float *)calloc(n, sizeof(float)), *p2 = (float *)calloc(n, sizeof(float));
@@ -609,7 +581,7 @@ int bs_mlp_create(int32_t D, int32_t H, const float *h_W1, const float *h_W2, in
     return fail(BS_ERR_CUDA, "bs_mlp_create: %s", cudaGetErrorString(e));
   }
   k_refresh<<<stream_grid((int64_t)n, 1, 256, 8), 256>>>(H, m->Dp, m->split, m->W1, m->W2,
-                                                          m->W1b, m->W2b, m->W2tb);
+                                                          m->W1b, m->W2b);
   e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     free_mlp(m);
@@ -699,7 +671,7 @@ int bs_mlp_load_state(bs_mlp *m, const void *h_buf, int64_t nbytes) {
   m->odd_step = -1;  // derived operands are stale
   m->int_step = -1;
   k_refresh<<<stream_grid((int64_t)n, 1, 256, 8), 256>>>(m->H, m->Dp, m->split, m->W1, m->W2,
-                                                          m->W1b, m->W2b, m->W2tb);
+                                                          m->W1b, m->W2b);
   BS_CUDA_TRY(cudaDeviceSynchronize());
   return BS_OK;
 }
@@ -735,7 +707,7 @@ int bs_mlp_loss_grad(bs_mlp *m, int64_t B, const float *d_X, const float *d_T, d
   BS_ARG(d_X && d_T && d_loss, "bs_mlp_loss_grad: NULL argument");
   if (int rc = mlp_ensure(m, B)) return rc;
   cudaStream_t s = as_stream(stream);
-  if (int rc = loss_grad(m, B, d_X, d_T, d_loss, s)) return rc;
+  if (int rc = loss_grad(m, B, d_X, d_T, d_loss, nullptr, s)) return rc;
   if (d_gW1) {
     k_unpad_cols<<<stream_grid((int64_t)m->H * m->D, 1, 256, 8), 256, 0, s>>>(m->H, m->D, m->Dp,
                                                                               m->g1, d_gW1);
@@ -757,16 +729,16 @@ int bs_mlp_train_step(bs_mlp *m, int64_t B, const float *d_X, const float *d_T, 
   BS_ARG(lr > 0.f && std::isfinite(lr), "bs_mlp_train_step: lr must be positive");
   if (int rc = mlp_ensure(m, B)) return rc;
   cudaStream_t s = as_stream(stream);
-  if (int rc = loss_grad(m, B, d_X, d_T, d_loss, s)) return rc;
-  m->step += 1;
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float c1 = 1.0f - powf(b1, (float)m->step), c2 = 1.0f - powf(b2, (float)m->step);
-  const int64_t n = (int64_t)m->H * m->Dp;
-  const int grid = stream_grid(n, 1, 256, 8);
-  k_adam<<<grid, 256, 0, s>>>(n, m->W1, m->g1, m->m1, m->v1, lr, b1, b2, eps, c1, c2);
-  k_adam<<<grid, 256, 0, s>>>(n, m->W2, m->g2, m->m2, m->v2, lr, b1, b2, eps, c1, c2);
-  k_refresh<<<grid, 256, 0, s>>>(m->H, m->Dp, m->split, m->W1, m->W2, m->W1b, m->W2b, m->W2tb);
-  BS_LAUNCH_CHECK();
+  const int step = m->step + 1;
+  TrainArgs ta{};
+  ta.lr = lr;
+  ta.b1 = 0.9f;
+  ta.b2 = 0.999f;
+  ta.eps = 1e-8f;
+  ta.c1 = 1.0f - powf(ta.b1, (float)step);
+  ta.c2 = 1.0f - powf(ta.b2, (float)step);
+  if (int rc = loss_grad(m, B, d_X, d_T, d_loss, &ta, s)) return rc;
+  m->step = step;
   return BS_OK;
 }
 

@@ -31,13 +31,13 @@ struct bs_mlp {
   float *W1, *W2;                   // FP32 master weights, W1 [H x Dp], W2 [Dp x H]
   float *m1, *v1, *m2, *v2;         // Adam moments
   // bf16 operands: W1b [H x K1], W2b [Dp x K2] (K1 = Dp, K2 = H, tripled in
-  // BF16x3 mode as [hi | lo | hi]) and W2tb = hi(W2)^T [H x Dp]
-  __nv_bfloat16 *W1b, *W2b, *W2tb;
+  // BF16x3 mode as [hi | lo | hi])
+  __nv_bfloat16 *W1b, *W2b;
   int step;                         // Adam steps taken
   // training scratch for batches of up to Bcap rows: Xb [B x K1], Hb [B x K2]
   // (activation operands, [hi | hi | lo] rows in BF16x3 mode), the rest bf16
   int64_t Bcap;
-  __nv_bfloat16 *Xb, *Xtb, *Hb, *Htb, *dYb, *dYtb, *dZtb;
+  __nv_bfloat16 *Xb, *Hb, *dYb, *dZb;
   float *Y, *g1, *g2;
   double *lossp;                    // per-block loss partials + counter
   unsigned int *cnt;

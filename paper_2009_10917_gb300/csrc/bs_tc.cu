@@ -229,8 +229,7 @@ __global__ void __launch_bounds__(kTcThreads) k_gemm_tc(GemmArgs g, int *err) {
 
 bool gemm_tc_supported(int epi, const GemmArgs &a) {
   return g_gemm_engine == 1 && a.K % 8 == 0 && a.K >= 8 && a.lda % 8 == 0 &&
-         a.ldb % 8 == 0 && ((uintptr_t)a.A % 16) == 0 && ((uintptr_t)a.B % 16) == 0 &&
-         epi != EPI_MASK_BF16;
+         a.ldb % 8 == 0 && ((uintptr_t)a.A % 16) == 0 && ((uintptr_t)a.B % 16) == 0;
 }
 
 template <int EPI>
