@@ -753,7 +753,7 @@ static int build_batch(Batch &B, int ns, const bs_problem *const *P, const doubl
     d.tabff = p->d_tabff;
     d.g = 0.5 * p->h;
     d.mlam = p->lambda * d.g * d.g * d.g;
-    const int64_t sv = m->NG + 2;
+    const int64_t sv = vec_stride(m->NG);
     d.x = x[s];
     d.b = b[s];
     d.r = p->d_vec;
@@ -761,7 +761,7 @@ static int build_batch(Batch &B, int ns, const bs_problem *const *P, const doubl
     d.Ap = p->d_vec + 2 * sv;
     d.ApL = p->d_ApL;
     if (f32) {
-      const size_t n = (size_t)m->NG + 8;
+      const size_t n = (size_t)vec_stride_f32(m->NG);
       d.rf = p->d_f32;
       d.pf = p->d_f32 + n;
       d.Apf = p->d_f32 + 2 * n;
@@ -946,7 +946,7 @@ static int check_batch(int32_t nsolves, const bs_problem *const *probs, const do
     for (int t = 0; t < s; ++t) BS_ARG(probs[t] != probs[s], "%s: problem %d repeats %d", fn, s, t);
     if (f32 && !probs[s]->d_f32) {
       bs_problem *p = const_cast<bs_problem *>(probs[s]);
-      BS_CUDA_TRY(cudaMalloc(&p->d_f32, sizeof(float) * 4 * ((size_t)p->map->NG + 8)));
+      BS_CUDA_TRY(cudaMalloc(&p->d_f32, sizeof(float) * 4 * (size_t)vec_stride_f32(p->map->NG)));
     }
   }
   return BS_OK;

@@ -150,7 +150,7 @@ struct CgVecs {
   double *r, *p, *Ap, *z, *dinv;
 };
 static CgVecs vecs(const bs_problem *P) {
-  const int64_t s = P->map->NG + 2;
+  const int64_t s = vec_stride(P->map->NG);
   return CgVecs{P->d_vec, P->d_vec + s, P->d_vec + 2 * s, P->d_vec + 3 * s, P->d_vec + 4 * s};
 }
 
@@ -543,7 +543,7 @@ extern "C" int bs_cg_solve(const bs_problem *Pc, const double *b, double *x, dou
       const double bb0 = P->h_state->bb;
       if (bb0 > 0.0 && std::isfinite(bb0)) {
         ff_scale = std::ldexp(1.0, -std::ilogb(std::sqrt(bb0 / (double)NG)));
-        double *bs_ = P->d_vec + 5 * (NG + 2);
+        double *bs_ = P->d_vec + 5 * vec_stride(NG);
         BS_TRY(launch_copy<double>(NG, b, bs_, s));
         const int grid = stream_grid(NG, 1, kStreamBlock, 8);
         k_scale<<<grid, kStreamBlock, 0, s>>>(NG, ff_scale, bs_);

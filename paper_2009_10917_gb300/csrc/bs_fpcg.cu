@@ -321,7 +321,7 @@ struct FpVecs {
   double *r, *p, *Ap, *z, *dinv, *corr;
 };
 static FpVecs fpvecs(const bs_problem *P) {
-  const int64_t s = P->map->NG + 2;
+  const int64_t s = vec_stride(P->map->NG);
   double *v = P->d_vec;
   return FpVecs{v, v + s, v + 2 * s, v + 3 * s, v + 4 * s, v + 5 * s};
 }

@@ -395,7 +395,7 @@ int bs_problem_create(const bs_map *map, double h, double lambda, const double *
   if (e == cudaSuccess) e = cudaMalloc(&p->d_tabff, sizeof(tabff));
   if (e == cudaSuccess) e = cudaMemcpy(p->d_tabff, &tabff, sizeof(tabff), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_ApL, sizeof(double) * (NL + 2));
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_vec, sizeof(double) * 6 * (NG + 2));
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_vec, sizeof(double) * 6 * vec_stride(NG));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_state, sizeof(CgState));
   if (e == cudaSuccess) e = cudaMemset(p->d_state, 0, sizeof(CgState));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_partials, sizeof(double) * kMaxPartials + 256);

@@ -464,6 +464,14 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
 
 struct OpTabFF;  // bs_op_ff.cuh
 
+// Distances of a problem's vectors in d_vec and d_f32, such that each starts
+// on a 16-byte boundary whatever N_G: with N_G + 2 an odd N_G (every
+// unmasked mesh of odd N, or even K) left every second vector 8 bytes off, and
+// the CG kernels, whose operands then shared no alignment, on their scalar
+// path.
+inline int64_t vec_stride(int64_t NG) { return (NG + 3) & ~(int64_t)1; }
+inline int64_t vec_stride_f32(int64_t NG) { return (NG + 11) & ~(int64_t)3; }
+
 }  // namespace bs
 
 // A problem: the map, the geometry and the device scratch of the solvers.
@@ -478,7 +486,7 @@ struct bs_problem {
   bs::OpTab<float> *d_tabf;       // FP32 tables
   bs::OpTabFF *d_tabff;           // float-pair tables of the float-float operator
   double *d_ApL;                  // [NL] local operator output (FP64 or FP32 view)
-  double *d_vec;                  // 6 x [NG]: r, p, Ap, z, dinv, spare
+  double *d_vec;                  // 6 x [vec_stride(NG)]: r, p, Ap, z, dinv, spare
   bs::CgState *d_state;
   double *d_partials;             // [kMaxPartials]
   double *d_op_partials;          // [E + 1] the fused operator's block partials (<= E blocks)
@@ -487,7 +495,7 @@ struct bs_problem {
   cudaStream_t cap_stream;        // private stream for graph capture
   cudaGraphExec_t graph;          // cached CG chunk graph
   const void *graph_key[4];       // (x, variant, chunk, map) the graph was made for
-  float *d_f32;                   // 4 x [NG + 8] FP32 vectors (refined solver), lazily
+  float *d_f32;                   // 4 x [vec_stride_f32(NG)] FP32 vectors (refined solver), lazily
   double *d_Lvec;                 // 6 x [NL + 2 rounded up to even] scattered CG vectors, lazily
   uint8_t *d_owner;               // [NL + 16] 1 at the lowest local copy of each node, lazily
   void *d_bj;                     // block-Jacobi tables and per-element flags, lazily

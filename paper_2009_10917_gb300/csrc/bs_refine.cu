@@ -103,13 +103,13 @@ struct F32Vecs {
 
 static int ensure_f32(bs_problem *P) {
   if (P->d_f32) return BS_OK;
-  const size_t n = (size_t)P->map->NG + 8;
+  const size_t n = (size_t)vec_stride_f32(P->map->NG);
   BS_CUDA_TRY(cudaMalloc(&P->d_f32, sizeof(float) * 4 * n));
   return BS_OK;
 }
 
 static F32Vecs f32vecs(const bs_problem *P) {
-  const size_t n = (size_t)P->map->NG + 8;  // keeps each vector 16-byte aligned
+  const size_t n = (size_t)vec_stride_f32(P->map->NG);
   return F32Vecs{P->d_f32, P->d_f32 + n, P->d_f32 + 2 * n, P->d_f32 + 3 * n};
 }
 
@@ -188,7 +188,7 @@ extern "C" int bs_cg_solve_refined_f32(const bs_problem *Pc, const double *b, do
   if (rc) return rc;
   cudaStream_t s = as_stream(stream);
   const bool graph = flags & BS_CG_GRAPH;
-  const int64_t sv = NG + 2;
+  const int64_t sv = vec_stride(NG);
   double *r64 = P->d_vec, *Ax = P->d_vec + 2 * sv, *scal = P->d_vec + 5 * sv;  // scal[0..1]
   F32Vecs v = f32vecs(P);
   CgState *st = P->d_state;
