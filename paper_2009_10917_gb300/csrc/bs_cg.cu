@@ -5,9 +5,9 @@
 //   1. ApL = A_L (Z p)                 fused scatter + element operator
 //   2. Ap = Z^T ApL, pAp = p.Ap        gather (BS6) with a fused dot;
 //                                      its last block forms alpha = rr / pAp
-//   3. x += alpha p, r -= alpha Ap,    fused CG update (BS5); its last block
-//      rr' = r.r                       forms beta = rr'/rr and the stop flag
-//   4. p = r + beta p                  AXPY (BS2), p = fma(1, r, beta p)
+//   3. r -= alpha Ap, rr' = r.r        the last block forms beta = rr'/rr and
+//                                      the stop flag
+//   4. x += alpha p, p = r + beta p    BS5's other half with BS2 (bs_cgvec.cuh)
 // Kernels return at once when the device stop flag is set, so a chunk of
 // iterations can be enqueued -- or replayed as one CUDA graph -- and the host
 // reads the flag back once per chunk.
@@ -27,6 +27,7 @@
 #include <cmath>
 
 #include "bs_bj.cuh"
+#include "bs_cgvec.cuh"
 #include "bs_op_ff.cuh"
 
 namespace bs {
@@ -76,30 +77,54 @@ struct EpBeta {  // rr' -> beta = rr'/rr (Algorithm 1, step 10)
   }
 };
 
-// Jacobi-PCG update: x += alpha p; r -= alpha Ap; z = dinv r; sums r.r, r.z.
+// Jacobi-PCG's r pass: r -= alpha Ap; z = dinv r; sums r.r, r.z (init: z and
+// the sums alone).  The vectors are the problem's own, 16-byte aligned.
 template <int U>
 __global__ void __launch_bounds__(kReduceBlock)
-    k_pcg_update(int64_t n, const double *__restrict__ p, const double *__restrict__ Ap,
-                 const double *__restrict__ dinv, double *__restrict__ x,
-                 double *__restrict__ r, double *__restrict__ z, double *partials,
-                 unsigned int *counter, CgState *st, int init, int defer) {
-  if (!init && cg_halted(st)) return;
-  const double alpha = init ? 0.0 : st->alpha;
-  const double nalpha = -alpha;
+    k_pcg_r(int64_t n, const double *__restrict__ Ap, const double *__restrict__ dinv,
+            double *__restrict__ r, double *__restrict__ z, double *partials,
+            unsigned int *counter, CgState *st, int init, int defer) {
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+  if (!init && cg_halted(st)) {
+    if (tid == 0) st->xdue = 0;
+    return;
+  }
+  const double nalpha = init ? 0.0 : -st->alpha;
   double rr = 0.0, rz = 0.0;
-  for (int64_t i = tid; i < n; i += nth) {
-    double ri = r[i];
-    if (!init) {
-      x[i] = fma(alpha, p[i], x[i]);
-      ri = fma(nalpha, Ap[i], ri);
-      r[i] = ri;
-    }
-    const double zi = ri * dinv[i];
-    z[i] = zi;
+  auto one = [&](double a, double d, double &ri, double &zi) {
+    if (!init) ri = fma(nalpha, a, ri);
+    zi = ri * d;
     rr = fma(ri, ri, rr);
     rz = fma(ri, zi, rz);
+  };
+  const int64_t nv = n / 2;
+  for (int64_t i0 = tid; i0 < nv; i0 += U * nth) {
+    double2 a[U], d[U], rv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + u * nth;
+      if (i >= nv) break;
+      a[u] = init ? make_double2(0.0, 0.0) : reinterpret_cast<const double2 *>(Ap)[i];
+      d[u] = ld_stream(reinterpret_cast<const double2 *>(dinv) + i);
+      rv[u] = reinterpret_cast<const double2 *>(r)[i];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + u * nth;
+      if (i >= nv) break;
+      double2 zv;
+      one(a[u].x, d[u].x, rv[u].x, zv.x);
+      one(a[u].y, d[u].y, rv[u].y, zv.y);
+      if (!init) reinterpret_cast<double2 *>(r)[i] = rv[u];
+      reinterpret_cast<double2 *>(z)[i] = zv;
+    }
+  }
+  if ((n & 1) && tid == 0) {
+    double ri = r[n - 1], zi;
+    one(init ? 0.0 : Ap[n - 1], dinv[n - 1], ri, zi);
+    r[n - 1] = ri;
+    z[n - 1] = zi;
   }
   const double prr = block_sum<kReduceBlock>(rr);
   const double prz = block_sum<kReduceBlock>(rz);
@@ -112,13 +137,16 @@ __global__ void __launch_bounds__(kReduceBlock)
       st->done = !(isfinite(trr) && isfinite(trz))
                      ? 2
                      : ((!st->fixed && trr <= st->eps) ? 1 : (st->maxit <= 0 ? 3 : 0));
-    } else if (defer) {  // block Jacobi completes z and r.z, then advances
-      st->rr_next = trr;
-      st->rz_next = trz;
     } else {
-      const double beta = trz / st->rz;
-      st->rz = trz;
-      cg_advance(st, trr, beta);
+      st->xdue = 1;
+      if (defer) {  // block Jacobi completes z and r.z, then advances
+        st->rr_next = trr;
+        st->rz_next = trz;
+      } else {
+        const double beta = trz / st->rz;
+        st->rz = trz;
+        cg_advance(st, trr, beta);
+      }
     }
   }
 }
@@ -154,15 +182,16 @@ static CgVecs vecs(const bs_problem *P) {
   return CgVecs{P->d_vec, P->d_vec + s, P->d_vec + 2 * s, P->d_vec + 3 * s, P->d_vec + 4 * s};
 }
 
-// The Jacobi-PCG update; bj: then the element-interior blocks of the
+// Jacobi-PCG's r pass; bj: then the element-interior blocks of the
 // block-Jacobi preconditioner, which complete z and r.z and advance.
-static int pcg_update_launch(const bs_problem *P, double *x, int init, cudaStream_t s,
-                             bool bj = false) {
+static int pcg_r_launch(const bs_problem *P, int init, cudaStream_t s, bool bj = false) {
   CgVecs v = vecs(P);
-  auto kern = k_pcg_update<1>;
-  int grid = stream_grid(P->map->NG, 2, kReduceBlock, blocks_per_sm(kern, kReduceBlock));
+  constexpr int U = 2;
+  auto kern = k_pcg_r<U>;
+  int grid =
+      stream_grid(P->map->NG / 2 + 1, U, kReduceBlock, blocks_per_sm(kern, kReduceBlock));
   if (grid > kMaxPartials / 2) grid = kMaxPartials / 2;
-  kern<<<grid, kReduceBlock, 0, s>>>(P->map->NG, v.p, v.Ap, v.dinv, x, v.r, v.z, P->d_partials,
+  kern<<<grid, kReduceBlock, 0, s>>>(P->map->NG, v.Ap, v.dinv, v.r, v.z, P->d_partials,
                                      P->d_counter, P->d_state, init, bj ? 1 : 0);
   BS_LAUNCH_CHECK();
   if (bj) return bj_apply(P, v.r, v.dinv, v.z, init, s);
@@ -434,8 +463,8 @@ static int scat_setup(bs_problem *P, const double *x, bool x0, bool precond, dou
   return launch_copy<double>(m->NL, precond ? L.z : L.r, L.p, s);
 }
 
-// One CG iteration (four launches: the operator with p.Ap, the fused update
-// with r.r, the direction).  ff: the float-float element operator.
+// One CG iteration (four launches: the operator with p.Ap, r with r.r, x and
+// the direction).  ff: the float-float element operator.
 static int cg_iteration(const bs_problem *P, double *x, bool precond, bool ff, cudaStream_t s,
                         bool bj = false) {
   const bs_map *m = P->map;
@@ -446,14 +475,13 @@ static int cg_iteration(const bs_problem *P, double *x, bool precond, bool ff, c
                                                  EpAlpha{st, precond ? 1 : 0}, st, s);
   if (rc) return rc;
   if (precond) {
-    rc = pcg_update_launch(P, x, 0, s, bj);
+    rc = pcg_r_launch(P, 0, s, bj);
   } else {
-    rc = launch_cg_update<double, EpBeta>(m->NG, Scalar<double>{0.0, &st->alpha}, v.p, v.Ap, x,
-                                          v.r, P->d_partials, P->d_counter, EpBeta{st}, st, s);
+    rc = launch_cg_r<double, EpBeta>(m->NG, &st->alpha, v.Ap, v.r, P->d_partials, P->d_counter,
+                                     EpBeta{st}, st, s);
   }
   if (rc) return rc;
-  return launch_axpy<double>(m->NG, Scalar<double>{1.0, nullptr}, precond ? v.z : v.r,
-                             Scalar<double>{0.0, &st->beta}, v.p, st, s);
+  return launch_cg_xp<double>(m->NG, &st->alpha, &st->beta, precond ? v.z : v.r, x, v.p, st, s);
 }
 
 static int capture_chunk(bs_problem *P, double *x, bool precond, bool ff, bool scat,
@@ -571,7 +599,7 @@ extern "C" int bs_cg_solve(const bs_problem *Pc, const double *b, double *x, dou
     } else if (precond) {
       if (bj) BS_TRY(bj_ensure(P, s));
       k_set_state<<<1, 1, 0, s>>>(st, tol * tol, maxit, fixed ? 1 : 0, d_hist);
-      BS_TRY(pcg_update_launch(P, x, 1, s, bj));  // z = M^-1 r, rr, rz, stop flag
+      BS_TRY(pcg_r_launch(P, 1, s, bj));  // z = M^-1 r, rr, rz, stop flag
       BS_TRY(launch_copy<double>(NG, v.z, v.p, s));
     } else {
       BS_TRY(launch_copy<double>(NG, v.r, v.p, s));

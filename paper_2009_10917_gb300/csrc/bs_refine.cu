@@ -5,7 +5,7 @@
 //   r = b - A x,  stop when ||r|| <= tol ||b||,  x = x + d.
 // Inner, Algorithm 1 on A d = r with every vector and the operator in FP32:
 // the same four kernels per iteration as the FP64 solver (fused scatter +
-// element operator, gather with p.Ap, fused update with r.r, AXPY), their
+// element operator, gather with p.Ap, r with r.r, x with the direction), their
 // reductions carried as float pairs and combined in double, alpha and beta
 // formed in double and rounded to float for the updates.  Each inner solve
 // stops at ||r_d|| <= inner_tol ||r||.  Halving the bytes of every vector and
@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "bs_cgvec.cuh"
 #include "bs_op_ff.cuh"
 
 namespace bs {
@@ -124,11 +125,10 @@ static int f32_iteration(const bs_problem *P, cudaStream_t s) {
   int rc = apply_A_global<float, true, EpAlphaF>(P, false, P->d_tabf, v.p, v.Ap, ApL, g, mlam,
                                                   EpAlphaF{st}, st, s);
   if (rc) return rc;
-  rc = launch_cg_update<float, EpBetaF>(m->NG, Scalar<float>{0.f, &st->alpha_f}, v.p, v.Ap, v.d,
-                                        v.r, P->d_partials, P->d_counter, EpBetaF{st}, st, s);
+  rc = launch_cg_r<float, EpBetaF>(m->NG, &st->alpha_f, v.Ap, v.r, P->d_partials, P->d_counter,
+                                   EpBetaF{st}, st, s);
   if (rc) return rc;
-  return launch_axpy<float>(m->NG, Scalar<float>{1.f, nullptr}, v.r,
-                            Scalar<float>{0.f, &st->beta_f}, v.p, st, s);
+  return launch_cg_xp<float>(m->NG, &st->alpha_f, &st->beta_f, v.r, v.d, v.p, st, s);
 }
 
 static int capture_f32(bs_problem *P, int chunk) {

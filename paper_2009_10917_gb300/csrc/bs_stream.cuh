@@ -102,6 +102,7 @@ struct CgState {
   double *hist;   // optional [3*(maxit+1)] alpha, beta, rr per iteration
   double rr_next; // block-Jacobi PCG: r.r and the Jacobi part of r.z of the
   double rz_next; // update, held until the interior blocks are solved
+  int xdue;       // 1: the r pass of this iteration ran, x and p follow
 };
 
 __device__ __forceinline__ bool cg_halted(const CgState *st) {
