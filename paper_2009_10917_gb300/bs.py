@@ -157,6 +157,8 @@ def _device_check(result, func, args):
 def lib():
     """Load libbs.so (building it first if the sources are newer)."""
     global _lib
+    if _lib is not None:  # set last, with every entry point bound
+        return _lib
     with _lock:
         if _lib is None:
             chk = checked()
@@ -189,20 +191,30 @@ def _check(rc, fn):
         raise BSError(rc, fn, L.bs_last_error().decode(errors="replace"))
 
 
+# A call on a few thousand values is host work: torch's stream objects, ctypes
+# pointer objects and a lock per call were two thirds of it (the five vector
+# operations on 4099 values: 73 us, 41 us with plain integers).
+_device = torch._C._cuda_getDevice if hasattr(torch._C, "_cuda_getDevice") else None
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """torch's current stream as an address (the caller holds a CUDA tensor, so
+    CUDA is initialised)."""
+    return _raw_stream(_device())
 
 
 def _ptr(t, dtype=torch.float64, name="tensor"):
+    """The checked tensor's address (0 for an empty one)."""
     if t is None:
         return None
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 class Workspace:
@@ -224,30 +236,37 @@ _ws = {}
 
 def workspace() -> Workspace:
     """The default workspace of the current device (one per device)."""
-    dev = torch.cuda.current_device()
-    if dev not in _ws:
-        _ws[dev] = Workspace()
-    return _ws[dev]
+    dev = _device()
+    ws = _ws.get(dev)
+    if ws is None:
+        ws = _ws[dev] = Workspace()
+    return ws
 
 
 # ---------------------------------------------------------------- BS1-BS5
 
-def _sfx(t):
-    return "_f32" if t.dtype == torch.float32 else ""
+def _f32(t):
+    return t.dtype is torch.float32
 
 
 def copy(x, y=None):
     """BS1: y = x."""
     y = torch.empty_like(x) if y is None else y
-    _check(getattr(lib(), "bs_copy" + _sfx(x))(x.numel(), _ptr(x, x.dtype, "x"),
-                                               _ptr(y, x.dtype, "y"), _stream()), "bs_copy")
+    L, t = lib(), x.dtype
+    rc = (L.bs_copy_f32 if t is torch.float32 else L.bs_copy)(
+        x.numel(), _ptr(x, t, "x"), _ptr(y, t, "y"), _stream())
+    if rc:
+        _check(rc, "bs_copy")
     return y
 
 
 def axpy(alpha, x, beta, y):
     """BS2: y = fma(alpha, x, beta*y), in place on y."""
-    _check(getattr(lib(), "bs_axpy" + _sfx(x))(x.numel(), alpha, _ptr(x, x.dtype, "x"), beta,
-                                               _ptr(y, x.dtype, "y"), _stream()), "bs_axpy")
+    L, t = lib(), x.dtype
+    rc = (L.bs_axpy_f32 if t is torch.float32 else L.bs_axpy)(
+        x.numel(), alpha, _ptr(x, t, "x"), beta, _ptr(y, t, "y"), _stream())
+    if rc:
+        _check(rc, "bs_axpy")
     return y
 
 
@@ -255,8 +274,11 @@ def norm(x, out=None, ws=None):
     """BS3: device tensor [x.x, sqrt(x.x)] (float64)."""
     out = torch.empty(2, dtype=torch.float64, device=x.device) if out is None else out
     ws = ws or workspace()
-    _check(getattr(lib(), "bs_norm" + _sfx(x))(x.numel(), _ptr(x, x.dtype, "x"), _ptr(out),
-                                               ws.handle, _stream()), "bs_norm")
+    L, t = lib(), x.dtype
+    rc = (L.bs_norm_f32 if t is torch.float32 else L.bs_norm)(
+        x.numel(), _ptr(x, t, "x"), _ptr(out), ws.handle, _stream())
+    if rc:
+        _check(rc, "bs_norm")
     return out
 
 
@@ -264,9 +286,11 @@ def dot(x, y, out=None, ws=None):
     """BS4: device tensor [x.y] (float64)."""
     out = torch.empty(1, dtype=torch.float64, device=x.device) if out is None else out
     ws = ws or workspace()
-    _check(getattr(lib(), "bs_dot" + _sfx(x))(x.numel(), _ptr(x, x.dtype, "x"),
-                                              _ptr(y, x.dtype, "y"), _ptr(out), ws.handle,
-                                              _stream()), "bs_dot")
+    L, t = lib(), x.dtype
+    rc = (L.bs_dot_f32 if t is torch.float32 else L.bs_dot)(
+        x.numel(), _ptr(x, t, "x"), _ptr(y, t, "y"), _ptr(out), ws.handle, _stream())
+    if rc:
+        _check(rc, "bs_dot")
     return out
 
 
@@ -274,10 +298,12 @@ def cg_update(alpha, p, Ap, x, r, out=None, ws=None):
     """BS5: x += alpha p; r -= alpha Ap (in place); device tensor [r.r]."""
     out = torch.empty(1, dtype=torch.float64, device=x.device) if out is None else out
     ws = ws or workspace()
-    t = x.dtype
-    _check(getattr(lib(), "bs_cg_update" + _sfx(x))(
+    L, t = lib(), x.dtype
+    rc = (L.bs_cg_update_f32 if t is torch.float32 else L.bs_cg_update)(
         x.numel(), alpha, _ptr(p, t, "p"), _ptr(Ap, t, "Ap"), _ptr(x, t, "x"), _ptr(r, t, "r"),
-        _ptr(out), ws.handle, _stream()), "bs_cg_update")
+        _ptr(out), ws.handle, _stream())
+    if rc:
+        _check(rc, "bs_cg_update")
     return out
 
 
@@ -321,17 +347,17 @@ class Map:
     def scatter(self, qG, qL=None):
         """BS7: qL = Z qG (masked entries of qL untouched)."""
         qL = torch.empty(self.NL, dtype=qG.dtype, device=qG.device) if qL is None else qL
-        _check(getattr(lib(), "bs_scatter" + _sfx(qG))(self.handle, _ptr(qG, qG.dtype, "qG"),
-                                                       _ptr(qL, qG.dtype, "qL"), _stream()),
-               "bs_scatter")
+        L, t = lib(), qG.dtype
+        _check((L.bs_scatter_f32 if _f32(qG) else L.bs_scatter)(
+            self.handle, _ptr(qG, t, "qG"), _ptr(qL, t, "qL"), _stream()), "bs_scatter")
         return qL
 
     def gather(self, qL, qG=None):
         """BS6: qG = Z^T qL."""
         qG = torch.empty(self.NG, dtype=qL.dtype, device=qL.device) if qG is None else qG
-        _check(getattr(lib(), "bs_gather" + _sfx(qL))(self.handle, _ptr(qL, qL.dtype, "qL"),
-                                                      _ptr(qG, qL.dtype, "qG"), _stream()),
-               "bs_gather")
+        L, t = lib(), qL.dtype
+        _check((L.bs_gather_f32 if _f32(qL) else L.bs_gather)(
+            self.handle, _ptr(qL, t, "qL"), _ptr(qG, t, "qG"), _stream()), "bs_gather")
         return qG
 
 
@@ -480,8 +506,8 @@ def _arrays(problems, bs_, xs=None):
     if n == 0 or n != len(bs_) or (xs is not None and n != len(xs)):
         raise ValueError("problems, b and x must be non-empty lists of one length")
     P = (ctypes.c_void_p * n)(*[p.handle.value for p in problems])
-    B = (ctypes.c_void_p * n)(*[_ptr(b, name="b").value for b in bs_])
-    X = None if xs is None else (ctypes.c_void_p * n)(*[_ptr(x, name="x").value for x in xs])
+    B = (ctypes.c_void_p * n)(*[_ptr(b, name="b") for b in bs_])
+    X = None if xs is None else (ctypes.c_void_p * n)(*[_ptr(x, name="x") for x in xs])
     return n, P, B, X
 
 
