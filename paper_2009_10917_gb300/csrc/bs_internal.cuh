@@ -65,6 +65,14 @@ constexpr int kMaxPartials = 4096;  // per-block partials a workspace holds
 // more blocks than there is work.
 int stream_grid(int64_t work, int per_thread, int block, int blocks_per_sm);
 
+// Grid of a reduction over `work` vectors: one block while its threads have
+// at most nine loads each in turn, since combining blocks (a fence, an atomic,
+// the partials read back) costs more than those.
+inline int reduce_grid(int64_t work, int per_thread, int blocks_per_sm) {
+  if (work <= 9 * kReduceBlock) return stream_grid(1, 1, 1, 1);
+  return stream_grid(work, per_thread, kReduceBlock, blocks_per_sm);
+}
+
 // Resident blocks per SM of `kernel` at `block` threads on the current
 // device (queried once per kernel and device, then cached).
 int occupancy_blocks(const void *kernel, int block);
@@ -120,6 +128,10 @@ template <int BLOCK>
 __device__ __forceinline__ bool grid_combine(double partial, double *partials,
                                              unsigned int *counter,
                                              double *total) {
+  if (gridDim.x == 1) {  // nothing to combine: no fence, no counter
+    if (threadIdx.x == 0) *total = partial;
+    return true;
+  }
   __shared__ bool s_last;
   if (threadIdx.x == 0) {
     partials[blockIdx.x] = partial;
