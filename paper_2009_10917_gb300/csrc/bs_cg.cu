@@ -419,7 +419,8 @@ static int scat_iteration(const bs_problem *P, bool precond, bool ff, cudaStream
                                                P->lambda, st, s)
                      : launch_ax_geo<false>(P->N, m->E, m->NL, nullptr, nullptr, L.p, P->d_ApL,
                                             P->d_tab, P->d_coef, P->d_geo, P->lambda, st, s))
-           : ff ? launch_ax_local_ff<false>(P->N, m->E, nullptr, nullptr, L.p, P->d_ApL,
+           : ff && !ff_takes_fx(P->N)
+               ? launch_ax_local_ff<false>(P->N, m->E, nullptr, nullptr, L.p, P->d_ApL,
                                             P->d_tabff, P->d_coef, g, mlam, st, s)
                 : launch_ax_local<double, false>(P->N, m->E, nullptr, nullptr, L.p, P->d_ApL,
                                                  P->d_tab, P->d_coef, g, mlam, st, s);

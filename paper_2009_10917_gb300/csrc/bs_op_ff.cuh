@@ -635,6 +635,12 @@ extern int g_op_fusion;
 // Ap = A p for a global p (FP64 or FP32 tables; ff: the float-float element
 // kernel, FP64 only).  DOT: ep(p . Ap), reduced in the gather's pass (and,
 // fused, in the element kernel's epilogue for the single-copy nodes).
+// Whether a float-float A p runs the FP64 fixed-point kernel (bs_op_fx.cuh): at
+// degrees 6 and 7 it is the faster of the two (10M local nodes, with the gather:
+// 160 against 221 us at N = 6, 125 against 216 at N = 7; N = 5 185 against 187,
+// N = 4 234 against 183) and exact to FP64's rounding.
+inline bool ff_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7); }
+
 template <typename T, bool DOT, class Ep>
 int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p, T *Ap, T *ApL,
                    T g, T mlam, Ep ep, const CgState *st, cudaStream_t s) {
@@ -657,8 +663,9 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
   const int32_t *ids = fused ? m->d_ids_f : m->d_ids;
   double *opp = fused && DOT ? P->d_op_partials : nullptr;
   int rc;
+  const bool ffk = ff && !ff_takes_fx(P->N);
   if constexpr (std::is_same<T, double>::value) {
-    if (ff)
+    if (ffk)
       rc = fused ? launch_ax_local_ff<true, true>(P->N, m->E, m->d_elem_order, ids, p, ApL,
                                                   P->d_tabff, P->d_coef, g, mlam, st, s, Ap, opp)
                  : launch_ax_local_ff<true>(P->N, m->E, m->d_elem_order, ids, p, ApL, P->d_tabff,
@@ -680,7 +687,7 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
     return launch_gather<T, DOT, Ep>(m, ApL, Ap, DOT ? p : nullptr, P->d_partials, P->d_counter,
                                      ep, st, s);
   return launch_gather_rows<T, DOT, Ep>(m, fused, ApL, Ap, DOT ? p : nullptr, P->d_partials,
-                                        P->d_counter, opp, opp ? ax_blocks(P->N, m->E, sizeof(T) == 8 && !ff) : 0, ep,
+                                        P->d_counter, opp, opp ? ax_blocks(P->N, m->E, sizeof(T) == 8 && !ffk) : 0, ep,
                                         st, s);
 }
 
