@@ -250,8 +250,9 @@ int bs_diag_A(const bs_problem *prob, double *d_diag, void *stream);
  * lambda L^3 with the mesh's length scale L, and below 2^-102 they count as
  * zero -- keep L above about 2^-28 (lambda of order 1) for the accuracy
  * stated here.  The gather is the same as bs_apply_A's.  At degrees 6 and 7
- * (affine elements, without BS_OP_DIRECT) the FP64 fixed-point kernel of
- * bs_apply_A is the faster one and runs instead: FP64's accuracy and range. */
+ * (5..7 with geometric factors; without BS_OP_DIRECT) the FP64 fixed-point
+ * kernel of bs_apply_A is the faster one and runs instead: FP64's accuracy and
+ * range. */
 int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *stream);
 
 /* How A p is formed, process-wide, by bs_apply_A, bs_apply_local,
@@ -279,7 +280,8 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   finite, lie outside [2^-900, 2^900] or differ too much in size takes
  *   the direct FP64 sums); results differ by rounding only.
  * Problems with geometric factors (bs_problem_create_geo) always use their
- * own unfused FP64 kernel.  Returns the previous mode; a negative value only
+ * own unfused kernels (FP64 and float-float; at degrees 5..7, without
+ * BS_OP_DIRECT, the FP64 one in the fixed-point form as well).  Returns the previous mode; a negative value only
  * queries it.  Not thread-safe against solves in flight. */
 enum { BS_OP_FUSED = 1, BS_OP_DIRECT = 2 };
 int bs_operator_mode(int32_t mode);

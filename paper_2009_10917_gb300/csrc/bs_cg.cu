@@ -414,7 +414,8 @@ static int scat_iteration(const bs_problem *P, bool precond, bool ff, cudaStream
   CgState *st = P->d_state;
   const double g = 0.5 * P->h, mlam = P->lambda * g * g * g;
   int rc = P->d_geo
-               ? (ff ? launch_ax_geo_ff<false>(P->N, m->E, m->NL, nullptr, nullptr, L.p,
+               ? (ff && !ff_geo_takes_fx(P->N)
+                      ? launch_ax_geo_ff<false>(P->N, m->E, m->NL, nullptr, nullptr, L.p,
                                                P->d_ApL, P->d_tabff, P->d_coef, P->d_geo,
                                                P->lambda, st, s)
                      : launch_ax_geo<false>(P->N, m->E, m->NL, nullptr, nullptr, L.p, P->d_ApL,

@@ -115,14 +115,70 @@ static DD operator/(DD a, DD b) {
   return dd_fast(q, (r.h + r.l) / b.h);
 }
 
-// The digits of Kh = W^-1 K (bs_op_fx.cuh), from GLL nodes, weights and
-// derivative matrix redone in double-double (Newton on the nodes x, as
-// gll_tables): a 58-bit entry holds more than a double, and an error common to
-// every element would shift the operator's low modes coherently.  Each entry
-// becomes an integer of at most 58 bits, the diagonal minus the rest of its
-// row (the rows sum to zero, as K's do), then signed 10-bit digits by the bias of 512
-// per digit that the kernel uses for its values, as the bits of a half.
-static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t) {
+// A matrix's digit words (bs_op_fx.cuh): each entry an integer of at most 58
+// bits, the diagonal minus the rest of its row where the rows sum to zero,
+// then signed 10-bit digits by the bias of 512 per digit that the kernels use
+// for their values, as the bits of a half.  False when a sum of products
+// could leave its accumulator (it cannot, for the matrices of degrees 4..7).
+template <class M>
+static bool fx_digits(int Nq, M mat, bool zero_rows, uint32_t (*w)[32], int *q) {
+  double big = 0.0;
+  for (int i = 0; i < Nq; ++i)
+    for (int m = 0; m < Nq; ++m) big = std::fmax(big, std::fabs(mat(i, m).h));
+  int e = 0;
+  std::frexp(big, &e);  // big < 2^e
+  *q = 58 - e;
+  int64_t Ki[kMaxNq][kMaxNq];
+  for (int i = 0; i < Nq; ++i) {
+    int64_t rest = 0;
+    for (int m = 0; m < Nq; ++m) {
+      const DD v = mat(i, m);
+      const double hi = std::ldexp(v.h, *q), n = std::rint(hi);
+      Ki[i][m] = (int64_t)n + (int64_t)std::rint((hi - n) + std::ldexp(v.l, *q));
+      if (m != i) rest += Ki[i][m];
+    }
+    if (zero_rows) Ki[i][i] = -rest;
+  }
+  int64_t bias = 0;
+  for (int d = 0; d < kFxDigits; ++d) bias += (int64_t)512 << (10 * d);
+  auto digit = [&](int i, int m, int d) {
+    return (int)(((bias + Ki[i][m]) >> (10 * (kFxDigits - 1 - d))) & 0x3ff) - 512;
+  };
+  // the largest sum an accumulator can meet: digits of a value up to 257
+  // (the first) or 512 in magnitude, products a + b = o of one row
+  for (int o = 0; o < kFxDigits; ++o)
+    for (int i = 0; i < Nq; ++i) {
+      int64_t s = 0;
+      for (int a = 0; a <= o; ++a)
+        for (int m = 0; m < Nq; ++m) s += (a ? 512 : 257) * std::abs(digit(i, m, o - a));
+      if (s > (o == kFxDigits - 1 ? 1 << 23 : 1 << 22)) return false;
+    }
+  auto half_bits = [](int v) -> uint32_t {  // |v| <= 512
+    if (v == 0) return 0;
+    const uint32_t sign = v < 0 ? 0x8000u : 0u, a = (uint32_t)(v < 0 ? -v : v);
+    int p = 31;
+    while (!(a >> p)) --p;
+    return sign | ((uint32_t)(p + 15) << 10) | ((a << (10 - p)) & 0x3ffu);
+  };
+  for (int d = 0; d < kFxDigits; ++d)
+    for (int lane = 0; lane < 32; ++lane) {
+      uint32_t word = 0;
+      for (int hf = 0; hf < 2; ++hf) {
+        const int i = lane >> 2, m = 2 * (lane & 3) + hf;
+        if (i < Nq && m < Nq) word |= half_bits(digit(i, m, d)) << (16 * hf);
+      }
+      w[d][lane] = word;
+    }
+  return true;
+}
+
+// The digits of Kh = W^-1 K, D and D^T (bs_op_fx.cuh, bs_op_geo_fx.cuh), from GLL
+// nodes, weights and derivative matrix redone in double-double (Newton on the
+// nodes x, as gll_tables): a 58-bit entry holds more than a double, and an
+// error common to every element would shift the operator's low modes
+// coherently.  Also the weights' products of the affine kernel.
+static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t,
+                     FxGeoTab *tg) {
   const int Nq = N + 1;
   DD x[kMaxNq], w[kMaxNq], D[kMaxNq][kMaxNq], Kh[kMaxNq][kMaxNq];
   auto legendre = [&](DD z, DD *pn, DD *pm) {  // P_N, P_{N-1}
@@ -161,57 +217,16 @@ static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t)
       }
     D[a][a] = diag;
   }
-  double big = 0.0;
   for (int i = 0; i < Nq; ++i)
     for (int m = 0; m < Nq; ++m) {
       DD s;
       for (int a = 0; a < Nq; ++a) s = s + D[a][i] * w[a] * D[a][m];
       Kh[i][m] = s / w[i];
-      big = std::fmax(big, std::fabs(Kh[i][m].h));
     }
-  int e = 0;
-  std::frexp(big, &e);  // big < 2^e
-  t->q = 58 - e;
-  int64_t Ki[kMaxNq][kMaxNq];
-  for (int i = 0; i < Nq; ++i) {
-    int64_t rest = 0;
-    for (int m = 0; m < Nq; ++m) {
-      const double hi = std::ldexp(Kh[i][m].h, t->q), n = std::rint(hi);
-      Ki[i][m] = (int64_t)n + (int64_t)std::rint((hi - n) + std::ldexp(Kh[i][m].l, t->q));
-      if (m != i) rest += Ki[i][m];
-    }
-    Ki[i][i] = -rest;
-  }
-  int64_t bias = 0;
-  for (int d = 0; d < kFxDigits; ++d) bias += (int64_t)512 << (10 * d);
-  auto digit = [&](int i, int m, int d) {
-    return (int)(((bias + Ki[i][m]) >> (10 * (kFxDigits - 1 - d))) & 0x3ff) - 512;
-  };
-  // the largest sum an accumulator can meet: digits of a value up to 257
-  // (the first) or 512 in magnitude, products a + b = o of one row
-  for (int o = 0; o < kFxDigits; ++o)
-    for (int i = 0; i < Nq; ++i) {
-      int64_t s = 0;
-      for (int a = 0; a <= o; ++a)
-        for (int m = 0; m < Nq; ++m) s += (a ? 512 : 257) * std::abs(digit(i, m, o - a));
-      if (s > (o == kFxDigits - 1 ? 1 << 23 : 1 << 22)) return false;
-    }
-  auto half_bits = [](int v) -> uint32_t {  // |v| <= 512
-    if (v == 0) return 0;
-    const uint32_t sign = v < 0 ? 0x8000u : 0u, a = (uint32_t)(v < 0 ? -v : v);
-    int p = 31;
-    while (!(a >> p)) --p;
-    return sign | ((uint32_t)(p + 15) << 10) | ((a << (10 - p)) & 0x3ffu);
-  };
-  for (int d = 0; d < kFxDigits; ++d)
-    for (int lane = 0; lane < 32; ++lane) {
-      uint32_t word = 0;
-      for (int hf = 0; hf < 2; ++hf) {
-        const int i = lane >> 2, m = 2 * (lane & 3) + hf;
-        if (i < Nq && m < Nq) word |= half_bits(digit(i, m, d)) << (16 * hf);
-      }
-      t->w[d][lane] = word;
-    }
+  if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, t->w, &t->q) ||
+      !fx_digits(Nq, [&](int i, int m) { return D[i][m]; }, true, tg->d, &tg->qd) ||
+      !fx_digits(Nq, [&](int i, int m) { return D[m][i]; }, false, tg->dt, &tg->qdt))
+    return false;
   const DD g(0.5 * h), ml = DD(lambda) * g * g * g;
   for (int k = 0; k < Nq; ++k)
     for (int lane = 0; lane < 32; ++lane)
@@ -363,7 +378,7 @@ int bs_problem_create(const bs_map *map, double h, double lambda, const double *
         split(o, tabff.Eoh[a * hq + m], tabff.Eol[a * hq + m]);
       }
   }
-  if (Nq >= kFxMinNq && Nq <= kFxMaxNq && !fx_table(N, x, h, lambda, &tab.fx)) {
+  if (Nq >= kFxMinNq && Nq <= kFxMaxNq && !fx_table(N, x, h, lambda, &tab.fx, &tab.fxg)) {
     free(p);
     return fail(BS_ERR_ARG, "bs_problem_create: digit tables of degree %d out of range", N);
   }

@@ -48,6 +48,11 @@ struct __align__(16) FxTab {
   double wg[kFxMaxNq * 64], wm[kFxMaxNq * 64];
   int q;
 };
+// The same digits of the derivative matrix D (d, scale qd) and of D^T (dt, qdt).
+struct FxGeoTab {
+  uint32_t d[kFxDigits][32], dt[kFxDigits][32];
+  int qd, qdt;
+};
 
 // Per-problem constant tables, in device memory.
 template <typename T>
@@ -60,6 +65,7 @@ struct OpTab {
   T Ee[(kMaxNq / 2) * (kMaxNq / 2)];
   T Eo[(kMaxNq / 2) * (kMaxNq / 2)];
   FxTab fx;        // FP64 tables only
+  FxGeoTab fxg;
   int64_t ne, ng;  // the problem's E and N_G (index checks of the checked build)
 };
 

@@ -640,6 +640,9 @@ extern int g_op_fusion;
 // 160 against 221 us at N = 6, 125 against 216 at N = 7; N = 5 185 against 187,
 // N = 4 234 against 183) and exact to FP64's rounding.
 inline bool ff_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7); }
+// The same on general hexahedra, degrees 5..7: 559 against 608 us, 438 against
+// 753, 324 against 770.
+inline bool ff_geo_takes_fx(int N) { return g_op_evenodd && N >= 5 && N <= 7; }
 
 template <typename T, bool DOT, class Ep>
 int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p, T *Ap, T *ApL,
@@ -647,7 +650,8 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
   const bs_map *m = P->map;
   if (P->d_geo) {  // general hexahedra: FP64 or float-float, unfused
     if constexpr (std::is_same<T, double>::value) {
-      if (int rc = ff ? launch_ax_geo_ff<true>(P->N, m->E, m->NL, m->d_elem_order, m->d_ids, p,
+      if (int rc = ff && !ff_geo_takes_fx(P->N)
+                      ? launch_ax_geo_ff<true>(P->N, m->E, m->NL, m->d_elem_order, m->d_ids, p,
                                                ApL, P->d_tabff, P->d_coef, P->d_geo, P->lambda,
                                                st, s)
                       : launch_ax_geo<true>(P->N, m->E, m->NL, m->d_elem_order, m->d_ids, p, ApL,

@@ -190,6 +190,142 @@ __device__ __forceinline__ double fx_double(int64_t v, int p) {
   return __longlong_as_double((int64_t)(b | ((uint64_t)v & 0x8000000000000000ull)));
 }
 
+// The matrix's digit words of a lane and the sums' start values, and the three
+// contractions of digit planes (dig_s: shared address; plane a, layer k, row
+// g ^ k, word t) with it.  The sums still hold their start values' bits.
+template <int NQ>
+struct FxMul {
+  static constexpr int D = kFxDigits, PLANE = FxShape<NQ>::PLANE;
+  uint32_t kw[D];
+  FxStart start1, start2, start12;
+  int mrow, mmat;  // ldmatrix: row, matrix of this lane
+  __device__ __forceinline__ FxMul(const uint32_t (*w)[32], int lane)
+      : start1(kFxMagicBits, kFxMagicBits),
+        start2(kFxMagic2Bits, kFxMagic2Bits),
+        start12(kFxMagicBits, kFxMagic2Bits),
+        mrow(lane & 7),
+        mmat(lane >> 3) {
+    set(w, lane);
+  }
+  __device__ __forceinline__ void set(const uint32_t (*w)[32], int lane) {
+#pragma unroll
+    for (int b = 0; b < D; ++b) kw[b] = __ldg(&w[b][lane]);
+  }
+  __device__ __forceinline__ uint32_t kd(int b) const { return b >= 0 ? kw[b < D ? b : 0] : 0u; }
+  // A = the matrix for the orders o (rows 0-7) and o + 1 (rows 8-15) against
+  // digits a, a + 1, B = f; nodes (2t, row g), (2t + 1, row g)
+  __device__ __forceinline__ void rows(const uint32_t *f, uint32_t *s0, uint32_t *s1) const {
+#pragma unroll
+    for (int o = 0; o < D; o += 2) {
+      float c[4];
+      fx_mma0(c, kd(o), kd(o + 1), kd(o - 1), kd(o), f[0], f[1], o + 2 == D ? start12 : start1);
+#pragma unroll
+      for (int a = 2; a <= o; a += 2)
+        fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
+      s0[o] = __float_as_uint(c[0]);
+      s1[o] = __float_as_uint(c[1]);
+      s0[o + 1] = __float_as_uint(c[2]);
+      s1[o + 1] = __float_as_uint(c[3]);
+    }
+  }
+  // along t, plane j: rows k of the digit planes, transposed (rows past Nq
+  // repeat the last one; the matrix's digits are zero there).  Nodes k = g.
+  __device__ __forceinline__ void along_t(uint32_t dig_s, int j, uint32_t *s0,
+                                          uint32_t *s1) const {
+    const int krow = mrow < NQ ? mrow : NQ - 1;
+    uint32_t f[D];
+    const uint32_t row = dig_s + (krow * 8 + (j ^ krow)) * 16;
+    fx_ldsm4t(f, row + mmat * PLANE);
+    fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * PLANE);
+    rows(f, s0, s1);
+  }
+  // along s, layer k: the transposed layer.  Nodes j = g.
+  __device__ __forceinline__ void along_s(uint32_t dig_s, int k, uint32_t *s0,
+                                          uint32_t *s1) const {
+    uint32_t f[D];
+    const uint32_t row = dig_s + (k * 8 + (mrow ^ k)) * 16;
+    fx_ldsm4t(f, row + mmat * PLANE);
+    fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * PLANE);
+    rows(f, s0, s1);
+  }
+  // along r, layers l0 and l1: A = digits a, a + 1 of l0 (rows 0-7) and l1, B =
+  // the matrix transposed.  s: (l0, 2t), (l0, 2t + 1), (l1, 2t), (l1, 2t + 1).
+  __device__ __forceinline__ void along_r(uint32_t dig_s, int l0, int l1,
+                                          uint32_t (*s)[D]) const {
+    uint32_t f[D / 2][4];
+    const int kk = (mmat & 1) ? l1 : l0;
+#pragma unroll
+    for (int a = 0; a < D; a += 2)
+      fx_ldsm4(f[a / 2], dig_s + (a + (mmat >> 1)) * PLANE + (kk * 8 + (mrow ^ kk)) * 16);
+#pragma unroll
+    for (int o = 0; o < D; ++o) {
+      float c[4];
+      fx_mma0(c, f[0][0], f[0][1], f[0][2], f[0][3], kd(o), kd(o - 1),
+              o + 1 == D ? start2 : start1);
+#pragma unroll
+      for (int a = 2; a <= o; a += 2)
+        fx_mma(c, f[a / 2][0], f[a / 2][1], f[a / 2][2], f[a / 2][3], kd(o - a), kd(o - a - 1));
+#pragma unroll
+      for (int n = 0; n < 4; ++n) s[n][o] = __float_as_uint(c[n]);
+    }
+  }
+};
+
+// The digits of a lane's values of layer k into the planes.
+template <int NQ>
+__device__ __forceinline__ void fx_store_digits(unsigned char *dig, int k, int g, int t, double a,
+                                                double b, int emax) {
+  const uint64_t x = fx_fixed(a, emax), y = fx_fixed(b, emax);
+  uint32_t *p = reinterpret_cast<uint32_t *>(dig) + (k * 8 + (g ^ k)) * 4 + t;
+  constexpr int PW = FxShape<NQ>::PLANE / 4;
+  p[0 * PW] = fx_digit2<0>(x, y);
+  p[1 * PW] = fx_digit2<1>(x, y);
+  p[2 * PW] = fx_digit2<2>(x, y);
+  p[3 * PW] = fx_digit2<3>(x, y);
+  p[4 * PW] = fx_digit2<4>(x, y);
+  p[5 * PW] = fx_digit2<5>(x, y);
+}
+
+// Exchange of the sums along t between the layout they arrive in (plane j,
+// node k = g) and the owner's (j = g, layer k): 64-byte rows (j, k), in an
+// order that lets writes (fixed j, all k) and reads (fixed k, all j) miss no
+// bank.
+template <int NQ>
+__device__ __forceinline__ ulonglong2 *fx_xch(unsigned char *xch, int j, int k, int t) {
+  const int kk = NQ == 8 ? (k ^ j) : k;
+  return reinterpret_cast<ulonglong2 *>(xch + (j * NQ + kk) * 64 + t * 16);
+}
+
+// High word of |x|, or 1 for a value whose high word is zero but which is not.
+__device__ __forceinline__ uint32_t fx_size(double x) {
+  return ((uint32_t)__double2hiint(x) & 0x7fffffffu) | min((uint32_t)__double2loint(x), 1u);
+}
+
+// From the largest values of a lane's two columns over its warp's layers: the
+// element's largest exponent, and whether its values are beyond the digits
+// (col: 256 bytes per warp; two barriers' worth of a gap between uses).
+template <int WPE, class Sync>
+__device__ __forceinline__ int fx_range(uint32_t big0, uint32_t big1, uint32_t *col, int warp,
+                                        int lane, Sync sync, bool *direct) {
+  if (WPE > 1) {
+    reinterpret_cast<uint2 *>(col)[warp * 32 + lane] = make_uint2(big0, big1);
+    sync();
+#pragma unroll
+    for (int w = 0; w < WPE; ++w) {
+      const uint2 c = reinterpret_cast<const uint2 *>(col)[w * 32 + lane];
+      big0 = max(big0, c.x);
+      big1 = max(big1, c.y);
+    }
+  }
+  const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0, big1));
+  const uint32_t low = __reduce_min_sync(  // columns of zeros left out
+      0xffffffffu, min(big0 ? big0 : 0x7fffffffu, big1 ? big1 : 0x7fffffffu));
+  const int emax = big ? (int)(big >> 20) : 1023;  // an element of zeros has zero digits
+  *direct = emax < 123 || emax > 1923 ||           // outside [2^-900, 2^900]
+            (big && emax - (int)(low >> 20) > kFxRange);
+  return emax;
+}
+
 // Direct FP64 sums of one element (values in x[], node order as in memory)
 // for the node (i, j, k): (W^-1 D^T W D applied along r, s and t).
 template <int NQ>
@@ -278,33 +414,15 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
       }
     }
   }
-  // ---- the columns' largest values (high words; 1 for a value whose high
-  // word is zero but which is not), the largest exponent, and whether the
-  // digits serve
+  // ---- the largest exponent, and whether the digits serve
   uint32_t big0 = 0, big1 = 0;
 #pragma unroll
   for (int l = 0; l < L; ++l) {
-    big0 = max(big0, ((uint32_t)__double2hiint(u0[l]) & 0x7fffffffu) |
-                         min((uint32_t)__double2loint(u0[l]), 1u));
-    big1 = max(big1, ((uint32_t)__double2hiint(u1[l]) & 0x7fffffffu) |
-                         min((uint32_t)__double2loint(u1[l]), 1u));
+    big0 = max(big0, fx_size(u0[l]));
+    big1 = max(big1, fx_size(u1[l]));
   }
-  if (WPE > 1) {
-    reinterpret_cast<uint2 *>(col)[k0 / L * 32 + lane] = make_uint2(big0, big1);
-    sync();
-#pragma unroll
-    for (int w = 0; w < WPE; ++w) {
-      const uint2 c = reinterpret_cast<const uint2 *>(col)[w * 32 + lane];
-      big0 = max(big0, c.x);
-      big1 = max(big1, c.y);
-    }
-  }
-  const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0, big1));
-  const uint32_t low = __reduce_min_sync(  // columns of zeros left out
-      0xffffffffu, min(big0 ? big0 : 0x7fffffffu, big1 ? big1 : 0x7fffffffu));
-  const int emax = big ? (int)(big >> 20) : 1023;  // an element of zeros has zero digits
-  const bool direct = emax < 123 || emax > 1923 ||  // outside [2^-900, 2^900]
-                      (big && emax - (int)(low >> 20) > kFxRange);
+  bool direct;
+  const int emax = fx_range<WPE>(big0, big1, col, k0 / L, lane, sync, &direct);
   const double ce = coef ? coef[e] : 1.0;
   auto store = [&](int l, double r0, double r1, int32_t i0, int32_t i1, double v0, double v1) {
     if (FUSED) {
@@ -327,113 +445,39 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
     }
   };
   if (!direct) {
-    // ---- digits into shared memory: word (a, k, g ^ k, t)
 #pragma unroll
     for (int l = 0; l < L; ++l) {
       if (!layer(l)) break;
-      const int k = k0 + l;
-      const uint64_t x = fx_fixed(u0[l], emax), y = fx_fixed(u1[l], emax);
-      uint32_t *p = reinterpret_cast<uint32_t *>(dig) + (k * 8 + (g ^ k)) * 4 + t;
-      constexpr int PW = S::PLANE / 4;
-      p[0 * PW] = fx_digit2<0>(x, y);
-      p[1 * PW] = fx_digit2<1>(x, y);
-      p[2 * PW] = fx_digit2<2>(x, y);
-      p[3 * PW] = fx_digit2<3>(x, y);
-      p[4 * PW] = fx_digit2<4>(x, y);
-      p[5 * PW] = fx_digit2<5>(x, y);
+      fx_store_digits<NQ>(dig, k0 + l, g, t, u0[l], u1[l], emax);
     }
-    const FxStart start1(kFxMagicBits, kFxMagicBits), start2(kFxMagic2Bits, kFxMagic2Bits),
-        start12(kFxMagicBits, kFxMagic2Bits);
-    uint32_t kw[D];
-#pragma unroll
-    for (int b = 0; b < D; ++b) kw[b] = __ldg(&tab->fx.w[b][lane]);
+    const FxMul<NQ> mul(tab->fx.w, lane);
     sync();
-    // A fragments of Kh for the orders o (rows 0-7) and o + 1 (rows 8-15)
-    // against digits a, a + 1: digits o - a, o + 1 - a, o - a - 1, o - a
-    auto kd = [&](int b) { return b >= 0 ? kw[b < D ? b : 0] : 0u; };
-    const int mrow = lane & 7, mmat = lane >> 3;  // ldmatrix: row, matrix of this lane
-    // ---- along t, planes j = k0 + l: rows k of the digit planes, transposed
-    // (rows past Nq repeat the last one; their Kh digits are zero)
-    const int krow = mrow < NQ ? mrow : NQ - 1;
+    // ---- along t, planes j = k0 + l (the start values come off along r and s)
 #pragma unroll
     for (int l = 0; l < L; ++l) {
       if (!layer(l)) break;
-      const int j = k0 + l;
-      uint32_t f[D];
-      const uint32_t row = dig_s + (krow * 8 + (j ^ krow)) * 16;
-      fx_ldsm4t(f, row + mmat * S::PLANE);
-      fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * S::PLANE);
-      uint32_t s0[D], s1[D];  // with the start values' bits: removed along r and s
-#pragma unroll
-      for (int o = 0; o < D; o += 2) {
-        float c[4];
-        fx_mma0(c, kd(o), kd(o + 1), kd(o - 1), kd(o), f[0], f[1],
-                o + 2 == D ? start12 : start1);
-#pragma unroll
-        for (int a = 2; a <= o; a += 2)
-          fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
-        s0[o] = __float_as_uint(c[0]);
-        s1[o] = __float_as_uint(c[1]);
-        s0[o + 1] = __float_as_uint(c[2]);
-        s1[o + 1] = __float_as_uint(c[3]);
-      }
-      // the lane holds nodes (2t, j, k = g), (2t + 1, j, g)
-      if (NQ == 8 || g < NQ) {
-        // 64-byte rows (j, k), in an order that lets the owner's reads
-        // (fixed k, all j) and these writes (fixed j, all k) miss no bank
-        const int kk = NQ == 8 ? (g ^ j) : g;
-        *reinterpret_cast<ulonglong2 *>(xch + (j * NQ + kk) * 64 + t * 16) =
-            make_ulonglong2(fx_join(s0), fx_join(s1));
-      }
+      uint32_t s0[D], s1[D];
+      mul.along_t(dig_s, k0 + l, s0, s1);
+      if (NQ == 8 || g < NQ)
+        *fx_xch<NQ>(xch, k0 + l, g, t) = make_ulonglong2(fx_join(s0), fx_join(s1));
     }
     // ---- along r and s, two layers at a time
     uint64_t T0[L], T1[L];
 #pragma unroll
     for (int l = 0; l < L; l += 2) {
       if (!layer(l)) break;
-      const int ka = k0 + l, kb = ka + 1 < NQ ? ka + 1 : ka;  // odd Nq: the last layer twice
-      uint32_t s[4][D];  // (ka, 2t), (ka, 2t + 1), (kb, 2t), (kb, 2t + 1)
-      // r: A = digits a, a + 1 of layers ka (rows 0-7) and kb, B = Kh^T
-      uint32_t fr[D / 2][4];  // (a, ka), (a, kb), (a + 1, ka), (a + 1, kb)
-      const int kk = (mmat & 1) ? kb : ka;
-#pragma unroll
-      for (int a = 0; a < D; a += 2)
-        fx_ldsm4(fr[a / 2], dig_s + (a + (mmat >> 1)) * S::PLANE + (kk * 8 + (mrow ^ kk)) * 16);
-#pragma unroll
-      for (int o = 0; o < D; ++o) {
-        float c[4];
-        fx_mma0(c, fr[0][0], fr[0][1], fr[0][2], fr[0][3], kd(o), kd(o - 1),
-                o + 1 == D ? start2 : start1);
-#pragma unroll
-        for (int a = 2; a <= o; a += 2)
-          fx_mma(c, fr[a / 2][0], fr[a / 2][1], fr[a / 2][2], fr[a / 2][3], kd(o - a),
-                 kd(o - a - 1));
-#pragma unroll
-        for (int n = 0; n < 4; ++n) s[n][o] = __float_as_uint(c[n]);
-      }
-      // s: A = Kh, B = the transposed layer; the start values of all three
-      // directions come off here
+      const int l0 = k0 + l, l1 = l0 + 1 < NQ ? l0 + 1 : l0;  // odd Nq: the last layer twice
+      uint32_t s[4][D];
+      mul.along_r(dig_s, l0, l1, s);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int k = h ? kb : ka;
-        uint32_t f[D];
-        const uint32_t row = dig_s + (k * 8 + (mrow ^ k)) * 16;
-        fx_ldsm4t(f, row + mmat * S::PLANE);
-        fx_ldsm2t(f + 4, row + (4 + (mmat & 1)) * S::PLANE);
+        uint32_t s0[D], s1[D];
+        mul.along_s(dig_s, h ? l1 : l0, s0, s1);
 #pragma unroll
-        for (int o = 0; o < D; o += 2) {
-          float c[4];
-          fx_mma0(c, kd(o), kd(o + 1), kd(o - 1), kd(o), f[0], f[1],
-                  o + 2 == D ? start12 : start1);
-#pragma unroll
-          for (int a = 2; a <= o; a += 2)
-            fx_mma(c, kd(o - a), kd(o + 1 - a), kd(o - a - 1), kd(o - a), f[a], f[a + 1]);
-          const uint32_t off = 3u * kFxMagicBits;
-          const uint32_t off1 = 3u * (o + 1 == D - 1 ? kFxMagic2Bits : kFxMagicBits);
-          s[2 * h][o] += __float_as_uint(c[0]) - off;
-          s[2 * h + 1][o] += __float_as_uint(c[1]) - off;
-          s[2 * h][o + 1] += __float_as_uint(c[2]) - off1;
-          s[2 * h + 1][o + 1] += __float_as_uint(c[3]) - off1;
+        for (int o = 0; o < D; ++o) {
+          const uint32_t off = 3u * (o == D - 1 ? kFxMagic2Bits : kFxMagicBits);
+          s[2 * h][o] += s0[o] - off;
+          s[2 * h + 1][o] += s1[o] - off;
         }
         T0[l + h] = fx_join(s[2 * h]);
         T1[l + h] = fx_join(s[2 * h + 1]);
@@ -451,10 +495,7 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
         if (!layer(l)) break;
         const int k = k0 + l;
         ulonglong2 v = make_ulonglong2(0, 0);
-        if (NQ == 8 || g < NQ) {
-          const int kk = NQ == 8 ? (k ^ g) : k;
-          v = *reinterpret_cast<const ulonglong2 *>(xch + (g * NQ + kk) * 64 + t * 16);
-        }
+        if (NQ == 8 || g < NQ) v = *fx_xch<NQ>(xch, g, k, t);
         double d0 = fx_double((int64_t)(T0[l] + v.x), p2);
         double d1 = fx_double((int64_t)(T1[l] + v.y), p2);
         const double2 wg = __ldg(reinterpret_cast<const double2 *>(tab->fx.wg) + k * 32 + lane);

@@ -110,6 +110,12 @@ __global__ void __launch_bounds__(GeoShape<NQ>::THREADS)
   }
 }
 
+}  // namespace bs
+
+#include "bs_op_geo_fx.cuh"
+
+namespace bs {
+
 template <bool GATHER_IN>
 int launch_ax_geo(int N, int64_t E, int64_t NL, const int32_t *order, const int32_t *ids,
                   const double *in, double *out, const OpTab<double> *tab, const double *coef,
@@ -117,6 +123,14 @@ int launch_ax_geo(int N, int64_t E, int64_t NL, const int32_t *order, const int3
   if (E == 0) return BS_OK;
 #define BS_AXG_CASE(NQ)                                                                  \
   case NQ: {                                                                             \
+    if constexpr (use_fx_geo<NQ>()) {                                                        \
+      if (g_op_evenodd) {                                                                \
+        using Sf = FxGeoShape<NQ>;                                                       \
+        k_ax_geo_fx<NQ, GATHER_IN><<<(unsigned)E, Sf::THREADS, Sf::SMEM, s>>>(           \
+            E, NL, order, ids, in, out, tab, coef, geo, lambda, st);                     \
+        break;                                                                           \
+      }                                                                                  \
+    }                                                                                    \
     using Sh = GeoShape<NQ>;                                                             \
     const int64_t grid = (E + Sh::EPB - 1) / Sh::EPB;                                    \
     k_ax_geo<NQ, GATHER_IN><<<(unsigned)grid, Sh::THREADS, 0, s>>>(                      \

@@ -92,3 +92,48 @@ def test_not_finite_values_stay_in_their_lines(mode, N):
     assert np.array_equal(np.isfinite(got), np.isfinite(want))
     assert np.array_equal(np.isnan(got), np.isnan(want))
     assert np.array_equal(got[np.isinf(got)], want[np.isinf(want)])
+
+
+@pytest.mark.parametrize("N", [5, 6, 7])
+@pytest.mark.parametrize("kind", ["uniform", "ones", "graded", "extremes"])
+@pytest.mark.parametrize("with_coef", [False, True])
+def test_general_hexahedra_entrywise(mode, N, kind, with_coef):
+    """The same against the direct FP64 kernel on perturbed hexahedra.  Each
+    gradient and flux component is a line sum within (Nq + 2) 2^-53 of the sum
+    of its terms' sizes and is carried on through at most Nq + 3 more terms, so
+    an entry is off by at most (2 Nq + 8) 2^-53 of B, the sum of |D|^T |G| |D|
+    |u| and the mass term over the element -- here with the lines' terms
+    replaced by the element's largest gradient and flux, as the digits are
+    relative to those -- for either kernel; a factor two of margin."""
+    m = synth.Mesh(2, N, seed=N, perturb=0.2)
+    lam = 0.4
+    coef = synth.lognormal(m.E, 2) if with_coef else np.ones(m.E)
+    P = bs.Problem(bs.Map(m.E, N, m.NG, m.ids), m.h, lam, coef if with_coef else None,
+                   verts=m.verts())
+    u = values(kind, m)
+    _, w, D = fem_ref.gll_np(N)
+    rows, cols = np.abs(D).sum(1).max(), np.abs(D).sum(0).max()
+    # |G| <= w_max (edge)^2 / det-scale: bounded through the affine size, the
+    # perturbation (0.2) at most quadruples it
+    big = np.abs(u).reshape(m.E, -1).max(1)
+    B = coef * 3 * cols * 4 * 3 * m.h * w.max() ** 3 * rows * big + lam * m.h ** 3 * big
+    got = P.apply_local(cuda(u)).cpu().numpy().reshape(m.E, -1)
+    odd = torch.zeros(m.NL + 1, dtype=torch.float64, device="cuda")
+    odd[1:] = cuda(u)
+    assert np.array_equal(P.apply_local(odd[1:]).cpu().numpy(), got.reshape(-1))
+    mode(bs.BS_OP_DIRECT)
+    want = P.apply_local(cuda(u)).cpu().numpy().reshape(m.E, -1)
+    bound = 4 * (2 * (N + 1) + 8) * 2.0 ** -53 * B
+    assert np.all(np.abs(got - want) <= bound[:, None] + 2.0 ** -1070)
+
+
+def test_general_hexahedra_not_finite(mode):
+    m = synth.Mesh(2, 7, seed=1, perturb=0.2)
+    P = bs.Problem(bs.Map(m.E, 7, m.NG, m.ids), m.h, 1.0, verts=m.verts())
+    u = synth.uniform(m.NL, 3)
+    u[m.Np // 2] = np.inf
+    u[3 * m.Np + 1] = np.nan
+    got = P.apply_local(cuda(u)).cpu().numpy()
+    mode(bs.BS_OP_DIRECT)
+    want = P.apply_local(cuda(u)).cpu().numpy()
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
