@@ -8,9 +8,12 @@
 //   B  gather with the p.Ap partial         items = (solve, gather tile)
 //      -> the last tile of a solve to finish sums that solve's partials in
 //         item order and forms alpha (deterministic, no float atomics)
-//   C  fused update x += a p, r -= a Ap     items = (solve, 4096-entry chunk)
-//      with the r.r partial; the last chunk forms beta and the stop flag
-//   D  p = r + beta p                       items = (solve, chunk)
+//   C  r -= a Ap with the r.r partial       items = (solve, 4096-entry chunk)
+//      the last chunk forms beta and the stop flag
+//   D  x += a p, p = r + beta p             items = (solve, chunk)
+// (x waits for D as in bs_cgvec.cuh: 64 bytes a node instead of 72, and the
+// phase that every solve's next scalar waits for moves 24 of them; phase A
+// takes back the flags that D goes by.)
 // The host reads one flag per solve at every convergence check and, once a
 // quarter of the listed solves have stopped, rebuilds the work lists from the
 // solves still running (and re-captures the graph), so finished solves stop
@@ -332,6 +335,7 @@ __device__ void finish_iteration(const BLists &L, int s, CgState *st, double rr_
     done = 1;
   else if (j + 1 >= st->maxit)
     done = 3;
+  st->xdue = 1;
   if (done) stop_solve(L, s, st, done);
 }
 
@@ -368,7 +372,9 @@ __global__ void __launch_bounds__(kBBlock, FF ? 3 : (sizeof(T) == 8 ? 2 : 4))
   extern __shared__ __align__(16) unsigned char bi_smem[];
   T *smem = reinterpret_cast<T *>(bi_smem);
   if (*(volatile int *)L.err) return;
-  // A: ApL = A_L (Z p)
+  // A: ApL = A_L (Z p); the x flags of the last iteration are taken back
+  if (blockIdx.x == gridDim.x - 1)
+    for (int s = threadIdx.x; s < L.ns; s += kBBlock) L.d[s].st->xdue = 0;
   for (int it = blockIdx.x; it < L.nA; it += gridDim.x) {
     const int2 w = L.iA[it];
     if (!chk(bs_pred_index(w.x, L.ns) && w.y >= 0, BS_CHK_BATCH)) continue;
@@ -404,35 +410,32 @@ __global__ void __launch_bounds__(kBBlock, FF ? 3 : (sizeof(T) == 8 ? 2 : 4))
     }
   }
   if (!grid_sync(L.bar, L.err)) return;
-  // C: x += alpha p; r -= alpha Ap; r.r -> beta, stop flag
+  // C: r -= alpha Ap; r.r -> beta, stop flag
   for (int it = blockIdx.x; it < L.nC; it += gridDim.x) {
     const int2 w = L.iC[it];
     if (!chk(bs_pred_index(w.x, L.ns) && w.y >= 0, BS_CHK_BATCH)) continue;
     const BDesc &d = L.d[w.x];
     if (solve_off(d)) continue;
-    const T a = BV<T>::alpha(d.st), na = -a;
-    T *x = BV<T>::x(d), *r = BV<T>::r(d);
-    const T *p = BV<T>::p(d), *Ap = BV<T>::Ap(d);
+    const T na = -BV<T>::alpha(d.st);
+    T *r = BV<T>::r(d);
+    const T *Ap = BV<T>::Ap(d);
     const int64_t i0 = (int64_t)w.y * L.chunk;
     const int64_t i1 = i0 + L.chunk < d.NG ? i0 + L.chunk : d.NG;
     Acc<T> acc;
-    // U entries per thread per sweep, all 4 U loads issued together
-    for (int64_t i = i0 + threadIdx.x; i < i1; i += U * kBBlock) {
-      T pv[U], av[U], xv[U], rv[U];
+    // 2 U entries per thread per sweep, all 4 U loads issued together
+    for (int64_t i = i0 + threadIdx.x; i < i1; i += 2 * U * kBBlock) {
+      T av[2 * U], rv[2 * U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
+      for (int u = 0; u < 2 * U; ++u) {
         const int64_t k = i + u * kBBlock;
         const bool in = k < i1;
-        pv[u] = in ? p[k] : T(0);
         av[u] = in ? Ap[k] : T(0);
-        xv[u] = in ? x[k] : T(0);
         rv[u] = in ? r[k] : T(0);
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
+      for (int u = 0; u < 2 * U; ++u) {
         const int64_t k = i + u * kBBlock;
         if (k < i1) {
-          x[k] = fmaT(a, pv[u], xv[u]);
           const T ri = fmaT(na, av[u], rv[u]);
           r[k] = ri;
           acc.add(ri, ri);
@@ -446,29 +449,33 @@ __global__ void __launch_bounds__(kBBlock, FF ? 3 : (sizeof(T) == 8 ? 2 : 4))
       finish_iteration(L, w.x, d.st, rr);
   }
   if (!grid_sync(L.bar, L.err)) return;
-  // D: p = r + beta p
+  // D: x += alpha p, p = r + beta p, also where C has just stopped the solve
   for (int it = blockIdx.x; it < L.nC; it += gridDim.x) {
     const int2 w = L.iC[it];
     if (!chk(bs_pred_index(w.x, L.ns) && w.y >= 0, BS_CHK_BATCH)) continue;
     const BDesc &d = L.d[w.x];
-    if (solve_off(d)) continue;
-    const T bt = BV<T>::beta(d.st);
-    T *p = BV<T>::p(d);
+    if (!d.active || *(volatile const int *)&d.st->xdue == 0) continue;
+    const T a = BV<T>::alpha(d.st), bt = BV<T>::beta(d.st);
+    T *x = BV<T>::x(d), *p = BV<T>::p(d);
     const T *r = BV<T>::r(d);
     const int64_t i0 = (int64_t)w.y * L.chunk;
     const int64_t i1 = i0 + L.chunk < d.NG ? i0 + L.chunk : d.NG;
     for (int64_t i = i0 + threadIdx.x; i < i1; i += U * kBBlock) {
-      T rv[U], pv[U];
+      T rv[U], pv[U], xv[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int64_t k = i + u * kBBlock;
         rv[u] = k < i1 ? r[k] : T(0);
         pv[u] = k < i1 ? p[k] : T(0);
+        xv[u] = k < i1 ? x[k] : T(0);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int64_t k = i + u * kBBlock;
-        if (k < i1) p[k] = fmaT(T(1), rv[u], bt * pv[u]);
+        if (k < i1) {
+          x[k] = fmaT(a, pv[u], xv[u]);
+          p[k] = fmaT(T(1), rv[u], bt * pv[u]);
+        }
       }
     }
   }

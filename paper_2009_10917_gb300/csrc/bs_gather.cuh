@@ -102,15 +102,44 @@ __device__ __forceinline__ void gather_tile(int2 lo, int2 hi,
         const int kk = threadIdx.x + u * kGatherBlock;
         if (kk < nk) s_v[kk] = v[u];
       }
+      // rows in batches whose starts (and w) a thread loads together, the first
+      // batch's before the values have landed: one latency for all of them
+      // instead of two per row
+      constexpr int R = 4;
+      int ra[R], rb[R];
+      int32_t rg[R];
+      T wv[DOT ? R : 1];
+      auto fetch = [&](int32_t first) {
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const int32_t r = first + q * kGatherBlock;
+          ra[q] = rb[q] = 0;
+          rg[q] = -1;
+          if (r >= r1) continue;
+          ra[q] = row_starts[r] - k0;
+          rb[q] = row_starts[r + 1] - k0;
+          rg[q] = ROWMAP ? __ldcs(rows + r) : r;
+        }
+        if (DOT)
+#pragma unroll
+          for (int q = 0; q < R; ++q)
+            wv[DOT ? q : 0] =
+                rg[q] >= 0 && chk(bs_pred_index(rg[q], gb.ng), BS_CHK_GATHER_ROW)
+                    ? __ldcs(w + rg[q]) : T(0);
+      };
+      fetch(r0 + threadIdx.x);
       __syncthreads();
-      for (int32_t r = r0 + threadIdx.x; r < r1; r += kGatherBlock) {
-        int a = row_starts[r] - k0, b = row_starts[r + 1] - k0;
-        if (!chk(bs_pred_row(a, b, nk), BS_CHK_GATHER_ROW)) a = b = 0;
-        const T s = row_sum(s_v, a, b);
-        const int32_t g = ROWMAP ? __ldcs(rows + r) : r;
-        if (!chk(bs_pred_index(g, gb.ng), BS_CHK_GATHER_ROW)) continue;
-        __stcs(qG + g, s);
-        if (DOT) acc.add(__ldcs(w + g), s);
+      for (int32_t first = r0 + threadIdx.x; first < r1; first += R * kGatherBlock) {
+        if (first != r0 + (int)threadIdx.x) fetch(first);
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          if (rg[q] < 0) continue;
+          if (!chk(bs_pred_row(ra[q], rb[q], nk), BS_CHK_GATHER_ROW)) ra[q] = rb[q] = 0;
+          const T s = row_sum(s_v, ra[q], rb[q]);
+          if (!chk(bs_pred_index(rg[q], gb.ng), BS_CHK_GATHER_ROW)) continue;
+          __stcs(qG + rg[q], s);
+          if (DOT) acc.add(wv[DOT ? q : 0], s);
+        }
       }
       __syncthreads();
     } else {  // a single row longer than a tile: read straight from memory
