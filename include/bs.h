@@ -274,7 +274,7 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   node).  Without it, for odd N <= 9, they use the even-odd form of the
  *   centrosymmetric W^-1 K (Solomonoff's decomposition; half-length
  *   contractions, about a quarter fewer operations per node), and the FP64
- *   kernels of degrees 4..7 (the batched solver's too) evaluate the
+ *   kernels of degrees 4..15 (the batched solver's of 4..7) evaluate the
  *   contractions exactly in 58-bit fixed point relative to each element's
  *   largest value, on the tensor cores (an element whose values are not
  *   finite, lie outside [2^-900, 2^900] or differ too much in size takes

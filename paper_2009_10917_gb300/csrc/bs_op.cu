@@ -119,9 +119,10 @@ static DD operator/(DD a, DD b) {
 // bits, the diagonal minus the rest of its row where the rows sum to zero,
 // then signed 10-bit digits by the bias of 512 per digit that the kernels use
 // for their values, as the bits of a half.  False when a sum of products
-// could leave its accumulator (it cannot, for the matrices of degrees 4..7).
-template <class M>
-static bool fx_digits(int Nq, M mat, bool zero_rows, uint32_t (*w)[32], int *q) {
+// could leave its accumulator (it cannot, for the matrices of degrees 4..15).
+// word(b, i, m, bits): the digits b of entries (i, m), (i, m + 1), m even.
+template <class M, class W>
+static bool fx_digits(int Nq, M mat, bool zero_rows, W word, int *q) {
   double big = 0.0;
   for (int i = 0; i < Nq; ++i)
     for (int m = 0; m < Nq; ++m) big = std::fmax(big, std::fabs(mat(i, m).h));
@@ -145,13 +146,17 @@ static bool fx_digits(int Nq, M mat, bool zero_rows, uint32_t (*w)[32], int *q) 
     return (int)(((bias + Ki[i][m]) >> (10 * (kFxDigits - 1 - d))) & 0x3ff) - 512;
   };
   // the largest sum an accumulator can meet: digits of a value up to 257
-  // (the first) or 512 in magnitude, products a + b = o of one row
+  // (the first) or 512 in magnitude, products a + b = o of one row; beyond
+  // kFxMaxNq those of digits 2 and 3 have an accumulator of their own (o >= 3)
   for (int o = 0; o < kFxDigits; ++o)
     for (int i = 0; i < Nq; ++i) {
-      int64_t s = 0;
+      int64_t s[2] = {0, 0};
       for (int a = 0; a <= o; ++a)
-        for (int m = 0; m < Nq; ++m) s += (a ? 512 : 257) * std::abs(digit(i, m, o - a));
-      if (s > (o == kFxDigits - 1 ? 1 << 23 : 1 << 22)) return false;
+        for (int m = 0; m < Nq; ++m)
+          s[Nq > kFxMaxNq && o >= 3 && (a == 2 || a == 3)] +=
+              (a ? 512 : 257) * std::abs(digit(i, m, o - a));
+      const int64_t most = o == kFxDigits - 1 ? 1 << 23 : 1 << 22;
+      if (s[0] > most || s[1] > most) return false;
     }
   auto half_bits = [](int v) -> uint32_t {  // |v| <= 512
     if (v == 0) return 0;
@@ -161,24 +166,20 @@ static bool fx_digits(int Nq, M mat, bool zero_rows, uint32_t (*w)[32], int *q) 
     return sign | ((uint32_t)(p + 15) << 10) | ((a << (10 - p)) & 0x3ffu);
   };
   for (int d = 0; d < kFxDigits; ++d)
-    for (int lane = 0; lane < 32; ++lane) {
-      uint32_t word = 0;
-      for (int hf = 0; hf < 2; ++hf) {
-        const int i = lane >> 2, m = 2 * (lane & 3) + hf;
-        if (i < Nq && m < Nq) word |= half_bits(digit(i, m, d)) << (16 * hf);
-      }
-      w[d][lane] = word;
-    }
+    for (int i = 0; i < Nq; ++i)
+      for (int m = 0; m < Nq; m += 2)
+        word(d, i, m,
+             half_bits(digit(i, m, d)) | (m + 1 < Nq ? half_bits(digit(i, m + 1, d)) << 16 : 0u));
   return true;
 }
 
-// The digits of Kh = W^-1 K, D and D^T (bs_op_fx.cuh, bs_op_geo_fx.cuh), from GLL
-// nodes, weights and derivative matrix redone in double-double (Newton on the
+// The digits of Kh = W^-1 K and, up to degree 7, D and D^T (bs_op_fx.cuh,
+// bs_op_fx16.cuh, bs_op_geo_fx.cuh), from GLL nodes, weights and derivative matrix redone in double-double (Newton on the
 // nodes x, as gll_tables): a 58-bit entry holds more than a double, and an
 // error common to every element would shift the operator's low modes
 // coherently.  Also the weights' products of the affine kernel.
 static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t,
-                     FxGeoTab *tg) {
+                     FxGeoTab *tg, FxTab16 *t16) {
   const int Nq = N + 1;
   DD x[kMaxNq], w[kMaxNq], D[kMaxNq][kMaxNq], Kh[kMaxNq][kMaxNq];
   auto legendre = [&](DD z, DD *pn, DD *pm) {  // P_N, P_{N-1}
@@ -223,11 +224,29 @@ static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t,
       for (int a = 0; a < Nq; ++a) s = s + D[a][i] * w[a] * D[a][m];
       Kh[i][m] = s / w[i];
     }
-  if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, t->w, &t->q) ||
-      !fx_digits(Nq, [&](int i, int m) { return D[i][m]; }, true, tg->d, &tg->qd) ||
-      !fx_digits(Nq, [&](int i, int m) { return D[m][i]; }, false, tg->dt, &tg->qdt))
-    return false;
   const DD g(0.5 * h), ml = DD(lambda) * g * g * g;
+  if (Nq > kFxMaxNq) {
+    auto word = [&](int b, int i, int m, uint32_t bits) {
+      t16->w[b][(i % 8) * 4 + m % 8 / 2][i / 8 + 2 * (m / 8)] = bits;
+    };
+    if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, word, &t16->q)) return false;
+    for (int k = 0; k < Nq; ++k) t16->w1[k] = w[k].h;
+    for (int lane = 0; lane < 32; ++lane)
+      for (int q = 0; q < 8; ++q) {
+        const int j = (lane >> 2) + 8 * (q >> 2), i = 2 * (lane & 3) + 8 * ((q >> 1) & 1) + (q & 1);
+        if (i >= Nq || j >= Nq) continue;
+        t16->wg[lane * 8 + q] = (w[i] * w[j] * g).h;
+        t16->wm[lane * 8 + q] = (w[i] * w[j] * ml).h;
+      }
+    return true;
+  }
+  auto words = [](uint32_t (*to)[32]) {
+    return [to](int b, int i, int m, uint32_t bits) { to[b][i * 4 + m / 2] = bits; };
+  };
+  if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, words(t->w), &t->q) ||
+      !fx_digits(Nq, [&](int i, int m) { return D[i][m]; }, true, words(tg->d), &tg->qd) ||
+      !fx_digits(Nq, [&](int i, int m) { return D[m][i]; }, false, words(tg->dt), &tg->qdt))
+    return false;
   for (int k = 0; k < Nq; ++k)
     for (int lane = 0; lane < 32; ++lane)
       for (int hf = 0; hf < 2; ++hf) {
@@ -378,7 +397,7 @@ int bs_problem_create(const bs_map *map, double h, double lambda, const double *
         split(o, tabff.Eoh[a * hq + m], tabff.Eol[a * hq + m]);
       }
   }
-  if (Nq >= kFxMinNq && Nq <= kFxMaxNq && !fx_table(N, x, h, lambda, &tab.fx, &tab.fxg)) {
+  if (Nq >= kFxMinNq && !fx_table(N, x, h, lambda, &tab.fx, &tab.fxg, &tab.fx16)) {
     free(p);
     return fail(BS_ERR_ARG, "bs_problem_create: digit tables of degree %d out of range", N);
   }

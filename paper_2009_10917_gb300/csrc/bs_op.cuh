@@ -48,6 +48,15 @@ struct __align__(16) FxTab {
   double wg[kFxMaxNq * 64], wm[kFxMaxNq * 64];
   int q;
 };
+// Degrees 8..15 (bs_op_fx16.cuh): w[b][lane] = digit b of Kh[g][2t ..], Kh[g + 8]
+// [2t ..], Kh[g][2t + 8 ..], Kh[g + 8][2t + 8 ..] as pairs of halves; wg, wm
+// [lane][q]: (h/2) w_i w_j and lambda (h/2)^3 w_i w_j of a lane's eight nodes of a
+// layer; w1: the weights.
+struct __align__(16) FxTab16 {
+  uint32_t w[kFxDigits][32][4];
+  double wg[256], wm[256], w1[kMaxNq];
+  int q;
+};
 // The same digits of the derivative matrix D (d, scale qd) and of D^T (dt, qdt).
 struct FxGeoTab {
   uint32_t d[kFxDigits][32], dt[kFxDigits][32];
@@ -66,6 +75,7 @@ struct OpTab {
   T Eo[(kMaxNq / 2) * (kMaxNq / 2)];
   FxTab fx;        // FP64 tables only
   FxGeoTab fxg;
+  FxTab16 fx16;
   int64_t ne, ng;  // the problem's E and N_G (index checks of the checked build)
 };
 
@@ -386,6 +396,7 @@ __global__ void __launch_bounds__(OpShape<NQ>::THREADS)
 }  // namespace bs
 
 #include "bs_op_fx.cuh"
+#include "bs_op_fx16.cuh"
 
 namespace bs {
 
@@ -396,7 +407,7 @@ inline int64_t ax_blocks(int N, int64_t E, bool fx) {
   switch (N + 1) {
 #define BS_AXB(NQ)                                                      \
   case NQ:                                                              \
-    if (fx && use_fx<NQ>() && g_op_evenodd)                             \
+    if (fx && (use_fx<NQ>() || use_fx16<NQ>()) && g_op_evenodd)         \
       return E;                                                         \
     return use_eo<NQ>() && g_op_evenodd                                 \
                ? (E + EoShape<NQ>::EPB - 1) / EoShape<NQ>::EPB          \
@@ -427,6 +438,16 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
         k_ax_fx<NQ, GATHER_IN, FUSED>                                                    \
             <<<(unsigned)E, Sf::THREADS, Sf::SMEM, s>>>(E, order, ids, in, out, tab, coef, \
                                                         st, outG, partials, vec);        \
+        break;                                                                           \
+      }                                                                                  \
+    } else if constexpr (use_fx16<NQ>() && sizeof(T) == 8) {                             \
+      if (g_op_evenodd) {                                                                \
+        using Sf = FxShape16<NQ>;                                                        \
+        auto kern = k_ax_fx16<NQ, GATHER_IN, FUSED>;                                     \
+        if (occupancy_blocks_smem((const void *)kern, Sf::THREADS, Sf::SMEM) < 1)        \
+          return fail(BS_ERR_CUDA, "element operator: shared memory refused");           \
+        kern<<<(unsigned)E, Sf::THREADS, Sf::SMEM, s>>>(E, order, ids, in, out, tab,     \
+                                                        coef, st, outG, partials);       \
         break;                                                                           \
       }                                                                                  \
     } else if constexpr (use_eo<NQ>()) {                                                 \
