@@ -249,8 +249,8 @@ int bs_diag_A(const bs_problem *prob, double *d_diag, void *stream);
  * the same way, so the same window applies to them: they scale as L and
  * lambda L^3 with the mesh's length scale L, and below 2^-102 they count as
  * zero -- keep L above about 2^-28 (lambda of order 1) for the accuracy
- * stated here.  The gather is the same as bs_apply_A's.  At degrees 6 and 7
- * (5..7 with geometric factors; without BS_OP_DIRECT) the FP64 fixed-point
+ * stated here.  The gather is the same as bs_apply_A's.  At degrees 6, 7 and
+ * 11..15 (5..7 with geometric factors; without BS_OP_DIRECT) the FP64 fixed-point
  * kernel of bs_apply_A is the faster one and runs instead: FP64's accuracy and
  * range. */
 int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *stream);

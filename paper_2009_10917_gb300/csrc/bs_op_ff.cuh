@@ -636,10 +636,11 @@ extern int g_op_fusion;
 // kernel, FP64 only).  DOT: ep(p . Ap), reduced in the gather's pass (and,
 // fused, in the element kernel's epilogue for the single-copy nodes).
 // Whether a float-float A p runs the FP64 fixed-point kernel (bs_op_fx.cuh): at
-// degrees 6 and 7 it is the faster of the two (10M local nodes, with the gather:
-// 160 against 221 us at N = 6, 125 against 216 at N = 7; N = 5 185 against 187,
-// N = 4 234 against 183) and exact to FP64's rounding.
-inline bool ff_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7); }
+// degrees 6, 7 and 11..15 it is the faster of the two (10M local nodes, with the
+// gather: 160 against 221 us at N = 6, 125 against 216 at N = 7, 289 against 397
+// at N = 11, 173 against 405 at N = 15; N = 5 185 against 187, N = 4 234 against
+// 183, N = 9 359 against 252) and exact to FP64's rounding.
+inline bool ff_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7 || N >= 11); }
 // The same on general hexahedra, degrees 5..7: 559 against 608 us, 438 against
 // 753, 324 against 770.
 inline bool ff_geo_takes_fx(int N) { return g_op_evenodd && N >= 5 && N <= 7; }
