@@ -279,10 +279,13 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   largest value, on the tensor cores (an element whose values are not
  *   finite, lie outside [2^-900, 2^900] or differ too much in size takes
  *   the direct FP64 sums); results differ by rounding only.
+ *   bs_fpcg_learned with a network takes the FP64 or float-float sums in any
+ *   case: its input is quantised, so single nodes would show the rounding.
  * Problems with geometric factors (bs_problem_create_geo) always use their
  * own unfused kernels (FP64 and float-float; at degrees 5..7, without
- * BS_OP_DIRECT, the FP64 one in the fixed-point form as well).  Returns the previous mode; a negative value only
- * queries it.  Not thread-safe against solves in flight. */
+ * BS_OP_DIRECT, the FP64 one in the fixed-point form as well).  Returns the
+ * previous mode; a negative value only queries it.  Not thread-safe against
+ * solves in flight. */
 enum { BS_OP_FUSED = 1, BS_OP_DIRECT = 2 };
 int bs_operator_mode(int32_t mode);
 

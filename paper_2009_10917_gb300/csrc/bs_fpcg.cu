@@ -321,7 +321,10 @@ struct FpVecs {
   double *r, *p, *Ap, *z, *dinv, *corr;
 };
 static FpVecs fpvecs(const bs_problem *P) {
-  const int64_t s = vec_stride(P->map->NG);
+  // not vec_stride: where that moves a vector to 16 bytes, the update's r.r is
+  // summed in another order, and k_fp_prep amplifies last-bit changes (see
+  // fpcg_iteration)
+  const int64_t s = P->map->NG + 2;
   double *v = P->d_vec;
   return FpVecs{v, v + s, v + 2 * s, v + 3 * s, v + 4 * s, v + 5 * s};
 }
@@ -401,8 +404,14 @@ static int fpcg_iteration(const bs_problem *P, bs_mlp *mlp, int odd, bool ff, do
   FpVecs v = fpvecs(P);
   CgState *st = P->d_state;
   const double g = 0.5 * P->h, mlam = P->lambda * g * g * g;
+  // With a network, no fixed-point element kernels: k_fp_prep's quantisers (24-bit
+  // truncation, then BF16 pairs) are discontinuous in r, so a last-bit change of
+  // A p flips some of an element's 2^-17 steps and single nodes of x move by up to
+  // 6e-8 of its RMS in 12 iterations (N = 5, 32^3), however accurate the change.
+  // The iterates stay those of the FP64 sums; the fixed-point form would take
+  // 365 us an iteration instead of 606.
   int rc = apply_A_global<double, true, EpAlphaRz>(P, ff, P->d_tab, v.p, v.Ap, P->d_ApL, g,
-                                                   mlam, EpAlphaRz{st}, st, s);
+                                                   mlam, EpAlphaRz{st}, st, s, !mlp);
   if (!rc)
     rc = launch_cg_update<double, EpResidual>(m->NG, Scalar<double>{0.0, &st->alpha}, v.p, v.Ap,
                                               x, v.r, P->d_partials, P->d_counter,

@@ -421,18 +421,19 @@ inline int64_t ax_blocks(int N, int64_t E, bool fx) {
 }
 
 // FUSED: ids is the fused encoding, outG the global output, partials (or
-// NULL: no dot product) ax_blocks(N, E) doubles.
+// NULL: no dot product) ax_blocks(N, E) doubles.  fx: FP64 may take the
+// fixed-point form.
 template <typename T, bool GATHER_IN, bool FUSED = false>
 int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, const T *in,
                     T *out,
                     const OpTab<T> *tab, const double *coef, T g, T mlam,
                     const CgState *st, cudaStream_t s, T *outG = nullptr,
-                    double *partials = nullptr) {
+                    double *partials = nullptr, bool fx = true) {
   if (E == 0) return BS_OK;
 #define BS_AX_CASE(NQ)                                                                   \
   case NQ: {                                                                             \
     if constexpr (use_fx<NQ>() && sizeof(T) == 8) {                                      \
-      if (g_op_evenodd) {                                                                \
+      if (fx && g_op_evenodd) {                                                          \
         const int vec = ((uintptr_t)out % 16 == 0) && (GATHER_IN || (uintptr_t)in % 16 == 0); \
         using Sf = FxShape<NQ>;                                                          \
         k_ax_fx<NQ, GATHER_IN, FUSED>                                                    \
@@ -441,7 +442,7 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
         break;                                                                           \
       }                                                                                  \
     } else if constexpr (use_fx16<NQ>() && sizeof(T) == 8) {                             \
-      if (g_op_evenodd) {                                                                \
+      if (fx && g_op_evenodd) {                                                          \
         using Sf = FxShape16<NQ>;                                                        \
         auto kern = k_ax_fx16<NQ, GATHER_IN, FUSED>;                                     \
         if (occupancy_blocks_smem((const void *)kern, Sf::THREADS, Sf::SMEM) < 1)        \
@@ -450,7 +451,9 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
                                                         coef, st, outG, partials);       \
         break;                                                                           \
       }                                                                                  \
-    } else if constexpr (use_eo<NQ>()) {                                                 \
+    }                                                                                    \
+    if constexpr (use_eo<NQ>() &&                                                        \
+                  (GATHER_IN || sizeof(T) == 4 || !(use_fx<NQ>() || use_fx16<NQ>()))) {  \
       if (g_op_evenodd) {                                                                \
         using Se = EoShape<NQ>;                                                          \
         const int64_t grid = (E + Se::EPB - 1) / Se::EPB;                                \

@@ -632,9 +632,6 @@ int launch_ax_geo_ff(int N, int64_t E, int64_t NL, const int32_t *order, const i
 // 0 (the default): element kernel, then the gather of every row.
 extern int g_op_fusion;
 
-// Ap = A p for a global p (FP64 or FP32 tables; ff: the float-float element
-// kernel, FP64 only).  DOT: ep(p . Ap), reduced in the gather's pass (and,
-// fused, in the element kernel's epilogue for the single-copy nodes).
 // Whether a float-float A p runs the FP64 fixed-point kernel (bs_op_fx.cuh): at
 // degrees 6, 7 and 11..15 it is the faster of the two (10M local nodes, with the
 // gather: 160 against 221 us at N = 6, 125 against 216 at N = 7, 289 against 397
@@ -645,18 +642,23 @@ inline bool ff_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7 || N >
 // 753, 324 against 770.
 inline bool ff_geo_takes_fx(int N) { return g_op_evenodd && N >= 5 && N <= 7; }
 
+// Ap = A p for a global p (FP64 or FP32 tables; ff: the float-float element
+// kernel, FP64 only).  DOT: ep(p . Ap), reduced in the gather's pass (and,
+// fused, in the element kernel's epilogue for the single-copy nodes).  fx: the
+// fixed-point element kernels may run.
 template <typename T, bool DOT, class Ep>
 int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p, T *Ap, T *ApL,
-                   T g, T mlam, Ep ep, const CgState *st, cudaStream_t s) {
+                   T g, T mlam, Ep ep, const CgState *st, cudaStream_t s, bool fx = true) {
   const bs_map *m = P->map;
   if (P->d_geo) {  // general hexahedra: FP64 or float-float, unfused
     if constexpr (std::is_same<T, double>::value) {
-      if (int rc = ff && !ff_geo_takes_fx(P->N)
+      if (int rc = ff && !(fx && ff_geo_takes_fx(P->N))
                       ? launch_ax_geo_ff<true>(P->N, m->E, m->NL, m->d_elem_order, m->d_ids, p,
                                                ApL, P->d_tabff, P->d_coef, P->d_geo, P->lambda,
                                                st, s)
                       : launch_ax_geo<true>(P->N, m->E, m->NL, m->d_elem_order, m->d_ids, p, ApL,
-                                            P->d_tab, P->d_coef, P->d_geo, P->lambda, st, s))
+                                            P->d_tab, P->d_coef, P->d_geo, P->lambda, st, s,
+                                            fx))
         return rc;
       return launch_gather<T, DOT, Ep>(m, ApL, Ap, DOT ? p : nullptr, P->d_partials,
                                        P->d_counter, ep, st, s);
@@ -668,7 +670,7 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
   const int32_t *ids = fused ? m->d_ids_f : m->d_ids;
   double *opp = fused && DOT ? P->d_op_partials : nullptr;
   int rc;
-  const bool ffk = ff && !ff_takes_fx(P->N);
+  const bool ffk = ff && !(fx && ff_takes_fx(P->N));
   if constexpr (std::is_same<T, double>::value) {
     if (ffk)
       rc = fused ? launch_ax_local_ff<true, true>(P->N, m->E, m->d_elem_order, ids, p, ApL,
@@ -677,9 +679,9 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
                                             P->d_coef, g, mlam, st, s);
     else
       rc = fused ? launch_ax_local<T, true, true>(P->N, m->E, m->d_elem_order, ids, p, ApL, tab,
-                                                  P->d_coef, g, mlam, st, s, Ap, opp)
+                                                  P->d_coef, g, mlam, st, s, Ap, opp, fx)
                  : launch_ax_local<T, true>(P->N, m->E, m->d_elem_order, ids, p, ApL, tab,
-                                            P->d_coef, g, mlam, st, s);
+                                            P->d_coef, g, mlam, st, s, nullptr, nullptr, fx);
   } else {
     if (ff) return fail(BS_ERR_ARG, "the float-float operator is FP64 only");
     rc = fused ? launch_ax_local<T, true, true>(P->N, m->E, m->d_elem_order, ids, p, ApL, tab,
@@ -692,8 +694,10 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
     return launch_gather<T, DOT, Ep>(m, ApL, Ap, DOT ? p : nullptr, P->d_partials, P->d_counter,
                                      ep, st, s);
   return launch_gather_rows<T, DOT, Ep>(m, fused, ApL, Ap, DOT ? p : nullptr, P->d_partials,
-                                        P->d_counter, opp, opp ? ax_blocks(P->N, m->E, sizeof(T) == 8 && !ffk) : 0, ep,
-                                        st, s);
+                                        P->d_counter, opp,
+                                        opp ? ax_blocks(P->N, m->E, fx && sizeof(T) == 8 && !ffk)
+                                            : 0,
+                                        ep, st, s);
 }
 
 }  // namespace bs
