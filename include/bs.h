@@ -267,14 +267,14 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   kernel writes every local value and the gather (BS6) sums every row.  Ap
  *   is bitwise the same either way (a one-copy row sums to +0 + v); p.Ap
  *   differs only by summation order.  Measured slower on GB300
- *   (partial-sector writes into Ap; N = 7 on 48^3: 1.37 vs 1.24 ms per
- *   float-float A p).
+ *   (partial-sector writes into Ap; N = 7 on 48^3: 0.69 vs 0.60 ms per
+ *   A p).
  *  BS_OP_DIRECT: the element kernels (FP64, FP32, float-float) contract
  *   with the full 1-D stiffness K = D^T W D (3 (N+1) multiply-adds per
  *   node).  Without it, for odd N <= 9, they use the even-odd form of the
  *   centrosymmetric W^-1 K (Solomonoff's decomposition; half-length
  *   contractions, about a quarter fewer operations per node), and the FP64
- *   kernels of degrees 4..15 (the batched solver's of 4..7) evaluate the
+ *   kernels of degrees 2..15 (the batched solver's of 4..7) evaluate the
  *   contractions exactly in 58-bit fixed point relative to each element's
  *   largest value, on the tensor cores (an element whose values are not
  *   finite, lie outside [2^-900, 2^900] or differ too much in size takes

@@ -119,7 +119,7 @@ static DD operator/(DD a, DD b) {
 // bits, the diagonal minus the rest of its row where the rows sum to zero,
 // then signed 10-bit digits by the bias of 512 per digit that the kernels use
 // for their values, as the bits of a half.  False when a sum of products
-// could leave its accumulator (it cannot, for the matrices of degrees 4..15).
+// could leave its accumulator (it cannot, for the matrices of degrees 2..15).
 // word(b, i, m, bits): the digits b of entries (i, m), (i, m + 1), m even.
 template <class M, class W>
 static bool fx_digits(int Nq, M mat, bool zero_rows, W word, int *q) {
@@ -174,12 +174,12 @@ static bool fx_digits(int Nq, M mat, bool zero_rows, W word, int *q) {
 }
 
 // The digits of Kh = W^-1 K and, up to degree 7, D and D^T (bs_op_fx.cuh,
-// bs_op_fx16.cuh, bs_op_geo_fx.cuh), from GLL nodes, weights and derivative matrix redone in double-double (Newton on the
+// bs_op_fx16.cuh, bs_op_fx4.cuh, bs_op_geo_fx.cuh), from GLL nodes, weights and derivative matrix redone in double-double (Newton on the
 // nodes x, as gll_tables): a 58-bit entry holds more than a double, and an
 // error common to every element would shift the operator's low modes
 // coherently.  Also the weights' products of the affine kernel.
 static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t,
-                     FxGeoTab *tg, FxTab16 *t16) {
+                     FxGeoTab *tg, FxTab16 *t16, FxTab4 *t4) {
   const int Nq = N + 1;
   DD x[kMaxNq], w[kMaxNq], D[kMaxNq][kMaxNq], Kh[kMaxNq][kMaxNq];
   auto legendre = [&](DD z, DD *pn, DD *pm) {  // P_N, P_{N-1}
@@ -237,6 +237,27 @@ static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t,
         if (i >= Nq || j >= Nq) continue;
         t16->wg[lane * 8 + q] = (w[i] * w[j] * g).h;
         t16->wm[lane * 8 + q] = (w[i] * w[j] * ml).h;
+      }
+    return true;
+  }
+  if (Nq < kFxMinNq) {
+    // every order in one accumulator counting by one: at most 0.23 of 2^22 with these
+    // matrices' digits, the check below allows twice that for the last
+    auto word = [&](int b, int i, int m, uint32_t bits) {
+      for (int x = 0; x < kFxDigits / 2; ++x)
+        for (int od = 0; od < 2; ++od)
+          for (int th = 0; th < 2; ++th)
+            if (2 * x + od - th == b) t4->w[x][(4 * od + i) * 4 + 2 * th + m / 2] = bits;
+    };
+    if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, word, &t4->q)) return false;
+    for (int lane = 0; lane < 32; ++lane)
+      for (int hf = 0; hf < 2; ++hf) {
+        const int g4 = lane >> 2, t = lane & 3;
+        const int i = 2 * (t & 1) + hf, j = g4 & 3, k = 2 * (g4 >> 2) + (t >> 1);
+        if (i >= Nq || j >= Nq || k >= Nq) continue;
+        const DD w3 = w[i] * w[j] * w[k];
+        t4->wg[lane * 2 + hf] = (w3 * g).h;
+        t4->wm[lane * 2 + hf] = (w3 * ml).h;
       }
     return true;
   }
@@ -397,7 +418,7 @@ int bs_problem_create(const bs_map *map, double h, double lambda, const double *
         split(o, tabff.Eoh[a * hq + m], tabff.Eol[a * hq + m]);
       }
   }
-  if (Nq >= kFxMinNq && !fx_table(N, x, h, lambda, &tab.fx, &tab.fxg, &tab.fx16)) {
+  if (Nq > 2 && !fx_table(N, x, h, lambda, &tab.fx, &tab.fxg, &tab.fx16, &tab.fx4)) {
     free(p);
     return fail(BS_ERR_ARG, "bs_problem_create: digit tables of degree %d out of range", N);
   }

@@ -13,6 +13,9 @@
 // element and walks k, keeping the column in registers; the element sits in
 // shared memory.  Reading the input through the map (GATHER_IN) fuses the
 // scatter Z p into the same pass, so the N_L-sized Z p is never stored.
+// That kernel, and its even-odd form below, serve FP32, BS_OP_DIRECT and the
+// FP64 calls that keep FP64 sums; by default FP64 at degrees 2..15 runs the
+// fixed-point kernels of bs_op_fx4.cuh, bs_op_fx.cuh and bs_op_fx16.cuh.
 //
 // Fused form (FUSED): the map comes re-encoded (bs_map::d_ids_f) so that the
 // kernel knows which global nodes have a single local copy -- element
@@ -22,8 +25,8 @@
 // per-block partial of p.Ap; only the shared nodes' local values go to the
 // N_L buffer, for a gather over the shared rows alone.  The result is
 // bitwise that of the unfused operator (a one-term row sum is +0 + v).
-// Measured slower on GB300 (N = 7 on 48^3: 1.365 vs 1.244 ms per A p with
-// the float-float kernel, 3.54 vs 3.44 ms in FP64): in the user's global
+// Measured slower on GB300 (N = 7 on 48^3: 0.69 vs 0.60 ms per A p, 3.52 vs
+// 3.40 ms with the direct kernel): in the user's global
 // numbering the single-copy nodes come in runs of N - 1 doubles and the
 // shared rows between them, so both kernels write partial sectors of A p,
 // which costs more than the N_L round trip saved.  Off by default.
@@ -57,6 +60,13 @@ struct __align__(16) FxTab16 {
   double wg[256], wm[256], w1[kMaxNq];
   int q;
 };
+// Degrees 2 and 3 (bs_op_fx4.cuh): w[x][lane] = digit 2x + g / 4 - t / 2 (none: zero) of
+// Kh[g % 4][2 (t % 2) ..]; wg, wm [lane][h] as FxTab's, of a lane's two nodes.
+struct __align__(16) FxTab4 {
+  uint32_t w[kFxDigits / 2][32];
+  double wg[64], wm[64];
+  int q;
+};
 // The same digits of the derivative matrix D (d, scale qd) and of D^T (dt, qdt).
 struct FxGeoTab {
   uint32_t d[kFxDigits][32], dt[kFxDigits][32];
@@ -76,6 +86,7 @@ struct OpTab {
   FxTab fx;        // FP64 tables only
   FxGeoTab fxg;
   FxTab16 fx16;
+  FxTab4 fx4;
   int64_t ne, ng;  // the problem's E and N_G (index checks of the checked build)
 };
 
@@ -397,6 +408,7 @@ __global__ void __launch_bounds__(OpShape<NQ>::THREADS)
 
 #include "bs_op_fx.cuh"
 #include "bs_op_fx16.cuh"
+#include "bs_op_fx4.cuh"
 
 namespace bs {
 
@@ -409,6 +421,8 @@ inline int64_t ax_blocks(int N, int64_t E, bool fx) {
   case NQ:                                                              \
     if (fx && (use_fx<NQ>() || use_fx16<NQ>()) && g_op_evenodd)         \
       return E;                                                         \
+    if (fx && use_fx4<NQ>() && g_op_evenodd)                            \
+      return (E + kFx4Epb - 1) / kFx4Epb;                               \
     return use_eo<NQ>() && g_op_evenodd                                 \
                ? (E + EoShape<NQ>::EPB - 1) / EoShape<NQ>::EPB          \
                : (E + OpShape<NQ>::EPB - 1) / OpShape<NQ>::EPB;
@@ -451,9 +465,16 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
                                                         coef, st, outG, partials);       \
         break;                                                                           \
       }                                                                                  \
+    } else if constexpr (use_fx4<NQ>() && sizeof(T) == 8) {                              \
+      if (fx && g_op_evenodd) {                                                          \
+        const int vec = ((uintptr_t)out % 16 == 0) && (GATHER_IN || (uintptr_t)in % 16 == 0); \
+        const int64_t grid = (E + kFx4Epb - 1) / kFx4Epb;                                \
+        k_ax_fx4<NQ, GATHER_IN, FUSED><<<(unsigned)grid, 32 * kFx4Warps, 0, s>>>(        \
+            E, order, ids, in, out, tab, coef, st, outG, partials, vec);                 \
+        break;                                                                           \
+      }                                                                                  \
     }                                                                                    \
-    if constexpr (use_eo<NQ>() &&                                                        \
-                  (GATHER_IN || sizeof(T) == 4 || !(use_fx<NQ>() || use_fx16<NQ>()))) {  \
+    if constexpr (use_eo<NQ>() && (GATHER_IN || sizeof(T) == 4 || NQ == 2)) {            \
       if (g_op_evenodd) {                                                                \
         using Se = EoShape<NQ>;                                                          \
         const int64_t grid = (E + Se::EPB - 1) / Se::EPB;                                \
