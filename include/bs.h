@@ -276,9 +276,14 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   contractions, about a quarter fewer operations per node), and the FP64
  *   kernels of degrees 2..15 (the batched solver's of 4..7) evaluate the
  *   contractions exactly in 58-bit fixed point relative to each element's
- *   largest value, on the tensor cores (an element whose values are not
- *   finite, lie outside [2^-900, 2^900] or differ too much in size takes
- *   the direct FP64 sums); results differ by rounding only.
+ *   largest value, on the tensor cores.  Nodes whose own terms are too small
+ *   for that -- and elements whose values are not finite or lie outside
+ *   [2^-900, 2^900] -- take FP64 sums, so that every entry of bs_apply_A,
+ *   bs_apply_local and, where it runs this kernel, bs_apply_A_ff is within
+ *   (2 Nq + 4) 2^-53 of the sum of the sizes of its own terms (four standard
+ *   deviations of the digits' rounding at the entries where it is largest;
+ *   (2 Nq + 8) 2^-53 with geometric factors), as the FP64 sums are; inside the
+ *   solvers the deviations may be N - 1 times that.
  *   bs_fpcg_learned with a network takes the FP64 or float-float sums in any
  *   case: its input is quantised, so single nodes would show the rounding.
  * Problems with geometric factors (bs_problem_create_geo) always use their

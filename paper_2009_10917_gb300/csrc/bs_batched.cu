@@ -180,7 +180,7 @@ __device__ __noinline__ void ax_call_fx(int64_t slot0, int64_t slot1, const int3
     if (!chk(bs_pred_index(e, tab->ne), BS_CHK_OP_ENTRY)) continue;
     sync();  // the last element's exchange buffer has been read
     fx_element<NQ, S::L, true, false>(e, (warp - group * S::WPE) * S::L, ids, in, out, tab, coef,
-                                      nullptr, none, 1, smem + group * S::SMEM, sync);
+                                      nullptr, none, 1, 1.f / (NQ - 2), smem + group * S::SMEM, sync);
   }
 }
 

@@ -115,31 +115,37 @@ static DD operator/(DD a, DD b) {
   return dd_fast(q, (r.h + r.l) / b.h);
 }
 
-// A matrix's digit words (bs_op_fx.cuh): each entry an integer of at most 58
-// bits, the diagonal minus the rest of its row where the rows sum to zero,
-// then signed 10-bit digits by the bias of 512 per digit that the kernels use
-// for their values, as the bits of a half.  False when a sum of products
-// could leave its accumulator (it cannot, for the matrices of degrees 2..15).
-// word(b, i, m, bits): the digits b of entries (i, m), (i, m + 1), m even.
+// v (|v| < 2^15) as the bits of a half, rounded to nearest.
+static uint32_t half_bits(double v) {
+  const uint32_t sign = v < 0 ? 0x8000u : 0u;
+  const double a = std::fabs(v);
+  int e = 0;
+  std::frexp(a, &e);  // a in [2^(e-1), 2^e)
+  if (a == 0.0 || e < -13) return sign | (uint32_t)std::rint(std::ldexp(a, 24));  // subnormal
+  return sign | (((uint32_t)(e + 13) << 10) + (uint32_t)std::rint(std::ldexp(a, 11 - e)));
+}
+
+// A matrix in digits (bs_op_fx.cuh): each entry times a scale s 2^q, the largest near
+// 511 2^50 (the first digit then uses its range, and what the digit products leave out
+// is smallest against the entries), as an integer, the diagonal minus the rest of its
+// row where the rows sum to zero, then signed 10-bit digits by the bias of 512 per
+// digit that the kernels use for their values, as the bits of a half.  The scale is the
+// largest, in steps, for which no sum of products can leave its accumulator; false
+// where there is none (there is, for the matrices of degrees 2..15).
+// word(b, i, m, bits): the digits b of entries (i, m), (i, m + 1), m even; b =
+// kFxDigits: the entries' sizes, over 2^*e.
+// *low: with the digits that fall off taken as independent and uniform, an entry of
+// `dirs` such sums is off by 4 standard deviations at most (1 in 16000; the joins'
+// rounding and that of the values included).  Where the sum of the sizes of its terms,
+// in units of 2^*e and the power of two of the element's largest value, is *low, that
+// is `allow` 2^-53 of it.
 template <class M, class W>
-static bool fx_digits(int Nq, M mat, bool zero_rows, W word, int *q) {
+static bool fx_digits(int Nq, M mat, bool zero_rows, int dirs, double allow, W word, double *s,
+                      int *q, float *low) {
   double big = 0.0;
   for (int i = 0; i < Nq; ++i)
     for (int m = 0; m < Nq; ++m) big = std::fmax(big, std::fabs(mat(i, m).h));
-  int e = 0;
-  std::frexp(big, &e);  // big < 2^e
-  *q = 58 - e;
-  int64_t Ki[kMaxNq][kMaxNq];
-  for (int i = 0; i < Nq; ++i) {
-    int64_t rest = 0;
-    for (int m = 0; m < Nq; ++m) {
-      const DD v = mat(i, m);
-      const double hi = std::ldexp(v.h, *q), n = std::rint(hi);
-      Ki[i][m] = (int64_t)n + (int64_t)std::rint((hi - n) + std::ldexp(v.l, *q));
-      if (m != i) rest += Ki[i][m];
-    }
-    if (zero_rows) Ki[i][i] = -rest;
-  }
+  int64_t Ki[kMaxNq][kMaxNq] = {};
   int64_t bias = 0;
   for (int d = 0; d < kFxDigits; ++d) bias += (int64_t)512 << (10 * d);
   auto digit = [&](int i, int m, int d) {
@@ -148,28 +154,66 @@ static bool fx_digits(int Nq, M mat, bool zero_rows, W word, int *q) {
   // the largest sum an accumulator can meet: digits of a value up to 257
   // (the first) or 512 in magnitude, products a + b = o of one row; beyond
   // kFxMaxNq those of digits 2 and 3 have an accumulator of their own (o >= 3)
-  for (int o = 0; o < kFxDigits; ++o)
-    for (int i = 0; i < Nq; ++i) {
-      int64_t s[2] = {0, 0};
-      for (int a = 0; a <= o; ++a)
-        for (int m = 0; m < Nq; ++m)
-          s[Nq > kFxMaxNq && o >= 3 && (a == 2 || a == 3)] +=
-              (a ? 512 : 257) * std::abs(digit(i, m, o - a));
-      const int64_t most = o == kFxDigits - 1 ? 1 << 23 : 1 << 22;
-      if (s[0] > most || s[1] > most) return false;
-    }
-  auto half_bits = [](int v) -> uint32_t {  // |v| <= 512
-    if (v == 0) return 0;
-    const uint32_t sign = v < 0 ? 0x8000u : 0u, a = (uint32_t)(v < 0 ? -v : v);
-    int p = 31;
-    while (!(a >> p)) --p;
-    return sign | ((uint32_t)(p + 15) << 10) | ((a << (10 - p)) & 0x3ffu);
+  auto fits = [&] {
+    for (int o = 0; o < kFxDigits; ++o)
+      for (int i = 0; i < Nq; ++i) {
+        int64_t t[2] = {0, 0};
+        for (int a = 0; a <= o; ++a)
+          for (int m = 0; m < Nq; ++m)
+            t[Nq > kFxMaxNq && o >= 3 && (a == 2 || a == 3)] +=
+                (a ? 512 : 257) * std::abs(digit(i, m, o - a));
+        // the last order counts by two, but for degrees 2 and 3
+        const int64_t most = o == kFxDigits - 1 && Nq >= kFxMinNq ? 1 << 23 : 1 << 22;
+        if (t[0] > most || t[1] > most) return false;
+      }
+    return true;
   };
-  for (int d = 0; d < kFxDigits; ++d)
+  double scale = 0.0;
+  bool ok = false;
+  for (int step = 0; step < 96 && !ok; ++step) {
+    scale = std::ldexp(511.0 * (1.0 - step / 128.0), 50) / big;
+    for (int i = 0; i < Nq; ++i) {
+      int64_t rest = 0;
+      for (int m = 0; m < Nq; ++m) {
+        const DD v = mat(i, m) * DD(scale);
+        const double n = std::rint(v.h);
+        Ki[i][m] = (int64_t)n + (int64_t)std::rint((v.h - n) + v.l);
+        if (m != i) rest += Ki[i][m];
+      }
+      if (zero_rows) Ki[i][i] = -rest;
+    }
+    ok = fits();
+  }
+  if (!ok) return false;
+  *q = std::ilogb(scale);
+  *s = std::ldexp(scale, -*q);
+  // variance of one sum in units of 2^60 of the integer products: the products a + b = 6
+  // (digits uniform in +-512: 2^18 / 3) at 2^-20 each, the last places of the value and
+  // of the matrix, the join (1/12)
+  double var = 0.0;
+  for (int i = 0; i < Nq; ++i) {
+    double d = 0.0, v = 0.0;
+    for (int m = 0; m < Nq; ++m) {
+      for (int b = 1; b < kFxDigits; ++b) d += (double)digit(i, m, b) * digit(i, m, b);
+      v += std::ldexp((double)Ki[i][m], -60) * std::ldexp((double)Ki[i][m], -60);
+    }
+    var = std::fmax(var, d * std::ldexp(1.0, 18 - 40) / 3 + v / 12);
+  }
+  const double sigma = std::sqrt(dirs * (var + 1.0 / 12 + 0.01 * Nq));
+  int e = 0;
+  std::frexp(big, &e);  // big < 2^e
+  // 4 sigma 2^60 / scale in units of the value's 2^-57, against allow 2^-53 low 2^e
+  *low = (float)(4.0 * sigma * std::ldexp(1.0, 60 - 57 + 53 - e) / (allow * scale));
+  for (int d = 0; d <= kFxDigits; ++d)
     for (int i = 0; i < Nq; ++i)
-      for (int m = 0; m < Nq; m += 2)
-        word(d, i, m,
-             half_bits(digit(i, m, d)) | (m + 1 < Nq ? half_bits(digit(i, m + 1, d)) << 16 : 0u));
+      for (int m = 0; m < Nq; m += 2) {
+        auto bits = [&](int mm) -> uint32_t {
+          if (mm >= Nq) return 0;
+          return half_bits(d < kFxDigits ? (double)digit(i, mm, d)
+                                         : std::ldexp(std::fabs(mat(i, mm).h), -e));
+        };
+        word(d, i, m, bits(m) | bits(m + 1) << 16);
+      }
   return true;
 }
 
@@ -178,8 +222,11 @@ static bool fx_digits(int Nq, M mat, bool zero_rows, W word, int *q) {
 // nodes x, as gll_tables): a 58-bit entry holds more than a double, and an
 // error common to every element would shift the operator's low modes
 // coherently.  Also the weights' products of the affine kernel.
-static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t,
-                     FxGeoTab *tg, FxTab16 *t16, FxTab4 *t4) {
+static bool fx_table(int N, const double *x0, double h, double lambda, OpTab<double> *tab) {
+  FxTab *t = &tab->fx;
+  FxGeoTab *tg = &tab->fxg;
+  FxTab16 *t16 = &tab->fx16;
+  FxTab4 *t4 = &tab->fx4;
   const int Nq = N + 1;
   DD x[kMaxNq], w[kMaxNq], D[kMaxNq][kMaxNq], Kh[kMaxNq][kMaxNq];
   auto legendre = [&](DD z, DD *pn, DD *pm) {  // P_N, P_{N-1}
@@ -225,56 +272,91 @@ static bool fx_table(int N, const double *x0, double h, double lambda, FxTab *t,
       Kh[i][m] = s / w[i];
     }
   const DD g(0.5 * h), ml = DD(lambda) * g * g * g;
+  // (2 Nq + 4) 2^-53 of the sum of an entry's terms: the bound of the FP64 sums
+  const double allow = 2.0 * Nq + 4.0;
+  auto kh = [&](int i, int m) { return Kh[i][m]; };
+  double s = 1.0;
+  auto scaled_kh = [&] {
+    for (int i = 0; i < Nq; ++i)
+      for (int m = 0; m < Nq; ++m) tab->kh[i * Nq + m] = (Kh[i][m] * DD(s)).h;
+  };
   if (Nq > kFxMaxNq) {
     auto word = [&](int b, int i, int m, uint32_t bits) {
-      t16->w[b][(i % 8) * 4 + m % 8 / 2][i / 8 + 2 * (m / 8)] = bits;
+      (b < kFxDigits ? t16->w[b] : t16->a)[(i % 8) * 4 + m % 8 / 2][i / 8 + 2 * (m / 8)] = bits;
     };
-    if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, word, &t16->q)) return false;
+    if (!fx_digits(Nq, kh, true, 3, allow, word, &s, &t16->q, &t16->low)) return false;
+    scaled_kh();
     for (int k = 0; k < Nq; ++k) t16->w1[k] = w[k].h;
     for (int lane = 0; lane < 32; ++lane)
       for (int q = 0; q < 8; ++q) {
         const int j = (lane >> 2) + 8 * (q >> 2), i = 2 * (lane & 3) + 8 * ((q >> 1) & 1) + (q & 1);
         if (i >= Nq || j >= Nq) continue;
-        t16->wg[lane * 8 + q] = (w[i] * w[j] * g).h;
+        t16->wg[lane * 8 + q] = (w[i] * w[j] * g / DD(s)).h;
         t16->wm[lane * 8 + q] = (w[i] * w[j] * ml).h;
       }
     return true;
   }
   if (Nq < kFxMinNq) {
-    // every order in one accumulator counting by one: at most 0.23 of 2^22 with these
-    // matrices' digits, the check below allows twice that for the last
     auto word = [&](int b, int i, int m, uint32_t bits) {
+      if (b == kFxDigits)
+        for (int g4 = 0; g4 < 2; ++g4)
+          for (int th = 0; th < 2; ++th) t4->a[(4 * g4 + i) * 4 + 2 * th + m / 2] = bits;
       for (int x = 0; x < kFxDigits / 2; ++x)
         for (int od = 0; od < 2; ++od)
           for (int th = 0; th < 2; ++th)
             if (2 * x + od - th == b) t4->w[x][(4 * od + i) * 4 + 2 * th + m / 2] = bits;
     };
-    if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, word, &t4->q)) return false;
+    if (!fx_digits(Nq, kh, true, 3, allow, word, &s, &t4->q, &t4->low)) return false;
+    scaled_kh();
     for (int lane = 0; lane < 32; ++lane)
       for (int hf = 0; hf < 2; ++hf) {
         const int g4 = lane >> 2, t = lane & 3;
         const int i = 2 * (t & 1) + hf, j = g4 & 3, k = 2 * (g4 >> 2) + (t >> 1);
         if (i >= Nq || j >= Nq || k >= Nq) continue;
         const DD w3 = w[i] * w[j] * w[k];
-        t4->wg[lane * 2 + hf] = (w3 * g).h;
+        t4->wg[lane * 2 + hf] = (w3 * g / DD(s)).h;
         t4->wm[lane * 2 + hf] = (w3 * ml).h;
       }
     return true;
   }
-  auto words = [](uint32_t (*to)[32]) {
-    return [to](int b, int i, int m, uint32_t bits) { to[b][i * 4 + m / 2] = bits; };
+  auto words = [](uint32_t (*to)[32], uint32_t *sizes) {
+    return [to, sizes](int b, int i, int m, uint32_t bits) {
+      (b < kFxDigits ? to[b] : sizes)[i * 4 + m / 2] = bits;
+    };
   };
-  if (!fx_digits(Nq, [&](int i, int m) { return Kh[i][m]; }, true, words(t->w), &t->q) ||
-      !fx_digits(Nq, [&](int i, int m) { return D[i][m]; }, true, words(tg->d), &tg->qd) ||
-      !fx_digits(Nq, [&](int i, int m) { return D[m][i]; }, false, words(tg->dt), &tg->qdt))
+  auto M = [&](int i, int m) { return D[m][i] * DD(std::ldexp(1.0, tg->p[i] - tg->p[m])); };
+  // the weights' powers of two, by rounding down or to the nearest, whichever leaves
+  // P^-1 D^T P the smaller largest entry (7.5, 10.5, 14 at degrees 5, 6, 7; else 14, 20, 26)
+  auto powers = [&](double up) {
+    double big = 0.0;
+    for (int i = 0; i < Nq; ++i) tg->p[i] = -(int)std::floor(std::log2(w[i].h) + up);
+    for (int i = 0; i < Nq; ++i)
+      for (int m = 0; m < Nq; ++m) big = std::fmax(big, std::fabs(M(i, m).h));
+    return big;
+  };
+  powers(powers(0.5) < powers(0.0) ? 0.5 : 0.0);
+  double sd, sdt;
+  if (!fx_digits(Nq, kh, true, 3, allow, words(t->w, t->a), &s, &t->q, &t->low) ||
+      !fx_digits(Nq, [&](int i, int m) { return D[i][m]; }, true, 1, Nq + 2.0,
+                 words(tg->d, tg->da), &sd, &tg->qd, &tg->lowd) ||
+      !fx_digits(Nq, M, false, 3, Nq + 2.0,
+                 words(tg->dt, tg->dta), &sdt, &tg->qdt, &tg->lowdt))
     return false;
+  scaled_kh();
+  for (int i = 0; i < Nq; ++i)
+    for (int m = 0; m < Nq; ++m) {
+      tg->sD[i * Nq + m] = (D[i][m] * DD(sd)).h;
+      tg->D[i * Nq + m] = D[i][m].h;
+    }
+  tg->invd = 1.0 / sd;
+  tg->inv = (DD(1.0) / (DD(sd) * DD(sdt))).h;
   for (int k = 0; k < Nq; ++k)
     for (int lane = 0; lane < 32; ++lane)
       for (int hf = 0; hf < 2; ++hf) {
         const int i = 2 * (lane & 3) + hf, j = lane >> 2;
         if (i >= Nq || j >= Nq) continue;
         const DD w3 = w[i] * w[j] * w[k];
-        t->wg[(k * 32 + lane) * 2 + hf] = (w3 * g).h;
+        t->wg[(k * 32 + lane) * 2 + hf] = (w3 * g / DD(s)).h;
         t->wm[(k * 32 + lane) * 2 + hf] = (w3 * ml).h;
       }
   return true;
@@ -418,7 +500,7 @@ int bs_problem_create(const bs_map *map, double h, double lambda, const double *
         split(o, tabff.Eoh[a * hq + m], tabff.Eol[a * hq + m]);
       }
   }
-  if (Nq > 2 && !fx_table(N, x, h, lambda, &tab.fx, &tab.fxg, &tab.fx16, &tab.fx4)) {
+  if (Nq > 2 && !fx_table(N, x, h, lambda, &tab)) {
     free(p);
     return fail(BS_ERR_ARG, "bs_problem_create: digit tables of degree %d out of range", N);
   }

@@ -41,35 +41,51 @@ constexpr int kMaxNq = 16;  // degrees 1..15
 // Digit tables of the fixed-point contractions (bs_op_fx.cuh), degrees
 // kFxMinNq - 1 .. kFxMaxNq - 1: w[b][lane] = digit b of Kh[g][2t] and
 // Kh[g][2t + 1] (g = lane / 4, t = lane % 4; Kh = W^-1 K, zero past Nq) as a
-// pair of halves; Kh = sum_b digit_b 2^(10 (5 - b)) 2^-q.
+// pair of halves; s 2^q Kh = sum_b digit_b 2^(10 (5 - b)), 1 <= s < 2, the largest
+// entry near 511 2^50.
 constexpr int kFxDigits = 6;  // digits per operand, 10 bits each
 constexpr int kFxMinNq = 5, kFxMaxNq = 8;
-// wg, wm [k][lane][h]: (h/2) w_i w_j w_k and lambda (h/2)^3 w_i w_j w_k of the
+// a: |Kh|, in the layout of a digit, scaled below 1; low: the sum of a node's terms in
+// those units (the element's largest exponent as 1) below which its digits may be off
+// by more than the FP64 sums' bound.
+// wg, wm [k][lane][h]: (h/2) w_i w_j w_k / s and lambda (h/2)^3 w_i w_j w_k of the
 // node (2t + h, g, k), rounded once.
 struct __align__(16) FxTab {
-  uint32_t w[kFxDigits][32];
+  uint32_t w[kFxDigits][32], a[32];
   double wg[kFxMaxNq * 64], wm[kFxMaxNq * 64];
+  float low;
   int q;
 };
 // Degrees 8..15 (bs_op_fx16.cuh): w[b][lane] = digit b of Kh[g][2t ..], Kh[g + 8]
 // [2t ..], Kh[g][2t + 8 ..], Kh[g + 8][2t + 8 ..] as pairs of halves; wg, wm
-// [lane][q]: (h/2) w_i w_j and lambda (h/2)^3 w_i w_j of a lane's eight nodes of a
+// [lane][q]: (h/2) w_i w_j / s and lambda (h/2)^3 w_i w_j of a lane's eight nodes of a
 // layer; w1: the weights.
 struct __align__(16) FxTab16 {
-  uint32_t w[kFxDigits][32][4];
+  uint32_t w[kFxDigits][32][4], a[32][4];
   double wg[256], wm[256], w1[kMaxNq];
+  float low;
   int q;
 };
 // Degrees 2 and 3 (bs_op_fx4.cuh): w[x][lane] = digit 2x + g / 4 - t / 2 (none: zero) of
-// Kh[g % 4][2 (t % 2) ..]; wg, wm [lane][h] as FxTab's, of a lane's two nodes.
+// Kh[g % 4][2 (t % 2) ..]; a the same of |Kh|; wg, wm [lane][h] as FxTab's, of a lane's
+// two nodes.
 struct __align__(16) FxTab4 {
-  uint32_t w[kFxDigits / 2][32];
+  uint32_t w[kFxDigits / 2][32], a[32];
   double wg[64], wm[64];
+  float low;
   int q;
 };
-// The same digits of the derivative matrix D (d, scale qd) and of D^T (dt, qdt).
+// The same digits of the derivative matrix D (d, scale sd 2^qd) and of P^-1 D^T P (dt,
+// sdt 2^qdt), where P = diag(2^-p_i) are the quadrature weights' powers of two, their
+// sizes da, dta and the least sums lowd, lowdt of a gradient component's and of an
+// entry's terms; sD = sd D and D for the lines that take FP64 sums; invd = 1 / sd, inv =
+// 1 / (sd sdt).
 struct FxGeoTab {
-  uint32_t d[kFxDigits][32], dt[kFxDigits][32];
+  uint32_t d[kFxDigits][32], dt[kFxDigits][32], da[32], dta[32];
+  double sD[kFxMaxNq * kFxMaxNq], D[kFxMaxNq * kFxMaxNq];
+  double invd, inv;
+  int p[kFxMaxNq];
+  float lowd, lowdt;
   int qd, qdt;
 };
 
@@ -87,6 +103,7 @@ struct OpTab {
   FxGeoTab fxg;
   FxTab16 fx16;
   FxTab4 fx4;
+  double kh[kMaxNq * kMaxNq];  // s Kh, for the nodes that take FP64 sums
   int64_t ne, ng;  // the problem's E and N_G (index checks of the checked build)
 };
 

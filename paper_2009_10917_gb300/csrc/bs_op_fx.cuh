@@ -8,27 +8,37 @@
 // are integer arithmetic (an error-free splitting of the kind of Ozaki,
 // Ogita, Oishi & Rump, Numer. Algorithms 59, 2012):
 //  - an element's values are taken as 58-bit integers relative to its largest
-//    exponent and cut into six signed 10-bit digits; so is Kh, on the host
-//    (FxTab);
+//    exponent and cut into six signed 10-bit digits; so is Kh times a scale
+//    that puts its largest entry near 511 2^50, on the host (FxTab);
 //  - a digit fits a half exactly, and mma.sync m16n8k16 sums the products of
 //    equal weight (order o = a + b, 48 at most) into an FP32 accumulator that
 //    starts at 1.5 * 2^23: with the actual digits of Kh every partial sum is
-//    an integer in [2^23, 2^24) (below 0.95 of the 2^22 either way for
-//    degrees up to 7, checked where the table is made), so nothing rounds and
-//    the accumulator's bits ARE the integer: no conversion instructions,
-//    which share the FP64 pipe.  Order 5, the last, would reach 1.22 and
-//    starts at 1.5 * 2^24 instead, counting by two; its low ten bits are
-//    dropped anyway;
+//    an integer in [2^23, 2^24) (the host takes the largest scale for which
+//    that holds), so nothing rounds and the accumulator's bits ARE the
+//    integer: no conversion instructions, which share the FP64 pipe.  Order 5,
+//    the last, would reach 1.3 times the range and starts at 1.5 * 2^24
+//    instead, counting by two; its low ten bits are dropped anyway;
 //  - orders 0..5 are joined into one 64-bit integer per node, the three
 //    directions summed there, and only then is there a double, put together
 //    by integer operations: two FP64 operations per node (the weighted sum
 //    and the mass term), three with a coefficient.
-// Dropped: u below 2^-58 of the element's largest power of two, orders >= 6
-// and the last ten bits, together about 2^-57 of the element's max|u| times
-// sum|Kh| per node.  The FP64 forms round relative to each line's own values,
-// up to (2 Nq + 4) 2^-53 of sum|Kh||u|; an element in which some column along
-// t (so some line of every node) stays more than 2^-8 below the element's
-// largest value therefore takes the FP64 sums.
+// Dropped: u below 2^-58 of the element's largest power of two U, orders >= 6
+// and the last ten bits, together about 2^-57.7 of U times Kh's largest power
+// of two per node (standard deviation, N = 7), wherever the node is.  FP64
+// sums are off by up to (2 Nq + 4) 2^-53 of the sum T of the sizes of the
+// node's own terms, so the digits serve a node only where T is large enough
+// that four deviations stay within that (FxTab::low).  T is bounded from below
+// by its part along r, and where that is not enough by those along r and s,
+// from |u| and |Kh| in half precision on the tensor cores (2% of the kernel's
+// time: the halves are the lane's own fragments).  The other nodes, and all of
+// an element whose largest value is not finite or outside [2^-900, 2^900], take
+// FP64 sums from shared memory, compacted to full warps.  Inside the solvers,
+// where A p goes on into sums and updates of the vectors' size, four
+// deviations may be N - 1 times as large: the FP64 sums with tables made in
+// double are themselves off by N - 1 times the bound and more at small entries
+// (6.6 at N = 7, 53 at N = 15, the even-odd form 57 at N = 7).  CG's search
+// directions have a few per cent of nodes below the line without that (N = 7:
+// half of the elements, 8% of an iteration), almost none with it.
 //
 // One or two warps per element, each with its own layers k (and planes j of
 // the t direction).  With g = lane / 4 and t = lane % 4, a lane owns the nodes
@@ -43,16 +53,16 @@
 // the tensor pipe is not what bounds it, and the accumulators are wanted in
 // registers at once.
 //
-// Measured (N = 7 on 36^3, 23.9M local nodes): A_L Z p 176 us, the even-odd
+// Measured (N = 7 on 36^3, 23.9M local nodes): A_L Z p 182 us, the even-odd
 // FP64 kernel 1047 us; HBM alone would allow 60 us.  What bounds it now is
 // spread out: issue slots 61%, integer pipe 55%, FP64 pipe 46%, L1 65%, HBM 26%.
 // Conversions by two FP64 additions per node (instead of fx_double) and the
 // weights multiplied node by node took 312 us with the FP64 pipe at 82%.
-// Error against extended precision on uniform inputs 1.4e-16 normwise (the
-// even-odd kernel 8.3e-16), after 64 CG iterations 1.7e-15 (2.8e-14).
-//
-// The FP64 sums (fx_direct) also serve an element whose largest value is not
-// finite or outside [2^-900, 2^900].
+// Where every node takes FP64 sums (36^3, A_L u): 1177 us, the direct FP64
+// kernel 1352; where a third to two thirds do (a layer exp(-12 t), values spread
+// over e^+-9), digits and sums both, 1190 to 1310 us.
+// Error against extended precision on uniform inputs 6e-17 normwise (the
+// even-odd kernel 8.3e-16), entry by entry at most 0.1 of the bound.
 #pragma once
 
 #include <type_traits>
@@ -61,7 +71,6 @@
 
 namespace bs {
 
-constexpr int kFxRange = 8;          // log2 of the column range the digits serve
 constexpr uint32_t kFxMagicBits = 0x4B400000u;   // 1.5 * 2^23: counts by one
 constexpr uint32_t kFxMagic2Bits = 0x4BC00000u;  // 1.5 * 2^24: counts by two
 
@@ -135,6 +144,39 @@ __device__ __forceinline__ void fx_ldsm2t(uint32_t *r, uint32_t addr) {
                : "=r"(r[0]), "=r"(r[1])
                : "r"(addr)
                : "memory");
+}
+
+__device__ __forceinline__ void fx_ldsm1t(uint32_t *r, uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x1.trans.shared.b16 {%0}, [%1];\n"
+               : "=r"(r[0])
+               : "r"(addr)
+               : "memory");
+}
+__device__ __forceinline__ void fx_mma8(float *c, uint32_t a0, uint32_t a1, uint32_t b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, "
+      "{%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(b0));
+}
+// The transpose of an 8 x 8 matrix of halves held as a fragment.
+__device__ __forceinline__ uint32_t fx_trans(uint32_t a) {
+  uint32_t d;
+  asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(d) : "r"(a));
+  return d;
+}
+
+// High word of |x|: zero below 2^-1042 too.
+__device__ __forceinline__ uint32_t fx_size(double x) {
+  return (uint32_t)__double2hiint(x) & 0x7fffffffu;
+}
+// |a|, |b| as a pair of halves over 2^emax's power of two (the largest value in [1, 2)),
+// cut off, never rounded up; nothing below 2^-14.
+// pa, pb: powers of two the values count times.
+__device__ __forceinline__ uint32_t fx_sizes2(double a, double b, int emax, int pa = 0,
+                                              int pb = 0) {
+  const uint32_t x = (uint32_t)__viaddmax_s32((int)fx_size(a), (15 - emax + pa) << 20, 0);
+  const uint32_t y = (uint32_t)__viaddmax_s32((int)fx_size(b), (15 - emax + pb) << 20, 0);
+  return x >> 10 | (y << 6 & 0xffff0000u);
 }
 
 // x as an integer of 58 bits in units of 2^(emax - 1080), rounded to nearest,
@@ -271,11 +313,11 @@ struct FxMul {
   }
 };
 
-// The digits of a lane's values of layer k into the planes.
+// The digits of a lane's values of layer k (times 2^pa, 2^pb) into the planes.
 template <int NQ>
 __device__ __forceinline__ void fx_store_digits(unsigned char *dig, int k, int g, int t, double a,
-                                                double b, int emax) {
-  const uint64_t x = fx_fixed(a, emax), y = fx_fixed(b, emax);
+                                                double b, int emax, int pa = 0, int pb = 0) {
+  const uint64_t x = fx_fixed(a, emax - pa), y = fx_fixed(b, emax - pb);
   uint32_t *p = reinterpret_cast<uint32_t *>(dig) + (k * 8 + (g ^ k)) * 4 + t;
   constexpr int PW = FxShape<NQ>::PLANE / 4;
   p[0 * PW] = fx_digit2<0>(x, y);
@@ -296,49 +338,110 @@ __device__ __forceinline__ ulonglong2 *fx_xch(unsigned char *xch, int j, int k, 
   return reinterpret_cast<ulonglong2 *>(xch + (j * NQ + kk) * 64 + t * 16);
 }
 
-// High word of |x|, or 1 for a value whose high word is zero but which is not.
-__device__ __forceinline__ uint32_t fx_size(double x) {
-  return ((uint32_t)__double2hiint(x) & 0x7fffffffu) | min((uint32_t)__double2loint(x), 1u);
-}
-
-// From the largest values of a lane's two columns over its warp's layers: the
-// element's largest exponent, and whether its values are beyond the digits
-// (col: 256 bytes per warp; two barriers' worth of a gap between uses).
-template <int WPE, class Sync>
-__device__ __forceinline__ int fx_range(uint32_t big0, uint32_t big1, uint32_t *col, int warp,
-                                        int lane, Sync sync, bool *direct) {
+// The element's largest exponent from the largest value of a lane (a high word of
+// fx_size) and the low words of its values or'ed (`rest`: asked for only where all high
+// words are zero); *zero: all values are.  col: a word per warp, and WPE further on
+// another for that rare case.
+template <int WPE, class Sync, class Rest>
+__device__ __forceinline__ int fx_emax(uint32_t big, Rest rest, uint32_t *col, int warp, int lane,
+                                       Sync sync, bool *zero) {
+  big = __reduce_max_sync(0xffffffffu, big);
   if (WPE > 1) {
-    reinterpret_cast<uint2 *>(col)[warp * 32 + lane] = make_uint2(big0, big1);
+    if (lane == 0) col[warp] = big;
     sync();
 #pragma unroll
-    for (int w = 0; w < WPE; ++w) {
-      const uint2 c = reinterpret_cast<const uint2 *>(col)[w * 32 + lane];
-      big0 = max(big0, c.x);
-      big1 = max(big1, c.y);
-    }
+    for (int w = 0; w < WPE; ++w) big = max(big, col[w]);
   }
-  const uint32_t big = __reduce_max_sync(0xffffffffu, max(big0, big1));
-  const uint32_t low = __reduce_min_sync(  // columns of zeros left out
-      0xffffffffu, min(big0 ? big0 : 0x7fffffffu, big1 ? big1 : 0x7fffffffu));
-  const int emax = big ? (int)(big >> 20) : 1023;  // an element of zeros has zero digits
-  *direct = emax < 123 || emax > 1923 ||           // outside [2^-900, 2^900]
-            (big && emax - (int)(low >> 20) > kFxRange);
-  return emax;
+  *zero = false;
+  if (big == 0) {  // the same for all warps of the element
+    bool some = __any_sync(0xffffffffu, rest() != 0);
+    if (WPE > 1) {
+      if (lane == 0) col[WPE + warp] = some;
+      sync();
+#pragma unroll
+      for (int w = 0; w < WPE; ++w) some = some || col[WPE + w];
+    }
+    *zero = !some;
+    return some ? 0 : 1023;
+  }
+  return (int)(big >> 20);
+}
+// Beyond the digits: not finite, or outside [2^-900, 2^900].
+__device__ __forceinline__ bool fx_far(int emax) { return emax < 123 || emax > 1923; }
+
+// The sums of the sizes of the terms at the nodes (2t, g), (2t + 1, g) of two layers (h0,
+// h1: their sizes as of fx_sizes2; a: the matrix's), s[0], s[1] of the first layer, s[2],
+// s[3] of the second: those along r, and added to them those along s.
+__device__ __forceinline__ void fx_terms_r(float *s, uint32_t a, uint32_t h0, uint32_t h1) {
+#pragma unroll
+  for (int n = 0; n < 4; ++n) s[n] = 0.f;
+  fx_mma8(s, h0, h1, a);  // layers x matrix
+}
+__device__ __forceinline__ void fx_terms_s(float *s, uint32_t a, uint32_t h0, uint32_t h1) {
+  fx_mma(s, a, 0u, 0u, a, fx_trans(h0), fx_trans(h1));  // matrix x layers
 }
 
-// Direct FP64 sums of one element (values in x[], node order as in memory)
-// for the node (i, j, k): (W^-1 D^T W D applied along r, s and t).
+// The FP64 sums of one node (i, j, k) of an element with values x[] in memory order:
+// the scaled W^-1 D^T W D (OpTab::kh) along r, s and t.
 template <int NQ>
-__device__ __noinline__ double fx_direct(const double *x, const OpTab<double> *tab, int i, int j,
-                                         int k) {
-  const double *K = tab->K, *w = tab->w;
+__device__ __noinline__ double fx_direct(const double *x, const double *__restrict__ kh, int i,
+                                         int j, int k) {
   double ar = 0.0, as = 0.0, at = 0.0;
+#pragma unroll(NQ <= 8 ? NQ : 4)
   for (int m = 0; m < NQ; ++m) {
-    ar = fma(K[i * NQ + m], x[m + NQ * (j + NQ * k)], ar);
-    as = fma(K[j * NQ + m], x[i + NQ * (m + NQ * k)], as);
-    at = fma(K[k * NQ + m], x[i + NQ * (j + NQ * m)], at);
+    ar = fma(kh[i * NQ + m], x[m + NQ * (j + NQ * k)], ar);
+    as = fma(kh[j * NQ + m], x[i + NQ * (m + NQ * k)], as);
+    at = fma(kh[k * NQ + m], x[i + NQ * (j + NQ * m)], at);
   }
-  return (ar / w[i] + as / w[j]) + at / w[k];
+  return (ar + as) + at;
+}
+// The same of a warp's list of `count` nodes, result(n, sum) on one lane each.  An FP64
+// instruction takes the pipe 16 clocks however few lanes it serves, and a list is mostly
+// short: up to 16 nodes go eight at a time, a lane for each of their three lines (at N = 7
+// ten instructions for eight nodes instead of 26 for 32).
+template <int NQ, class Result>
+__device__ __forceinline__ void fx_direct_list(const double *x, const double *__restrict__ kh,
+                                               const uint16_t *list, int count, int lane,
+                                               Result result) {
+  if (count > 16) {
+    for (int q = lane; q < count; q += 32) {
+      const int n = list[q];
+      result(n, fx_direct<NQ>(x, kh, n % NQ, n / NQ % NQ, n / (NQ * NQ)));
+    }
+    return;
+  }
+  for (int q0 = 0; q0 < count; q0 += 8) {
+    const int q = q0 + (lane >> 2), d = lane & 3;
+    const int n = list[q < count ? q : q0], i = n % NQ, j = n / NQ % NQ, k = n / (NQ * NQ);
+    const int row = d == 0 ? i : (d == 1 ? j : k);
+    const int step = d == 0 ? 1 : (d == 1 ? NQ : NQ * NQ);
+    const double *line = x + (n - row * step), *c = kh + row * NQ;
+    double v = 0.0;
+#pragma unroll(NQ <= 8 ? NQ : 4)
+    for (int m = 0; m < NQ; ++m) v = fma(c[m], line[m * step], v);
+    const double v1 = __shfl_down_sync(0xffffffffu, v, 1), v2 = __shfl_down_sync(0xffffffffu, v, 2);
+    if (d == 0 && q < count) result(n, (v + v1) + v2);
+  }
+}
+
+// What FxTab::low is multiplied by: 1 for one A p (no solver state), 1 / (N - 1) inside
+// the solvers.
+template <int NQ>
+__device__ __forceinline__ float fx_slack(const CgState *st) {
+  return st ? 1.f / (NQ - 2) : 1.f;
+}
+
+// The nodes whose bit b of `low` is set (b < n; node(b): the index in the element), one
+// lane after the other, into a warp's list; how many.
+template <class Node>
+__device__ __forceinline__ int fx_list(uint32_t low, int n, int lane, uint16_t *list, Node node) {
+  int count = 0;
+  for (int b = 0; b < n; ++b) {
+    const uint32_t m = __ballot_sync(0xffffffffu, (low >> b) & 1u);
+    if ((low >> b) & 1u) list[count + __popc(m & ((1u << lane) - 1u))] = (uint16_t)node(b);
+    count += __popc(m);
+  }
+  return count;
 }
 
 // out = A_L in on one element e, by the WPE warps that call it with their own
@@ -352,7 +455,7 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
                                            const OpTab<double> *__restrict__ tab,
                                            const double *__restrict__ coef,
                                            double *__restrict__ outG, Acc<double> &acc, int vec,
-                                           unsigned char *dig, Sync sync) {
+                                           float slack, unsigned char *dig, Sync sync) {
   static_assert(!FUSED || GATHER_IN, "the fused operator reads its input through the map");
   using S = FxShape<NQ>;
   constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2, D = kFxDigits, WPE = (NQ + L - 1) / L;
@@ -414,15 +517,57 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
       }
     }
   }
-  // ---- the largest exponent, and whether the digits serve
-  uint32_t big0 = 0, big1 = 0;
+  // ---- the largest exponent, and the nodes the digits do not serve: bit 2l + h
+  uint32_t big = 0, low = 0;
 #pragma unroll
-  for (int l = 0; l < L; ++l) {
-    big0 = max(big0, fx_size(u0[l]));
-    big1 = max(big1, fx_size(u1[l]));
+  for (int l = 0; l < L; ++l) big = max(big, max(fx_size(u0[l]), fx_size(u1[l])));
+  auto rest = [&] {
+    uint32_t r = 0;
+#pragma unroll
+    for (int l = 0; l < L; ++l) r |= (uint32_t)(__double2loint(u0[l]) | __double2loint(u1[l]));
+    return r;
+  };
+  const int warp = k0 / L;
+  bool zero;
+  const int emax = fx_emax<WPE>(big, rest, col, warp, lane, sync, &zero);
+  const bool far = fx_far(emax);
+  bool some = far;  // of the element's nodes
+  auto used = [&] {  // of the bits set in `low`, those of nodes whose results are used
+#pragma unroll
+    for (int n = 0; n < 2 * L; ++n) {
+      bool use = (n & 1 ? on1 : on0) && layer(n / 2);
+      if (GATHER_IN && use && (low >> n & 1u) && (n & 1 ? u1[n / 2] : u0[n / 2]) == 0.0) {
+        const int32_t id = __ldg(ids + base + n / 2 * NQ2 + (n & 1));
+        use = FUSED ? id != -1 : id >= 0;
+      }
+      if (!use) low &= ~(1u << n);
+    }
+  };
+  if (far) {
+    low = (1u << 2 * L) - 1u;
+    used();
+  } else {
+    const uint32_t ka = __ldg(&tab->fx.a[lane]);
+    const float least = zero ? 0.f : slack * tab->fx.low;  // zeros: the digits are exact
+    // the terms along r mostly suffice (they are the lane's own fragments)
+    float s[2 * L], m = INFINITY;
+    uint32_t h[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) h[l] = fx_sizes2(u0[l], u1[l], emax);
+#pragma unroll
+    for (int l = 0; l < L; l += 2) fx_terms_r(s + 2 * l, ka, h[l], h[l + 1]);
+#pragma unroll
+    for (int n = 0; n < 2 * L; ++n)
+      if ((n & 1 ? on1 : on0) && layer(n / 2)) m = fminf(m, s[n]);
+    if (__any_sync(0xffffffffu, m < least)) {
+#pragma unroll
+      for (int l = 0; l < L; l += 2) fx_terms_s(s + 2 * l, ka, h[l], h[l + 1]);
+#pragma unroll
+      for (int n = 0; n < 2 * L; ++n) low |= s[n] < least ? 1u << n : 0u;
+      used();
+      some = __any_sync(0xffffffffu, low);
+    }
   }
-  bool direct;
-  const int emax = fx_range<WPE>(big0, big1, col, k0 / L, lane, sync, &direct);
   const double ce = coef ? coef[e] : 1.0;
   auto store = [&](int l, double r0, double r1, int32_t i0, int32_t i1, double v0, double v1) {
     if (FUSED) {
@@ -432,7 +577,7 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
         } else if (id != -1) {
           const double v = plus_zero(r);
           __stcs(outG + (-2 - id), v);
-          acc.add(u, v);
+          if (!(low >> (2 * l + h) & 1u)) acc.add(u, v);
         }
       };
       if (on0) one(r0, i0, v0, 0);
@@ -444,7 +589,14 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
       if (on1) __stcs(out + base + l * NQ2 + 1, r1);
     }
   };
-  if (!direct) {
+  // the element's values in memory order, over the digits once those are done with
+  double *x = reinterpret_cast<double *>(dig);
+  auto keep = [&](int l) {
+    const int n = 2 * t + NQ * (g + NQ * (k0 + l));
+    if (on0) x[n] = u0[l];
+    if (on1) x[n + 1] = u1[l];
+  };
+  if (!far) {
 #pragma unroll
     for (int l = 0; l < L; ++l) {
       if (!layer(l)) break;
@@ -483,7 +635,17 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
         T1[l + h] = fx_join(s[2 * h + 1]);
       }
     }
+    if (WPE > 1 && lane == 0) col[2 * WPE + warp] = some;
     sync();
+    if (WPE > 1)
+#pragma unroll
+      for (int w = 0; w < WPE; ++w) some = some || col[2 * WPE + w];
+    // (ahead of the results with two warps an element, along with them with one: 2 us of
+    // 273 at Nq = 8, 4 of 279 at Nq = 5 the other way round)
+    if (WPE > 1 && some)
+#pragma unroll
+      for (int l = 0; l < L; ++l)
+        if (layer(l)) keep(l);
     // ---- results: w_i w_j w_k (c h/2 sum + lambda (h/2)^3 u), the weights'
     // products from tables; sum = T 2^60 2^-q 2^(emax - 1080)
     const int p2 = emax - 1020 - tab->fx.q;
@@ -504,6 +666,7 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
           d0 = ce * d0;
           d1 = ce * d1;
         }
+        if (WPE == 1 && some) keep(l);
         store(l, fma(wg.x, d0, wm.x * u0[l]), fma(wg.y, d1, wm.y * u1[l]),
               id0[GATHER_IN ? l : 0], id1[GATHER_IN ? l : 0], u0[l], u1[l]);
       }
@@ -512,37 +675,38 @@ __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__r
       results(std::true_type{});
     else
       results(std::false_type{});
-  } else {  // ---- the direct sums, from the element's values in memory order
-    double *x = reinterpret_cast<double *>(dig);
+  } else {
 #pragma unroll
-    for (int l = 0; l < L; ++l) {
-      if (!layer(l)) break;
-      if (on0) x[2 * t + NQ * (g + NQ * (k0 + l))] = u0[l];
-      if (on1) x[2 * t + 1 + NQ * (g + NQ * (k0 + l))] = u1[l];
-    }
-    sync();
-#pragma unroll 1
-    for (int l = 0; l < L; ++l) {
-      if (!layer(l)) break;
-      const int k = k0 + l;
-      double r[2] = {0.0, 0.0}, u[2] = {0.0, 0.0};
-      int32_t id[2] = {-1, -1};
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        if (!(h ? on1 : on0)) continue;
-        const int i = 2 * t + h;
-        u[h] = x[i + NQ * (g + NQ * k)];
-        const double d = fx_direct<NQ>(x, tab, i, g, k);
-        r[h] = fma(tab->fx.wg[(k * 32 + lane) * 2 + h], coef ? ce * d : d,
-                   tab->fx.wm[(k * 32 + lane) * 2 + h] * u[h]);
-        if (FUSED) {
-          id[h] = ids[base + l * NQ2 + h];
-          if (!chk(bs_pred_fused_entry(id[h], tab->ng), BS_CHK_OP_ENTRY)) id[h] = -1;
-        }
-      }
-      store(l, r[0], r[1], id[0], id[1], u[0], u[1]);
-    }
+    for (int l = 0; l < L; ++l)
+      if (layer(l)) keep(l);
   }
+  if (!some) return;
+  // ---- the FP64 sums of the nodes in `low`, over what the digits gave, 32 nodes of
+  // the warp's at a time
+  sync();  // the exchanged sums have been read
+  uint16_t *list = reinterpret_cast<uint16_t *>(xch) + k0 * NQ2;
+  const int count = fx_list(low, 2 * L, lane, list, [&](int b) {
+    return 2 * t + (b & 1) + NQ * (g + NQ * (k0 + (b >> 1)));
+  });
+  sync();
+  fx_direct_list<NQ>(x, tab->kh, list, count, lane, [&](int n, double d) {
+    const int i = n % NQ, j = n / NQ % NQ, k = n / NQ2;
+    const int own = (k * 32 + j * 4 + (i >> 1)) * 2 + (i & 1);  // the owner's table entry
+    const double u = x[n];
+    const double r = fma(tab->fx.wg[own], coef ? ce * d : d, tab->fx.wm[own] * u);
+    int32_t id = 0;
+    if (FUSED) {
+      id = ids[e * NP + n];
+      if (!chk(bs_pred_fused_entry(id, tab->ng), BS_CHK_OP_ENTRY)) id = -1;
+    }
+    if (id >= 0) {
+      __stcs(out + e * NP + n, r);
+    } else if (id != -1) {
+      const double v = plus_zero(r);
+      __stcs(outG + (-2 - id), v);
+      acc.add(u, v);
+    }
+  });
 }
 
 template <int NQ, bool GATHER_IN, bool FUSED>
@@ -561,7 +725,7 @@ __global__ void __launch_bounds__(FxShape<NQ>::THREADS, FxShape<NQ>::BLOCKS)
   if (e >= 0 && !chk(bs_pred_index(e, tab->ne), BS_CHK_OP_ENTRY)) e = -1;
   if (e >= 0)
     fx_element<NQ, S::L, GATHER_IN, FUSED>(e, (int)(threadIdx.x / 32) * S::L, ids, in, out, tab,
-                                           coef, outG, acc, vec, fx_smem, [] {
+                                           coef, outG, acc, vec, fx_slack<NQ>(st), fx_smem, [] {
                                              if (S::WPE == 1)
                                                __syncwarp();
                                              else

@@ -7,10 +7,10 @@
 // t = lane % 4): its digit words are the A fragment along r (rows j, Kh^T as B, two
 // tiles of eight columns), the transposed layer is the B fragment along s and
 // the transposed (k, i) plane the one along t, with Kh as A.  Orders 3..5 take
-// two accumulators, products of digits 2 and 3 in the second (with the actual
-// digits of Kh below 0.99 of the range; checked where the table is made).
-// Every warp has L layers (and planes j) of one element; the smallest of the
-// largest values is taken over the lines along r, which lie within a warp.
+// two accumulators, products of digits 2 and 3 in the second (Kh's scale is the
+// largest for which both hold; checked where the table is made).
+// Every warp has L layers (and planes j) of one element.  Nodes whose terms along r and s
+// are too small for the digits take FP64 sums, as in bs_op_fx.cuh.
 //
 #pragma once
 
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
   using S = FxShape16<NQ>;
   constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2, D = kFxDigits, L = S::L, WPE = S::WPE;
   extern __shared__ __align__(128) unsigned char fx16_smem[];
-  __shared__ uint2 s_range[WPE];
+  __shared__ uint32_t s_col[3 * WPE];
   if (cg_halted(st)) return;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, warp = threadIdx.x >> 5;
   const int k0 = warp * L;
@@ -164,32 +164,61 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
           u[l][q] = on(q) && layer(l) ? __ldcs(in + base + l * NQ2 + at(q)) : 0.0;
         }
       }
-    // ---- the largest exponent, and the smallest of the lines' largest values
-    uint32_t big = 0, low = 0x7fffffffu;
+    // ---- the largest exponent, and the nodes the digits do not serve: bit 8l + q
+    uint32_t big = 0, low = 0;
 #pragma unroll
     for (int l = 0; l < L; ++l)
 #pragma unroll
-      for (int jj = 0; jj < 2; ++jj) {
-        uint32_t m = 0;
+      for (int q = 0; q < 8; ++q) big = max(big, fx_size(u[l][q]));
+    auto rest = [&] {
+      uint32_t r = 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) m = max(m, fx_size(u[l][4 * jj + q]));
-        m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-        m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-        big = max(big, m);
-        low = min(low, m ? m : 0x7fffffffu);  // lines of zeros left out
+      for (int l = 0; l < L; ++l)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) r |= (uint32_t)__double2loint(u[l][q]);
+      return r;
+    };
+    bool zero;
+    const int emax =
+        fx_emax<WPE>(big, rest, s_col, warp, lane, [] { __syncthreads(); }, &zero);
+    const bool far = fx_far(emax);
+    const float least = zero ? 0.f : fx_slack<NQ>(st) * tab->fx16.low;  // zeros: the digits are exact
+    // the sums of the sizes of layer l's terms along r and s: each(q, sum)
+    auto terms = [&](int l, auto each) {
+      const uint4 ka = __ldg(reinterpret_cast<const uint4 *>(&tab->fx16.a[lane][0]));
+      uint32_t h[4];  // rows g, g + 8 of columns 2t, then of 2t + 8
+#pragma unroll
+      for (int q = 0; q < 8; q += 2) h[(q >> 2) + (q & 2)] = fx_sizes2(u[l][q], u[l][q + 1], emax);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        fx_mma(s, h[0], h[1], h[2], h[3], c ? ka.y : ka.x, c ? ka.w : ka.z);            // along r
+        fx_mma(s, ka.x, ka.y, ka.z, ka.w, fx_trans(h[2 * c]), fx_trans(h[2 * c + 1]));  // along s
+#pragma unroll
+        for (int n = 0; n < 4; ++n) each(4 * (n >> 1) + 2 * c + (n & 1), s[n]);
       }
-    big = __reduce_max_sync(0xffffffffu, big);
-    low = __reduce_min_sync(0xffffffffu, low);
-    if (lane == 0) s_range[warp] = make_uint2(big, low);
-    __syncthreads();
+    };
+    bool some = far;  // of the element's nodes
+    if (far) {
+      low = (1u << 8 * L) - 1u;
+    } else {
 #pragma unroll
-    for (int w = 0; w < WPE; ++w) {
-      big = max(big, s_range[w].x);
-      low = min(low, s_range[w].y);
+      for (int l = 0; l < L; ++l)
+        terms(l, [&](int q, float s) { low |= s < least ? 1u << (8 * l + q) : 0u; });
     }
-    const int emax = big ? (int)(big >> 20) : 1023;  // an element of zeros has zero digits
-    const bool direct = emax < 123 || emax > 1923 ||  // outside [2^-900, 2^900]
-                        (big && emax - (int)(low >> 20) > kFxRange);
+    if (__any_sync(0xffffffffu, low)) {
+#pragma unroll
+      for (int b = 0; b < 8 * L; ++b) {  // those whose results are used
+        const int l = b >> 3, q = b & 7;
+        bool use = on(q) && layer(l);
+        if (GATHER_IN && use && (low >> b & 1u) && u[l][q] == 0.0) {
+          const int32_t v = __ldg(ids + base + l * NQ2 + at(q));
+          use = FUSED ? v != -1 : v >= 0;
+        }
+        if (!use) low &= ~(1u << b);
+      }
+      some = far || __any_sync(0xffffffffu, low);
+    }
     const double ce = coef ? coef[e] : 1.0;
     auto store = [&](int l, int q, double r, int32_t i, double v) {
       if (!on(q)) return;
@@ -198,10 +227,19 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
       } else if (i != -1) {
         const double p = plus_zero(r);
         __stcs(outG + (-2 - i), p);
-        acc.add(v, p);
+        if (!(low >> (8 * l + q) & 1u)) acc.add(v, p);
       }
     };
-    if (!direct) {
+    // the element's values in memory order, over the digits once those are done with
+    double *x = reinterpret_cast<double *>(dig);
+    auto keep = [&] {
+#pragma unroll
+      for (int l = 0; l < L; ++l)
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (on(q) && layer(l)) x[(k0 + l) * NQ2 + at(q)] = u[l][q];
+    };
+    if (!far) {
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         if (!layer(l)) break;
@@ -270,7 +308,11 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
           }
         }
       }
+      if (lane == 0) s_col[2 * WPE + warp] = some;
       __syncthreads();
+#pragma unroll
+      for (int w = 0; w < WPE; ++w) some = some || s_col[2 * WPE + w];
+      if (some) keep();
       // ---- results: w_k (c (h/2) w_i w_j sum + lambda (h/2)^3 w_i w_j u)
       const int p2 = emax - 1020 - tab->fx16.q;
       auto results = [&](auto with_coef) {
@@ -303,33 +345,36 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
         results(std::true_type{});
       else
         results(std::false_type{});
-    } else {  // ---- the direct sums, from the element's values in memory order
-      double *x = reinterpret_cast<double *>(dig);
-#pragma unroll
-      for (int l = 0; l < L; ++l)
-#pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (on(q) && layer(l)) x[(k0 + l) * NQ2 + at(q)] = u[l][q];
+    } else {
+      keep();
+    }
+    if (some) {  // ---- the FP64 sums of the nodes in `low`, as in fx_element
       __syncthreads();
-#pragma unroll 1
-      for (int l = 0; l < L; ++l) {
-        if (!layer(l)) break;
-        const int k = k0 + l;
-#pragma unroll 1
-        for (int q = 0; q < 8; ++q) {
-          if (!on(q)) continue;
-          const double v = x[k * NQ2 + at(q)];
-          const double d = fx_direct<NQ>(x, tab, node_i(q), node_j(q), k);
-          const double r = tab->fx16.w1[k] * fma(tab->fx16.wg[lane * 8 + q], coef ? ce * d : d,
-                                                 tab->fx16.wm[lane * 8 + q] * v);
-          int32_t i = -1;
-          if (FUSED) {
-            i = ids[base + l * NQ2 + at(q)];
-            if (!chk(bs_pred_fused_entry(i, tab->ng), BS_CHK_OP_ENTRY)) i = -1;
-          }
-          store(l, q, r, i, v);
+      uint16_t *list = reinterpret_cast<uint16_t *>(xch) + k0 * NQ2;
+      const int count = fx_list(low, 8 * L, lane, list, [&](int b) {
+        return (k0 + (b >> 3)) * NQ2 + node_j(b & 7) * NQ + node_i(b & 7);
+      });
+      __syncthreads();
+      fx_direct_list<NQ>(x, tab->kh, list, count, lane, [&](int n, double d) {
+        const int i = n % NQ, j = n / NQ % NQ, k = n / NQ2;
+        // the owner's table entry: lane (j % 8, i / 2 % 4), q
+        const int own = ((j & 7) * 4 + (i & 7) / 2) * 8 + 4 * (j >> 3) + 2 * (i >> 3) + (i & 1);
+        const double v = x[n];
+        const double r = tab->fx16.w1[k] *
+                         fma(tab->fx16.wg[own], coef ? ce * d : d, tab->fx16.wm[own] * v);
+        int32_t to = 0;
+        if (FUSED) {
+          to = ids[e * NP + n];
+          if (!chk(bs_pred_fused_entry(to, tab->ng), BS_CHK_OP_ENTRY)) to = -1;
         }
-      }
+        if (to >= 0) {
+          __stcs(out + e * NP + n, r);
+        } else if (to != -1) {
+          const double y = plus_zero(r);
+          __stcs(outG + (-2 - to), y);
+          acc.add(v, y);
+        }
+      });
     }
   }
   if (FUSED && partials) {

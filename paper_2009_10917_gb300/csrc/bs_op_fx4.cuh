@@ -15,11 +15,12 @@
 // k = 2 (g / 4) + t / 2.  One warp takes kFx4Epw elements, their values loaded
 // together.  Degree 2 runs in the same tiles with zero digits (27 of 64 nodes, and
 // still ahead).  With four nodes a line every order fits its start value of
-// 1.5 * 2^23 (at most 0.23 of the range): no second start value.
+// 1.5 * 2^23: no second start value.  Nodes whose terms are too small for the digits take
+// FP64 sums, each on its own lane.
 //
-// What bounds it: integer and issue slots, as bs_op_fx.cuh.  A p with the gather on
-// 10M (9.3M) local nodes: 395 -> 151 us at degree 3 (even-odd FP64 kernel before), 359
-// -> 271 at degree 2 (direct FP64).  Degree 1, 8 of 64 nodes, stays with the FP64 kernel.
+// What bounds it: integer and issue slots, as bs_op_fx.cuh.  A_L u on 16M (12.8M) local
+// nodes: 606 -> 171 us at degree 3 (direct FP64 kernel before), 435 -> 324 at degree 2;
+// where all nodes take FP64 sums 478 and 754.  Degree 1, 8 of 64 nodes, stays with the FP64 kernel.
 #pragma once
 
 #include "bs_op_fx16.cuh"
@@ -30,11 +31,6 @@ namespace bs {
 // for 592704 elements at Nq = 4, A_L Z p alone; 2 elements a warp 387 with spills,
 // 3 393, 6 404, 1 417; 124 registers (four blocks) 430.
 constexpr int kFx4Epw = 4, kFx4Warps = 4, kFx4Blocks = 5;
-// log2 of the lines' range that the digits serve: narrower than kFxRange, since a
-// short line has fewer terms for the FP64 sums to lose (at 8, entries of graded
-// elements of degree 2 were off by 9e-15 of their terms, the FP64 sums by 4e-16).
-// On uniform values one element in 450 (degree 2) or 4000 is beyond it.
-constexpr int kFx4Range = 4;
 constexpr int kFx4Epb = kFx4Epw * kFx4Warps;
 
 template <int NQ>
@@ -44,13 +40,6 @@ constexpr bool use_fx4() {
 
 constexpr int kFx4Digit = 36;                      // words of a digit: 32, and 4 of padding
 constexpr int kFx4Words = 2 * kFxDigits * kFx4Digit;  // both layouts of an element
-
-__device__ __forceinline__ void fx4_mma8(float *c, uint32_t a0, uint32_t a1, uint32_t b0) {
-  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(b0));
-}
 
 // A lane's half of the orders (x0, x1, x2: orders par, par + 2, par + 4, start
 // values included) in the units of fx_join.
@@ -152,17 +141,36 @@ __global__ void __launch_bounds__(32 * kFx4Warps, kFx4Blocks)
   const bool hiT = t >= 2;
   // where the sums along t of this lane's nodes arrive
   const int src = (kk | ((j >> 1) << 2)) * 4 + (((j & 1) << 1) | (t & 1));
+  const uint32_t ka = __ldg(&tab->fx4.a[lane]);  // |Kh[g % 4][2 (t % 2) ..]|
+  const float least = fx_slack<NQ>(st) * tab->fx4.low;
   auto element = [&](int64_t e, double a, double b, int32_t m0, int32_t m1) {
-    uint32_t m = max(fx_size(a), fx_size(b));
-    m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));  // the line along r
-    const uint32_t big = __reduce_max_sync(0xffffffffu, m);
-    const uint32_t low = __reduce_min_sync(0xffffffffu, m ? m : 0x7fffffffu);
-    const int emax = big ? (int)(big >> 20) : 1023;
-    const bool direct = emax < 123 || emax > 1923 || (big && emax - (int)(low >> 20) > kFx4Range);
+    bool zero;
+    const int emax = fx_emax<1>(
+        max(fx_size(a), fx_size(b)),
+        [&] { return (uint32_t)(__double2loint(a) | __double2loint(b)); }, nullptr, 0, lane,
+        [] {}, &zero);
+    const bool far = fx_far(emax);
+    const bool live0 = on0 && (!GATHER_IN || (FUSED ? m0 != -1 : m0 >= 0));
+    const bool live1 = on1 && (!GATHER_IN || (FUSED ? m1 != -1 : m1 >= 0));
+    bool low0 = far && live0, low1 = far && live1;  // nodes the digits do not serve
+    if (!far && !zero) {
+      // their terms' sizes: along r the lines with even k in columns 0-3 of rows
+      // 0-7, those with odd k in columns 4-7 of rows 8-15; along s the matrix once per od
+      const uint32_t h = fx_sizes2(a, b, emax);
+      float r[4] = {0.f, 0.f, 0.f, 0.f};
+      fx_mma8(r, hiT ? 0u : h, hiT ? h : 0u, ka);
+      const float r0 = hiT ? r[2] : r[0], r1 = hiT ? r[3] : r[1];
+      if (__any_sync(0xffffffffu, (live0 && r0 < least) || (live1 && r1 < least))) {
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        fx_mma8(s, od == (t >> 1) ? ka : 0u, 0u, fx_trans(h));
+        low0 = live0 && r0 + s[0] < least;
+        low1 = live1 && r1 + s[1] < least;
+      }
+    }
     const double ce = coef ? coef[e] : 1.0;
-    double r0, r1;
+    double r0 = 0.0, r1 = 0.0;
     __syncwarp();  // the last element's digits have been read
-    if (!direct) {
+    if (!far) {
       const uint64_t x = fx_fixed(a, emax), y = fx_fixed(b, emax);
       const uint32_t d[D] = {fx_digit2<0>(x, y), fx_digit2<1>(x, y), fx_digit2<2>(x, y),
                              fx_digit2<3>(x, y), fx_digit2<4>(x, y), fx_digit2<5>(x, y)};
@@ -185,7 +193,7 @@ __global__ void __launch_bounds__(32 * kFx4Warps, kFx4Blocks)
         fx_mma0(c0, f[0], f[1], f[2], f[3], v0, 0u, start);
         fx_mma0(c2, f[0], f[1], f[2], f[3], v2, v0, start);
         fx_mma0(c4, f[0], f[1], f[2], f[3], v4, v2, start);
-        fx4_mma8(c4, f[4], f[5], v0);
+        fx_mma8(c4, f[4], f[5], v0);
         uint64_t s[4];
 #pragma unroll
         for (int n = 0; n < 4; ++n)
@@ -207,7 +215,7 @@ __global__ void __launch_bounds__(32 * kFx4Warps, kFx4Blocks)
           float lo[4], hi[4];
           fx_mma0(lo, v0, v2, 0u, v0, b4[2 * c], b4[2 * c + 1], start);
           fx_mma0(hi, v4, 0u, v2, 0u, b4[2 * c], b4[2 * c + 1], start);
-          fx4_mma8(hi, v0, 0u, b2[c]);
+          fx_mma8(hi, v0, 0u, b2[c]);
 #pragma unroll
           for (int n = 0; n < 2; ++n)
             s[c][n] = fx4_join(__float_as_uint(lo[n]), __float_as_uint(lo[2 + n]),
@@ -226,13 +234,15 @@ __global__ void __launch_bounds__(32 * kFx4Warps, kFx4Blocks)
       const int p2 = emax - 1020 - tab->fx4.q;
       r0 = fx_double((int64_t)T0, p2);
       r1 = fx_double((int64_t)T1, p2);
-    } else {
+    }
+    if (__any_sync(0xffffffffu, low0 || low1)) {  // their FP64 sums
+      __syncwarp();  // the digits have been read
       double *x = reinterpret_cast<double *>(P);
       if (on0) x[own] = a;
       if (on1) x[own + 1] = b;
       __syncwarp();
-      r0 = on0 ? fx_direct<NQ>(x, tab, i0, j, kk) : 0.0;
-      r1 = on1 ? fx_direct<NQ>(x, tab, i0 + 1, j, kk) : 0.0;
+      if (low0) r0 = fx_direct<NQ>(x, tab->kh, i0, j, kk);
+      if (low1) r1 = fx_direct<NQ>(x, tab->kh, i0 + 1, j, kk);
     }
     if (coef) {
       r0 = ce * r0;

@@ -11,18 +11,25 @@
 // own layers, t all of them).  The three components share one exponent, the
 // element's largest flux.
 //
-// Elements that the digits do not serve, by u or by the fluxes (see
-// kFxRange), take the FP64 sums of fxg_direct.
+// The fluxes carry the quadrature weights, which differ by 1500 inside an element at
+// N = 7: the digits are those of the fluxes times the weights' inverse powers of two,
+// which the matrix then takes up exactly (P^-1 D^T P, P = diag(2^-p)).
+// As in bs_op_fx.cuh the digits serve a gradient component, and then an entry, only where
+// the sum of the sizes of its own terms is large enough (FxGeoTab::lowd, lowdt; a component
+// by its line, along t from a plane of |u| in halves; an entry by its lines along r and
+// s); the others take FP64 sums of the lines.  Elements beyond 2^+-900 or not finite, by u
+// or by the fluxes, take the FP64 sums of fxg_direct.
 #pragma once
 
 #include "bs_op_geo.cuh"
 
 namespace bs {
 
-// Three or four warps of two layers per element: 19683 elements at Nq = 6, 7, 8
-// in 229, 268 and 284 us (FP64 kernel 434, 800, 1020); warps of four layers, or
-// one warp per element, take 320 us and more (their registers spill or leave
-// too few warps).  Nq = 5 stays with the FP64 kernel: 225 us against 196, the
+// Three or four warps of two layers per element: 13824, 13824 and 19683 elements at Nq =
+// 6, 7, 8 in 195, 245 and 352 us on uniform values (FP64 kernel 295, 566, 1020; without the
+// second look at small entries 159, 191, 296), 447, 596 and 1030 where most nodes take
+// FP64 sums after all; warps of four layers, or one warp per element, take longer (their
+// registers spill or leave too few warps).  Nq = 5 stays with the FP64 kernel: 225 us against 196, the
 // 5 x 5 layers fill 39% of the tiles.
 template <int NQ>
 constexpr bool use_fx_geo() {
@@ -35,10 +42,13 @@ struct FxGeoShape {
   static constexpr int WPE = (NQ + L - 1) / L;
   static constexpr int THREADS = 32 * WPE;           // one element per block
   static constexpr int BLOCKS = NQ == 8 ? 5 : (NQ == 7 ? 6 : 8);
-  static constexpr int BASE = FxShape<NQ>::DIG + FxShape<NQ>::XCH;
-  static constexpr int FX = BASE + WPE * 256;        // + columns' maxima
+  static constexpr int SIZES = FxShape<NQ>::DIG + FxShape<NQ>::XCH;  // a plane of |u|
+  static constexpr int COL = SIZES + FxShape<NQ>::PLANE;             // words of the warps
+  static constexpr int X = COL + 128;                                // u in FP64
+  static constexpr int SMEM_FX = X + NP * 8;
   static constexpr int DIRECT = 4 * NP * 8;          // u and the three fluxes
-  static constexpr int SMEM = FX > DIRECT ? FX : DIRECT;
+  static constexpr int SMEM = SMEM_FX > DIRECT ? SMEM_FX : DIRECT;
+  // (the fluxes of the nodes that take FP64 sums lie over all of it)
 };
 
 // A sum's order values without their start values, joined.
@@ -84,6 +94,14 @@ __device__ __noinline__ void fxg_direct(double *x, double *__restrict__ out,
   }
 }
 
+template <int NQ>
+__device__ __noinline__ double fxg_line(const double *__restrict__ row, const double *x, int d) {
+  double v = 0.0;
+#pragma unroll
+  for (int m = 0; m < NQ; ++m) v = fma(row[m], x[m * d], v);
+  return v;
+}
+
 template <int NQ, bool GATHER_IN>
 __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCKS)
     k_ax_geo_fx(int64_t E, int64_t NL, const int32_t *__restrict__ order,
@@ -102,14 +120,10 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, warp = threadIdx.x >> 5;
   const int k0 = warp * L;
   unsigned char *dig = fxg_smem, *xch = dig + FxShape<NQ>::DIG;
-  uint32_t *col = reinterpret_cast<uint32_t *>(fxg_smem + S::BASE);
+  uint32_t *col = reinterpret_cast<uint32_t *>(fxg_smem + S::COL);
+  double *x = reinterpret_cast<double *>(fxg_smem + S::X);
   const uint32_t dig_s = (uint32_t)__cvta_generic_to_shared(dig);
-  auto sync = [] {
-    if (WPE == 1)
-      __syncwarp();
-    else
-      __syncthreads();
-  };
+  auto sync = [] { __syncthreads(); };
   auto layer = [&](int l) { return NQ % L == 0 || k0 + l < NQ; };
   const bool on0 = g < NQ && 2 * t < NQ, on1 = g < NQ && 2 * t + 1 < NQ;
   const int64_t base = e * NP, own = base + (int64_t)k0 * NQ2 + g * NQ + 2 * t;
@@ -125,31 +139,59 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
     return v;
   };
   double u0[L], u1[L];
+  uint32_t live = 0;  // bit 2l + h: outputs that are used
 #pragma unroll
   for (int l = 0; l < L; ++l) {
+    const bool a_on = on0 && layer(l), b_on = on1 && layer(l);
     if (GATHER_IN) {
-      int32_t a = on0 && layer(l) ? __ldcs(ids + own + l * NQ2) : -1;
-      int32_t b = on1 && layer(l) ? __ldcs(ids + own + l * NQ2 + 1) : -1;
+      int32_t a = a_on ? __ldcs(ids + own + l * NQ2) : -1;
+      int32_t b = b_on ? __ldcs(ids + own + l * NQ2 + 1) : -1;
       if (!chk(bs_pred_map_entry(a, tab->ng), BS_CHK_OP_ENTRY)) a = -1;
       if (!chk(bs_pred_map_entry(b, tab->ng), BS_CHK_OP_ENTRY)) b = -1;
       u0[l] = a >= 0 ? in[a] : 0.0;
       u1[l] = b >= 0 ? in[b] : 0.0;
+      live |= (a >= 0 ? 1u : 0u) << 2 * l | (b >= 0 ? 2u : 0u) << 2 * l;
     } else {  // a caller's vector may be 8-byte aligned only
-      u0[l] = on0 && layer(l) ? __ldcs(in + own + l * NQ2) : 0.0;
-      u1[l] = on1 && layer(l) ? __ldcs(in + own + l * NQ2 + 1) : 0.0;
+      u0[l] = a_on ? __ldcs(in + own + l * NQ2) : 0.0;
+      u1[l] = b_on ? __ldcs(in + own + l * NQ2 + 1) : 0.0;
+      live |= (a_on ? 1u : 0u) << 2 * l | (b_on ? 2u : 0u) << 2 * l;
     }
+    if (a_on) x[(k0 + l) * NQ2 + g * NQ + 2 * t] = u0[l];
+    if (b_on) x[(k0 + l) * NQ2 + g * NQ + 2 * t + 1] = u1[l];
   }
   const double ce = coef ? coef[e] : 1.0;
-  uint32_t big0 = 0, big1 = 0;
+  uint32_t big = 0;
 #pragma unroll
-  for (int l = 0; l < L; ++l) {
-    big0 = max(big0, fx_size(u0[l]));
-    big1 = max(big1, fx_size(u1[l]));
-  }
-  bool direct;
-  int emax = fx_range<WPE>(big0, big1, col, warp, lane, sync, &direct);
-  double r0[L], r1[L], s0[L], s1[L], t0[L], t1[L];  // grad u, then the flux
-  if (!direct) {
+  for (int l = 0; l < L; ++l) big = max(big, max(fx_size(u0[l]), fx_size(u1[l])));
+  bool zero;
+  int emax = fx_emax<WPE>(
+      big,
+      [&] {
+        uint32_t r = 0;
+#pragma unroll
+        for (int l = 0; l < L; ++l) r |= (uint32_t)(__double2loint(u0[l]) | __double2loint(u1[l]));
+        return r;
+      },
+      col, warp, lane, sync, &zero);
+  // a component's FP64 sum: row r of D on the line from node n, nodes d apart
+  auto line = [&](int r, int n, int d) { return fxg_line<NQ>(tab->fxg.sD + r * NQ, x + n, d); };
+  double r0[L], r1[L], s0[L], s1[L], t0[L], t1[L];  // sd grad u, then the flux
+  if (!fx_far(emax)) {
+    const uint32_t da = __ldg(&tab->fxg.da[lane]);
+    const float lowd = zero ? 0.f : fx_slack<NQ>(st) * tab->fxg.lowd;  // zeros: the digits are exact
+    float cr[L / 2 * 4], cs[L / 2 * 4];            // the sizes of the terms along r and s
+#pragma unroll
+    for (int l = 0; l < L; l += 2) {
+      const uint32_t h0 = fx_sizes2(u0[l], u1[l], emax), h1 = fx_sizes2(u0[l + 1], u1[l + 1], emax);
+      fx_terms_r(cr + 2 * l, da, h0, h1);
+#pragma unroll
+      for (int n = 0; n < 4; ++n) cs[2 * l + n] = 0.f;
+      fx_terms_s(cs + 2 * l, da, h0, h1);
+      uint32_t *hp = reinterpret_cast<uint32_t *>(fxg_smem + S::SIZES);
+      const int k = k0 + l;
+      if (layer(l)) hp[(k * 8 + (g ^ k)) * 4 + t] = h0;
+      if (layer(l + 1)) hp[((k + 1) * 8 + (g ^ (k + 1))) * 4 + t] = h1;
+    }
 #pragma unroll
     for (int l = 0; l < L; ++l) {
       if (!layer(l)) break;
@@ -157,16 +199,25 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
     }
     FxMul<NQ> mul(tab->fxg.d, lane);
     sync();
-    // ---- the gradient
+    // ---- the gradient; along t in the exchange's layout: nodes (2t, k0 + l, g)
+    int p2 = emax - 1020 - tab->fxg.qd;
 #pragma unroll
     for (int l = 0; l < L; ++l) {
       if (!layer(l)) break;
-      uint32_t a[D], b[D];
-      mul.along_t(dig_s, k0 + l, a, b);
+      const int j = k0 + l, krow = mul.mrow < NQ ? mul.mrow : NQ - 1;
+      uint32_t a[D], b[D], h;
+      mul.along_t(dig_s, j, a, b);
+      fx_ldsm1t(&h, dig_s + S::SIZES + (krow * 8 + (j ^ krow)) * 16);
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
+      fx_mma8(c, da, 0u, h);
+      double v0 = fx_double((int64_t)fx_join0(a), p2), v1 = fx_double((int64_t)fx_join0(b), p2);
+      if (__any_sync(0xffffffffu, fminf(c[0], c[1]) < lowd)) {
+        if (on0 && c[0] < lowd) v0 = line(g, j * NQ + 2 * t, NQ2);
+        if (on1 && c[1] < lowd) v1 = line(g, j * NQ + 2 * t + 1, NQ2);
+      }
       if (NQ == 8 || g < NQ)
-        *fx_xch<NQ>(xch, k0 + l, g, t) = make_ulonglong2(fx_join0(a), fx_join0(b));
+        *reinterpret_cast<double2 *>(fx_xch<NQ>(xch, j, g, t)) = make_double2(v0, v1);
     }
-    int p2 = emax - 1020 - tab->fxg.qd;
 #pragma unroll
     for (int l = 0; l < L; l += 2) {
       if (!layer(l)) break;
@@ -183,43 +234,105 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
         s1[l + h] = fx_double((int64_t)fx_join0(b), p2);
       }
     }
+    float m = INFINITY;
+#pragma unroll
+    for (int n = 0; n < 2 * L; ++n)
+      if ((n & 1 ? on1 : on0) && layer(n / 2)) m = fminf(m, fminf(cr[n], cs[n]));
+    if (__any_sync(0xffffffffu, m < lowd)) {
+#pragma unroll
+      for (int n = 0; n < 2 * L; ++n) {
+        if (!((n & 1 ? on1 : on0) && layer(n / 2))) continue;
+        const int i = 2 * t + (n & 1), k = (k0 + n / 2) * NQ2;
+        double &r = n & 1 ? r1[n / 2] : r0[n / 2], &s = n & 1 ? s1[n / 2] : s0[n / 2];
+        if (cr[n] < lowd) r = line(i, k + g * NQ, 1);
+        if (cs[n] < lowd) s = line(g, k + i, NQ);
+      }
+    }
     sync();
-    // ---- the flux; u becomes lambda M u
-    big0 = big1 = 0;
+    // ---- the flux; u becomes lambda M u.  The fluxes carry the quadrature weights, whose
+    // range is 1500 at N = 7: their digits are those of 2^p times them, p = p_i + p_j + p_k
+    const int q0 = on0 ? tab->fxg.p[2 * t] + tab->fxg.p[g] : 0;
+    const int q1 = on1 ? tab->fxg.p[2 * t + 1] + tab->fxg.p[g] : 0;
+    int w0[L], w1[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
-      if (!layer(l)) break;
-      ulonglong2 v = make_ulonglong2(0, 0);
-      if (NQ == 8 || g < NQ) v = *fx_xch<NQ>(xch, g, k0 + l, t);
-      const double ut0 = fx_double((int64_t)v.x, p2), ut1 = fx_double((int64_t)v.y, p2);
+      const int q = layer(l) ? tab->fxg.p[k0 + l] : 0;
+      w0[l] = q0 + q;
+      w1[l] = q1 + q;
+    }
+    auto size = [](double v, int p) {
+      const uint32_t z = fx_size(v);
+      return z ? z + ((uint32_t)p << 20) : 0u;
+    };
+    big = 0;
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      t0[l] = t1[l] = 0.0;
+      if (!layer(l)) {
+        r0[l] = r1[l] = s0[l] = s1[l] = 0.0;
+        break;
+      }
+      double2 v = make_double2(0.0, 0.0);
+      if (NQ == 8 || g < NQ) v = *reinterpret_cast<double2 *>(fx_xch<NQ>(xch, g, k0 + l, t));
       const double2 g0 = pair(geo, l), g1 = pair(geo + NL, l), g2 = pair(geo + 2 * NL, l);
       const double2 g3 = pair(geo + 3 * NL, l), g4 = pair(geo + 4 * NL, l);
       const double2 g5 = pair(geo + 5 * NL, l), M = pair(geo + 6 * NL, l);
-      const double a0 = fma(g0.x, r0[l], fma(g1.x, s0[l], g2.x * ut0));
-      const double b0 = fma(g1.x, r0[l], fma(g3.x, s0[l], g4.x * ut0));
-      t0[l] = fma(g2.x, r0[l], fma(g4.x, s0[l], g5.x * ut0));
-      const double a1 = fma(g0.y, r1[l], fma(g1.y, s1[l], g2.y * ut1));
-      const double b1 = fma(g1.y, r1[l], fma(g3.y, s1[l], g4.y * ut1));
-      t1[l] = fma(g2.y, r1[l], fma(g4.y, s1[l], g5.y * ut1));
+      const double a0 = fma(g0.x, r0[l], fma(g1.x, s0[l], g2.x * v.x));
+      const double b0 = fma(g1.x, r0[l], fma(g3.x, s0[l], g4.x * v.x));
+      t0[l] = fma(g2.x, r0[l], fma(g4.x, s0[l], g5.x * v.x));
+      const double a1 = fma(g0.y, r1[l], fma(g1.y, s1[l], g2.y * v.y));
+      const double b1 = fma(g1.y, r1[l], fma(g3.y, s1[l], g4.y * v.y));
+      t1[l] = fma(g2.y, r1[l], fma(g4.y, s1[l], g5.y * v.y));
       r0[l] = a0;
       r1[l] = a1;
       s0[l] = b0;
       s1[l] = b1;
       u0[l] = lambda * (M.x * u0[l]);
       u1[l] = lambda * (M.y * u1[l]);
-      big0 = max(big0, max(fx_size(a0), max(fx_size(b0), fx_size(t0[l]))));
-      big1 = max(big1, max(fx_size(a1), max(fx_size(b1), fx_size(t1[l]))));
+      big = max(big, max(size(a0, w0[l]), max(size(b0, w0[l]), size(t0[l], w0[l]))));
+      big = max(big, max(size(a1, w1[l]), max(size(b1, w1[l]), size(t1[l], w1[l]))));
     }
-    emax = fx_range<WPE>(big0, big1, col, warp, lane, sync, &direct);
-    if (WPE == 1) __syncwarp();  // every lane has read its exchanged sums
-    if (!direct) {
+    // (the low words of the fluxes: those that are zero in the high word count as far)
+    emax = fx_emax<WPE>(
+        big,
+        [&] {
+          uint32_t r = 0;
+#pragma unroll
+          for (int l = 0; l < L; ++l)
+            r |= (uint32_t)(__double2loint(r0[l]) | __double2loint(r1[l]) |
+                            __double2loint(s0[l]) | __double2loint(s1[l]) |
+                            __double2loint(t0[l]) | __double2loint(t1[l]));
+          return r;
+        },
+        col + 2 * WPE, warp, lane, sync, &zero);
+    if (!fx_far(emax)) {
+      // the entries that the fluxes' digits do not serve: bit 2l + h
+      uint32_t low = 0;
+      if (!zero) {
+        const uint32_t dta = __ldg(&tab->fxg.dta[lane]);
+        const float lowdt = fx_slack<NQ>(st) * tab->fxg.lowdt;
+#pragma unroll
+        for (int l = 0; l < L; l += 2) {
+          auto sizes = [&](const double *a, const double *b, int m) {
+            return fx_sizes2(a[m], b[m], emax, w0[m], w1[m]);
+          };
+          float c[4];
+          fx_terms_r(c, dta, sizes(r0, r1, l), sizes(r0, r1, l + 1));
+          fx_terms_s(c, dta, sizes(s0, s1, l), sizes(s0, s1, l + 1));
+#pragma unroll
+          for (int n = 0; n < 4; ++n) low |= c[n] < lowdt ? 1u << (2 * l + n) : 0u;
+        }
+        low &= live;
+      }
+      bool some = __any_sync(0xffffffffu, low);
+      if (lane == 0) col[4 * WPE + warp] = some;
       mul.set(tab->fxg.dt, lane);
       uint64_t T0[L], T1[L];
       // ---- D^T along r and s: a warp's own layers
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         if (!layer(l)) break;
-        fx_store_digits<NQ>(dig, k0 + l, g, t, r0[l], r1[l], emax);
+        fx_store_digits<NQ>(dig, k0 + l, g, t, r0[l], r1[l], emax, w0[l], w1[l]);
       }
       __syncwarp();
 #pragma unroll
@@ -238,7 +351,7 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         if (!layer(l)) break;
-        fx_store_digits<NQ>(dig, k0 + l, g, t, s0[l], s1[l], emax);
+        fx_store_digits<NQ>(dig, k0 + l, g, t, s0[l], s1[l], emax, w0[l], w1[l]);
       }
       __syncwarp();
 #pragma unroll
@@ -254,9 +367,11 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         if (!layer(l)) break;
-        fx_store_digits<NQ>(dig, k0 + l, g, t, t0[l], t1[l], emax);
+        fx_store_digits<NQ>(dig, k0 + l, g, t, t0[l], t1[l], emax, w0[l], w1[l]);
       }
       sync();
+#pragma unroll
+      for (int w = 0; w < WPE; ++w) some = some || col[4 * WPE + w];
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         if (!layer(l)) break;
@@ -267,22 +382,50 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
       }
       sync();
       p2 = emax - 1020 - tab->fxg.qdt;
+      const double c = ce * tab->fxg.inv;
 #pragma unroll
       for (int l = 0; l < L; ++l) {
         if (!layer(l)) break;
         ulonglong2 v = make_ulonglong2(0, 0);
         if (NQ == 8 || g < NQ) v = *fx_xch<NQ>(xch, g, k0 + l, t);
-        const double d0 = fx_double((int64_t)(T0[l] + v.x), p2);
-        const double d1 = fx_double((int64_t)(T1[l] + v.y), p2);
-        if (on0) __stcs(out + own + l * NQ2, fma(ce, d0, u0[l]));
-        if (on1) __stcs(out + own + l * NQ2 + 1, fma(ce, d1, u1[l]));
+        const double d0 = fx_double((int64_t)(T0[l] + v.x), p2 - w0[l]);
+        const double d1 = fx_double((int64_t)(T1[l] + v.y), p2 - w1[l]);
+        if (on0) __stcs(out + own + l * NQ2, fma(c, d0, u0[l]));
+        if (on1) __stcs(out + own + l * NQ2 + 1, fma(c, d1, u1[l]));
+      }
+      if (!some) return;
+      // ---- the FP64 sums of the nodes in `low`, each by its own lane
+      sync();  // the exchanged sums have been read
+      double *f = reinterpret_cast<double *>(fxg_smem);
+#pragma unroll
+      for (int l = 0; l < L; ++l) {
+        if (!layer(l)) break;
+        const int n = (k0 + l) * NQ2 + g * NQ + 2 * t;
+        if (on0) f[n] = r0[l], f[NP + n] = s0[l], f[2 * NP + n] = t0[l];
+        if (on1) f[n + 1] = r1[l], f[NP + n + 1] = s1[l], f[2 * NP + n + 1] = t1[l];
+      }
+      sync();
+      const double cd = ce * tab->fxg.invd, *DT = tab->fxg.D;
+#pragma unroll
+      for (int b = 0; b < 2 * L; ++b) {
+        if (!(low >> b & 1u)) continue;
+        const int i = 2 * t + (b & 1), k = k0 + (b >> 1);
+        double v = 0.0;
+#pragma unroll 4
+        for (int m = 0; m < NQ; ++m) {
+          v = fma(DT[m * NQ + i], f[m + NQ * g + NQ2 * k], v);
+          v = fma(DT[m * NQ + g], f[NP + i + NQ * m + NQ2 * k], v);
+          v = fma(DT[m * NQ + k], f[2 * NP + i + NQ * g + NQ2 * m], v);
+        }
+        __stcs(out + own + (b >> 1) * NQ2 + (b & 1),
+               fma(cd, v, (b & 1) ? u1[b >> 1] : u0[b >> 1]));
       }
       return;
     }
   }
   // ---- the FP64 sums (block-uniform), on the element's values read again
   __syncthreads();
-  double *x = reinterpret_cast<double *>(fxg_smem);
+  x = reinterpret_cast<double *>(fxg_smem);
   for (int n = threadIdx.x; n < NP; n += S::THREADS) {
     if (GATHER_IN) {
       int32_t id = ids[base + n];
