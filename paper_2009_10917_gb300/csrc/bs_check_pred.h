@@ -45,6 +45,11 @@ BS_PRED int bs_pred_tile(int64_t r0, int64_t r1, int64_t k0, int64_t k1, int64_t
          (k1 - k0 <= max_entries || r1 - r0 == 1);
 }
 
+/* Whether a row is before the end of its tile, where a block's threads run over the rows
+ * in steps: rows reach 2^31 - 2, and a thread's next one may lie past 2^31 - 1, so they
+ * are counted unsigned. */
+BS_PRED int bs_row_before(uint32_t row, int32_t end) { return row < (uint32_t)end; }
+
 /* An offset into a staged tile of n_staged values. */
 BS_PRED int bs_pred_staged(int64_t off, int64_t n_staged) { return off >= 0 && off < n_staged; }
 

@@ -109,16 +109,16 @@ __device__ __forceinline__ void gather_tile(int2 lo, int2 hi,
       int ra[R], rb[R];
       int32_t rg[R];
       T wv[DOT ? R : 1];
-      auto fetch = [&](int32_t first) {
+      auto fetch = [&](uint32_t first) {
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-          const int32_t r = first + q * kGatherBlock;
+          const uint32_t r = first + q * kGatherBlock;
           ra[q] = rb[q] = 0;
           rg[q] = -1;
-          if (r >= r1) continue;
+          if (!bs_row_before(r, r1)) continue;
           ra[q] = row_starts[r] - k0;
           rb[q] = row_starts[r + 1] - k0;
-          rg[q] = ROWMAP ? __ldcs(rows + r) : r;
+          rg[q] = ROWMAP ? __ldcs(rows + r) : (int32_t)r;
         }
         if (DOT)
 #pragma unroll
@@ -129,8 +129,9 @@ __device__ __forceinline__ void gather_tile(int2 lo, int2 hi,
       };
       fetch(r0 + threadIdx.x);
       __syncthreads();
-      for (int32_t first = r0 + threadIdx.x; first < r1; first += R * kGatherBlock) {
-        if (first != r0 + (int)threadIdx.x) fetch(first);
+      for (uint32_t first = r0 + threadIdx.x; bs_row_before(first, r1);
+           first += R * kGatherBlock) {
+        if (first != r0 + threadIdx.x) fetch(first);
 #pragma unroll
         for (int q = 0; q < R; ++q) {
           if (rg[q] < 0) continue;
@@ -143,7 +144,7 @@ __device__ __forceinline__ void gather_tile(int2 lo, int2 hi,
       }
       __syncthreads();
     } else {  // a single row longer than a tile: read straight from memory
-      for (int32_t r = r0 + threadIdx.x; r < r1; r += kGatherBlock) {
+      for (uint32_t r = r0 + threadIdx.x; bs_row_before(r, r1); r += kGatherBlock) {
         int32_t a = row_starts[r], b = row_starts[r + 1];
         if (!chk(bs_pred_row(a, b, gb.nnz), BS_CHK_GATHER_ROW)) a = b = 0;
         T s = T(0);
@@ -155,7 +156,7 @@ __device__ __forceinline__ void gather_tile(int2 lo, int2 hi,
           const int32_t c = col_ids[k];
           if (chk(bs_pred_index(c, gb.nl), BS_CHK_GATHER_COL)) s = s + qL[c];
         }
-        const int32_t g = ROWMAP ? rows[r] : r;
+        const int32_t g = ROWMAP ? rows[r] : (int32_t)r;
         if (!chk(bs_pred_index(g, gb.ng), BS_CHK_GATHER_ROW)) continue;
         qG[g] = s;
         if (DOT) acc.add(w[g], s);
@@ -353,7 +354,7 @@ __global__ void __launch_bounds__(kAgBlock)
     } else {  // rows longer than a tile: straight from the CSR
       int r1 = info[t + 1].x;
       if (!chk(r0 >= 0 && r0 <= r1 && r1 <= gb.ng, BS_CHK_GATHER_TILE)) r1 = r0;
-      for (int r = r0 + threadIdx.x; r < r1; r += kAgBlock) {
+      for (uint32_t r = r0 + threadIdx.x; bs_row_before(r, r1); r += kAgBlock) {
         int32_t b0 = row_starts[r], b1 = row_starts[r + 1];
         if (!chk(bs_pred_row(b0, b1, gb.nnz), BS_CHK_GATHER_ROW)) b0 = b1 = 0;
         T s = T(0);
