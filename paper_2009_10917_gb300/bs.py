@@ -194,8 +194,10 @@ def _check(rc, fn):
 # A call on a few thousand values is host work: torch's stream objects, ctypes
 # pointer objects and a lock per call were two thirds of it (the five vector
 # operations on 4099 values: 73 us, 41 us with plain integers).
-_device = torch._C._cuda_getDevice if hasattr(torch._C, "_cuda_getDevice") else None
-_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+# The public calls serve where torch does not have these two.
+_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
+_raw_stream = (getattr(torch._C, "_cuda_getCurrentRawStream", None)
+               or (lambda device: torch.cuda.current_stream(device).cuda_stream))
 
 
 def _stream():
