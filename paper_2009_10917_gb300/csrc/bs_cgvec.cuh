@@ -86,7 +86,7 @@ int launch_cg_r(int64_t n, const T *alpha, const T *Ap, T *r, double *partials,
   Split sp = make_split<T>(n, ptrs, 2);
   auto kern = k_cg_r<T, U, Ep>;
   const int64_t work = sp.nvec > 0 ? sp.nvec : n;
-  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock));
+  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock), kOneBlockDot);
   if (grid < 1) return fail(BS_ERR_CUDA, "no device");
   if (grid > kMaxPartials) grid = kMaxPartials;
   kern<<<grid, kReduceBlock, 0, s>>>(sp, alpha, Ap, r, partials, counter, ep, st);

@@ -65,11 +65,21 @@ constexpr int kMaxPartials = 4096;  // per-block partials a workspace holds
 // more blocks than there is work.
 int stream_grid(int64_t work, int per_thread, int block, int blocks_per_sm);
 
-// Grid of a reduction over `work` vectors: one block while its threads have
-// at most nine loads each in turn, since combining blocks (a fence, an atomic,
-// the partials read back) costs more than those.
-inline int reduce_grid(int64_t work, int per_thread, int blocks_per_sm) {
-  if (work <= 9 * kReduceBlock) return stream_grid(1, 1, 1, 1);
+// Grid of a reduction over `work` 16-byte vectors: one block while its threads have at
+// most `most` vectors each in turn, since combining blocks (a fence, an atomic, the
+// partials read back) takes about 2 us, and several where one would take longer.  The
+// two meet where (device time of one block against several, us):
+//   norm        FP64 4.8 / 5.0 at 15.6 vectors a thread, 5.7 / 5.4 at 19.5; FP32 4.7 /
+//               4.8 at 23.4, 5.1 / 4.9 at 31
+//   dot         FP64 4.9 / 5.4 at 11.7, 5.1 / 4.9 at 15.6; FP32 4.8 / 5.3 at 13.7, 5.0 /
+//               4.8 at 15.6
+//   CG's r pass (an iteration) FP64 24.6 / 24.8 at 13.4, 26.7 / 24.7 at 18; FP32 21.9 /
+//               22.9 at 10.4, 23.0 / 22.3 at 15.3
+//   update      FP64 5.35 / 5.39 at 5.9, 6.5 / 5.6 at 8; FP32 4.0 / 4.6 at 5.9, 4.6 /
+//               4.6 at 7.8, 5.2 / 4.6 at 9.8
+constexpr int kOneBlockNorm = 16, kOneBlockDot = 13, kOneBlockUpdate = 6;
+inline int reduce_grid(int64_t work, int per_thread, int blocks_per_sm, int most) {
+  if (work <= most * kReduceBlock) return stream_grid(1, 1, 1, 1);
   return stream_grid(work, per_thread, kReduceBlock, blocks_per_sm);
 }
 

@@ -60,7 +60,7 @@ extern "C" int bs_dot_noalloc(int64_t n, const double *x, const double *y, doubl
   const Split sp = make_split<double>(n, ptrs, 2);
   auto kern = k_dot<double, U, false, EpStore>;
   const int64_t work = sp.nvec > 0 ? sp.nvec : n;
-  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock));
+  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock), kOneBlockDot);
   if (grid < 1) return fail(BS_ERR_CUDA, "bs_dot_noalloc: no device");
   // k_dot is grid-stride: a smaller grid covers any n, so the partials never
   // outgrow the static array (the workspace form clamps the same way)

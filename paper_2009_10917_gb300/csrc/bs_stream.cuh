@@ -335,7 +335,8 @@ int launch_dot(int64_t n, const T *x, const T *y, double *partials, unsigned int
   Split sp = make_split<T>(n, ptrs, SELF ? 1 : 2);
   auto kern = k_dot<T, U, SELF, Ep>;
   const int64_t work = sp.nvec > 0 ? sp.nvec : n;
-  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock));
+  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock),
+                         SELF ? kOneBlockNorm : kOneBlockDot);
   if (grid < 1) return fail(BS_ERR_CUDA, "no device");
   if (grid > kMaxPartials) grid = kMaxPartials;
   kern<<<grid, kReduceBlock, 0, s>>>(sp, x, y, partials, counter, ep, st);
@@ -452,7 +453,7 @@ int launch_norm_split(int64_t n, const double *x, double *partials, unsigned int
   Split sp = make_split<double>(n, ptrs, 1);
   auto kern = k_norm_split<U, Ep>;
   const int64_t work = sp.nvec > 0 ? sp.nvec : n;
-  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock));
+  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock), kOneBlockNorm);
   if (grid < 1) return fail(BS_ERR_CUDA, "no device");
   if (grid > kMaxPartials) grid = kMaxPartials;
   kern<<<grid, kReduceBlock, 0, s>>>(sp, x, partials, counter, ep);
@@ -538,7 +539,7 @@ int launch_cg_update(int64_t n, Scalar<T> alpha, const T *p, const T *Ap, T *x, 
   Split sp = make_split<T>(n, ptrs, 4);
   auto kern = k_cg_update<T, U, Ep>;
   const int64_t work = sp.nvec > 0 ? sp.nvec : n;
-  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock));
+  int grid = reduce_grid(work, U, blocks_per_sm(kern, kReduceBlock), kOneBlockUpdate);
   if (grid < 1) return fail(BS_ERR_CUDA, "no device");
   if (grid > kMaxPartials) grid = kMaxPartials;
   kern<<<grid, kReduceBlock, 0, s>>>(sp, alpha, p, Ap, x, r, partials, counter, ep, st);
