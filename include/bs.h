@@ -250,9 +250,9 @@ int bs_diag_A(const bs_problem *prob, double *d_diag, void *stream);
  * lambda L^3 with the mesh's length scale L, and below 2^-102 they count as
  * zero -- keep L above about 2^-28 (lambda of order 1) for the accuracy
  * stated here.  The gather is the same as bs_apply_A's.  At degrees 6, 7 and
- * 11..15 (5..7 with geometric factors; without BS_OP_DIRECT) the FP64 fixed-point
- * kernel of bs_apply_A is the faster one and runs instead: FP64's accuracy and
- * range. */
+ * 11..15 (6, 7 with geometric factors; without BS_OP_DIRECT) the FP64 fixed-point
+ * kernel of bs_apply_A is the faster one and runs instead: FP64's range, entries
+ * within 16 (2 Nq + 4) 2^-53 of the sum of the sizes of their own terms. */
 int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *stream);
 
 /* How A p is formed, process-wide, by bs_apply_A, bs_apply_local,
@@ -278,12 +278,12 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   contractions exactly in 58-bit fixed point relative to each element's
  *   largest value, on the tensor cores.  Nodes whose own terms are too small
  *   for that -- and elements whose values are not finite or lie outside
- *   [2^-900, 2^900] -- take FP64 sums, so that every entry of bs_apply_A,
- *   bs_apply_local and, where it runs this kernel, bs_apply_A_ff is within
- *   (2 Nq + 4) 2^-53 of the sum of the sizes of its own terms (four standard
- *   deviations of the digits' rounding at the entries where it is largest;
- *   (2 Nq + 8) 2^-53 with geometric factors), as the FP64 sums are; inside the
- *   solvers the deviations may be N - 1 times that.
+ *   [2^-900, 2^900] -- take FP64 sums, so that every entry of bs_apply_A and
+ *   bs_apply_local is within (2 Nq + 4) 2^-53 of the sum of the sizes of its own
+ *   terms (four standard deviations of the digits' rounding at the entries
+ *   where it is largest; (2 Nq + 8) 2^-53 with geometric factors), as the FP64
+ *   sums are; inside the solvers the deviations may be N - 1 times that, 16
+ *   times with BS_CG_FF_OPERATOR.
  *   bs_fpcg_learned with a network takes the FP64 or float-float sums in any
  *   case: its input is quantised, so single nodes would show the rounding.
  * Problems with geometric factors (bs_problem_create_geo) always use their

@@ -419,12 +419,14 @@ static int scat_iteration(const bs_problem *P, bool precond, bool ff, cudaStream
                                                P->d_ApL, P->d_tabff, P->d_coef, P->d_geo,
                                                P->lambda, st, s)
                      : launch_ax_geo<false>(P->N, m->E, m->NL, nullptr, nullptr, L.p, P->d_ApL,
-                                            P->d_tab, P->d_coef, P->d_geo, P->lambda, st, s))
+                                            P->d_tab, P->d_coef, P->d_geo, P->lambda, st, s, true,
+                                            ff))
            : ff && !ff_takes_fx(P->N)
                ? launch_ax_local_ff<false>(P->N, m->E, nullptr, nullptr, L.p, P->d_ApL,
                                             P->d_tabff, P->d_coef, g, mlam, st, s)
                 : launch_ax_local<double, false>(P->N, m->E, nullptr, nullptr, L.p, P->d_ApL,
-                                                 P->d_tab, P->d_coef, g, mlam, st, s);
+                                                 P->d_tab, P->d_coef, g, mlam, st, s, nullptr,
+                                                 nullptr, true, ff);
   if (!rc)
     rc = launch_gather<double, false, EpNone>(m, P->d_ApL, v.Ap, nullptr, nullptr, nullptr,
                                               EpNone{}, st, s);

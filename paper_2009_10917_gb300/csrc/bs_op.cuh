@@ -451,16 +451,24 @@ inline int64_t ax_blocks(int N, int64_t E, bool fx) {
   }
 }
 
+// What the line below which a node takes FP64 sums (FxTab::low) is multiplied by: 1 for
+// one A p; inside the solvers 1 / (N - 1), see bs_op_fx.cuh; 1 / 16 where the caller asked
+// for the float-float operator, whose own error is 64 times that of FP64 sums.
+inline float fx_slack(int N, bool solver, bool ff) {
+  return ff ? 1.f / 16 : (solver && N > 2 ? 1.f / (N - 1) : 1.f);
+}
+
 // FUSED: ids is the fused encoding, outG the global output, partials (or
 // NULL: no dot product) ax_blocks(N, E) doubles.  fx: FP64 may take the
-// fixed-point form.
+// fixed-point form; ff: in place of the float-float kernel.
 template <typename T, bool GATHER_IN, bool FUSED = false>
 int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, const T *in,
                     T *out,
                     const OpTab<T> *tab, const double *coef, T g, T mlam,
                     const CgState *st, cudaStream_t s, T *outG = nullptr,
-                    double *partials = nullptr, bool fx = true) {
+                    double *partials = nullptr, bool fx = true, bool ff = false) {
   if (E == 0) return BS_OK;
+  [[maybe_unused]] const float slack = fx_slack(N, st != nullptr, ff);
 #define BS_AX_CASE(NQ)                                                                   \
   case NQ: {                                                                             \
     if constexpr (use_fx<NQ>() && sizeof(T) == 8) {                                      \
@@ -469,7 +477,7 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
         using Sf = FxShape<NQ>;                                                          \
         k_ax_fx<NQ, GATHER_IN, FUSED>                                                    \
             <<<(unsigned)E, Sf::THREADS, Sf::SMEM, s>>>(E, order, ids, in, out, tab, coef, \
-                                                        st, outG, partials, vec);        \
+                                                        st, outG, partials, vec, slack); \
         break;                                                                           \
       }                                                                                  \
     } else if constexpr (use_fx16<NQ>() && sizeof(T) == 8) {                             \
@@ -479,7 +487,7 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
         if (occupancy_blocks_smem((const void *)kern, Sf::THREADS, Sf::SMEM) < 1)        \
           return fail(BS_ERR_CUDA, "element operator: shared memory refused");           \
         kern<<<(unsigned)E, Sf::THREADS, Sf::SMEM, s>>>(E, order, ids, in, out, tab,     \
-                                                        coef, st, outG, partials);       \
+                                                        coef, st, outG, partials, slack); \
         break;                                                                           \
       }                                                                                  \
     } else if constexpr (use_fx4<NQ>() && sizeof(T) == 8) {                              \
@@ -487,7 +495,7 @@ int launch_ax_local(int N, int64_t E, const int32_t *order, const int32_t *ids, 
         const int vec = ((uintptr_t)out % 16 == 0) && (GATHER_IN || (uintptr_t)in % 16 == 0); \
         const int64_t grid = (E + kFx4Epb - 1) / kFx4Epb;                                \
         k_ax_fx4<NQ, GATHER_IN, FUSED><<<(unsigned)grid, 32 * kFx4Warps, 0, s>>>(        \
-            E, order, ids, in, out, tab, coef, st, outG, partials, vec);                 \
+            E, order, ids, in, out, tab, coef, st, outG, partials, vec, slack);          \
         break;                                                                           \
       }                                                                                  \
     }                                                                                    \

@@ -638,9 +638,9 @@ extern int g_op_fusion;
 // at N = 11, 173 against 405 at N = 15; N = 5 185 against 187, N = 4 234 against
 // 183, N = 9 359 against 252) and exact to FP64's rounding.
 inline bool ff_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7 || N >= 11); }
-// The same on general hexahedra, degrees 5..7: 559 against 608 us, 438 against
-// 753, 324 against 770.
-inline bool ff_geo_takes_fx(int N) { return g_op_evenodd && N >= 5 && N <= 7; }
+// The same on general hexahedra: 519 against 743 us at N = 6, 350 against 754 at N = 7
+// (10M local nodes, uniform values); N = 5 636 against 599.
+inline bool ff_geo_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7); }
 
 // Ap = A p for a global p (FP64 or FP32 tables; ff: the float-float element
 // kernel, FP64 only).  DOT: ep(p . Ap), reduced in the gather's pass (and,
@@ -658,7 +658,7 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
                                                st, s)
                       : launch_ax_geo<true>(P->N, m->E, m->NL, m->d_elem_order, m->d_ids, p, ApL,
                                             P->d_tab, P->d_coef, P->d_geo, P->lambda, st, s,
-                                            fx))
+                                            fx, ff))
         return rc;
       return launch_gather<T, DOT, Ep>(m, ApL, Ap, DOT ? p : nullptr, P->d_partials,
                                        P->d_counter, ep, st, s);
@@ -679,9 +679,9 @@ int apply_A_global(const bs_problem *P, bool ff, const OpTab<T> *tab, const T *p
                                             P->d_coef, g, mlam, st, s);
     else
       rc = fused ? launch_ax_local<T, true, true>(P->N, m->E, m->d_elem_order, ids, p, ApL, tab,
-                                                  P->d_coef, g, mlam, st, s, Ap, opp, fx)
+                                                  P->d_coef, g, mlam, st, s, Ap, opp, fx, ff)
                  : launch_ax_local<T, true>(P->N, m->E, m->d_elem_order, ids, p, ApL, tab,
-                                            P->d_coef, g, mlam, st, s, nullptr, nullptr, fx);
+                                            P->d_coef, g, mlam, st, s, nullptr, nullptr, fx, ff);
   } else {
     if (ff) return fail(BS_ERR_ARG, "the float-float operator is FP64 only");
     rc = fused ? launch_ax_local<T, true, true>(P->N, m->E, m->d_elem_order, ids, p, ApL, tab,

@@ -424,13 +424,6 @@ __device__ __forceinline__ void fx_direct_list(const double *x, const double *__
   }
 }
 
-// What FxTab::low is multiplied by: 1 for one A p (no solver state), 1 / (N - 1) inside
-// the solvers.
-template <int NQ>
-__device__ __forceinline__ float fx_slack(const CgState *st) {
-  return st ? 1.f / (NQ - 2) : 1.f;
-}
-
 // The nodes whose bit b of `low` is set (b < n; node(b): the index in the element), one
 // lane after the other, into a warp's list; how many.
 template <class Node>
@@ -447,7 +440,8 @@ __device__ __forceinline__ int fx_list(uint32_t low, int n, int lane, uint16_t *
 // out = A_L in on one element e, by the WPE warps that call it with their own
 // first layer k0 (of L) and the same shared memory (dig; see FxShape); sync()
 // is a barrier of these warps.  Other arguments as k_ax_local (FUSED
-// likewise); vec: out (and, without GATHER_IN, in) is 16-byte aligned.
+// likewise); vec: out (and, without GATHER_IN, in) is 16-byte aligned; slack: what
+// FxTab::low is multiplied by (fx_slack).
 template <int NQ, int L, bool GATHER_IN, bool FUSED, class Sync>
 __device__ __forceinline__ void fx_element(int64_t e, int k0, const int32_t *__restrict__ ids,
                                            const double *__restrict__ in,
@@ -715,7 +709,7 @@ __global__ void __launch_bounds__(FxShape<NQ>::THREADS, FxShape<NQ>::BLOCKS)
             const double *__restrict__ in, double *__restrict__ out,
             const OpTab<double> *__restrict__ tab, const double *__restrict__ coef,
             const CgState *st, double *__restrict__ outG, double *__restrict__ partials,
-            int vec) {
+            int vec, float slack) {
   using S = FxShape<NQ>;
   extern __shared__ __align__(128) unsigned char fx_smem[];
   if (cg_halted(st)) return;
@@ -725,7 +719,7 @@ __global__ void __launch_bounds__(FxShape<NQ>::THREADS, FxShape<NQ>::BLOCKS)
   if (e >= 0 && !chk(bs_pred_index(e, tab->ne), BS_CHK_OP_ENTRY)) e = -1;
   if (e >= 0)
     fx_element<NQ, S::L, GATHER_IN, FUSED>(e, (int)(threadIdx.x / 32) * S::L, ids, in, out, tab,
-                                           coef, outG, acc, vec, fx_slack<NQ>(st), fx_smem, [] {
+                                           coef, outG, acc, vec, slack, fx_smem, [] {
                                              if (S::WPE == 1)
                                                __syncwarp();
                                              else

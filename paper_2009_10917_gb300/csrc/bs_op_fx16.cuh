@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
     k_ax_fx16(int64_t E, const int32_t *__restrict__ order, const int32_t *__restrict__ ids,
               const double *__restrict__ in, double *__restrict__ out,
               const OpTab<double> *__restrict__ tab, const double *__restrict__ coef,
-              const CgState *st, double *__restrict__ outG, double *__restrict__ partials) {
+              const CgState *st, double *__restrict__ outG, double *__restrict__ partials,
+              float slack) {
   static_assert(!FUSED || GATHER_IN, "the fused operator reads its input through the map");
   using S = FxShape16<NQ>;
   constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2, D = kFxDigits, L = S::L, WPE = S::WPE;
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
     const int emax =
         fx_emax<WPE>(big, rest, s_col, warp, lane, [] { __syncthreads(); }, &zero);
     const bool far = fx_far(emax);
-    const float least = zero ? 0.f : fx_slack<NQ>(st) * tab->fx16.low;  // zeros: the digits are exact
+    const float least = zero ? 0.f : slack * tab->fx16.low;  // zeros: the digits are exact
     // the sums of the sizes of layer l's terms along r and s: each(q, sum)
     auto terms = [&](int l, auto each) {
       const uint4 ka = __ldg(reinterpret_cast<const uint4 *>(&tab->fx16.a[lane][0]));

@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(32 * kFx4Warps, kFx4Blocks)
              const double *__restrict__ in, double *__restrict__ out,
              const OpTab<double> *__restrict__ tab, const double *__restrict__ coef,
              const CgState *st, double *__restrict__ outG, double *__restrict__ partials,
-             int vec) {
+             int vec, float slack) {
   static_assert(!FUSED || GATHER_IN, "the fused operator reads its input through the map");
   constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2, D = kFxDigits, EPW = kFx4Epw;
   constexpr bool EVEN = NQ % 2 == 0;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(32 * kFx4Warps, kFx4Blocks)
   // where the sums along t of this lane's nodes arrive
   const int src = (kk | ((j >> 1) << 2)) * 4 + (((j & 1) << 1) | (t & 1));
   const uint32_t ka = __ldg(&tab->fx4.a[lane]);  // |Kh[g % 4][2 (t % 2) ..]|
-  const float least = fx_slack<NQ>(st) * tab->fx4.low;
+  const float least = slack * tab->fx4.low;
   auto element = [&](int64_t e, double a, double b, int32_t m0, int32_t m1) {
     bool zero;
     const int emax = fx_emax<1>(

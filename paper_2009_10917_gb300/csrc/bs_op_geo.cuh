@@ -122,15 +122,16 @@ template <bool GATHER_IN>
 int launch_ax_geo(int N, int64_t E, int64_t NL, const int32_t *order, const int32_t *ids,
                   const double *in, double *out, const OpTab<double> *tab, const double *coef,
                   const double *geo, double lambda, const CgState *st, cudaStream_t s,
-                  bool fx = true) {
+                  bool fx = true, bool ff = false) {
   if (E == 0) return BS_OK;
+  const float slack = fx_slack(N, st != nullptr, ff);
 #define BS_AXG_CASE(NQ)                                                                  \
   case NQ: {                                                                             \
     if constexpr (use_fx_geo<NQ>()) {                                                    \
       if (fx && g_op_evenodd) {                                                          \
         using Sf = FxGeoShape<NQ>;                                                       \
         k_ax_geo_fx<NQ, GATHER_IN><<<(unsigned)E, Sf::THREADS, Sf::SMEM, s>>>(           \
-            E, NL, order, ids, in, out, tab, coef, geo, lambda, st);                     \
+            E, NL, order, ids, in, out, tab, coef, geo, lambda, st, slack);              \
         break;                                                                           \
       }                                                                                  \
     }                                                                                    \

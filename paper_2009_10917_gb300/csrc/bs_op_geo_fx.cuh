@@ -18,7 +18,8 @@
 // the sum of the sizes of its own terms is large enough (FxGeoTab::lowd, lowdt; a component
 // by its line, along t from a plane of |u| in halves; an entry by its lines along r and
 // s); the others take FP64 sums of the lines.  Elements beyond 2^+-900 or not finite, by u
-// or by the fluxes, take the FP64 sums of fxg_direct.
+// or by the fluxes, and those in which a quarter of the components do not, take the FP64 sums of
+// fxg_direct.
 #pragma once
 
 #include "bs_op_geo.cuh"
@@ -26,8 +27,8 @@
 namespace bs {
 
 // Three or four warps of two layers per element: 13824, 13824 and 19683 elements at Nq =
-// 6, 7, 8 in 195, 245 and 352 us on uniform values (FP64 kernel 295, 566, 1020; without the
-// second look at small entries 159, 191, 296), 447, 596 and 1030 where most nodes take
+// 6, 7, 8 in 198, 247 and 359 us on uniform values (FP64 kernel 295, 566, 1020; without the
+// second look at small entries 159, 191, 296), 275, 470 and 1059 where all elements take
 // FP64 sums after all; warps of four layers, or one warp per element, take longer (their
 // registers spill or leave too few warps).  Nq = 5 stays with the FP64 kernel: 225 us against 196, the
 // 5 x 5 layers fill 39% of the tiles.
@@ -65,7 +66,7 @@ __device__ __noinline__ void fxg_direct(double *x, double *__restrict__ out,
                                         const OpTab<double> *tab, const double *__restrict__ geo,
                                         int64_t NL, int64_t base, double ce, double lambda) {
   constexpr int NQ2 = NQ * NQ, NP = NQ * NQ2;
-  const double *D = tab->D;
+  const double *D = tab->fxg.D;
   double *fr = x + NP, *fs = fr + NP, *ft = fs + NP;
   for (int n = threadIdx.x; n < NP; n += blockDim.x) {
     const int i = n % NQ, j = n / NQ % NQ, k = n / NQ2;
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
                 const int32_t *__restrict__ ids, const double *__restrict__ in,
                 double *__restrict__ out, const OpTab<double> *__restrict__ tab,
                 const double *__restrict__ coef, const double *__restrict__ geo, double lambda,
-                const CgState *st) {
+                const CgState *st, float slack) {
   using S = FxGeoShape<NQ>;
   constexpr int NQ2 = NQ * NQ, NP = S::NP, D = kFxDigits, L = S::L, WPE = S::WPE;
   constexpr bool EVEN = NQ % 2 == 0;
@@ -176,10 +177,12 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
   // a component's FP64 sum: row r of D on the line from node n, nodes d apart
   auto line = [&](int r, int n, int d) { return fxg_line<NQ>(tab->fxg.sD + r * NQ, x + n, d); };
   double r0[L], r1[L], s0[L], s1[L], t0[L], t1[L];  // sd grad u, then the flux
-  if (!fx_far(emax)) {
-    const uint32_t da = __ldg(&tab->fxg.da[lane]);
-    const float lowd = zero ? 0.f : fx_slack<NQ>(st) * tab->fxg.lowd;  // zeros: the digits are exact
-    float cr[L / 2 * 4], cs[L / 2 * 4];            // the sizes of the terms along r and s
+  bool sums = fx_far(emax);  // all of the element by FP64 sums
+  const uint32_t da = __ldg(&tab->fxg.da[lane]);
+  const float lowd = zero ? 0.f : slack * tab->fxg.lowd;  // zeros: the digits are exact
+  float cr[2 * L], cs[2 * L];  // the sizes of the terms along r and s
+  float least = INFINITY;
+  if (!sums) {
 #pragma unroll
     for (int l = 0; l < L; l += 2) {
       const uint32_t h0 = fx_sizes2(u0[l], u1[l], emax), h1 = fx_sizes2(u0[l + 1], u1[l + 1], emax);
@@ -197,8 +200,28 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
       if (!layer(l)) break;
       fx_store_digits<NQ>(dig, k0 + l, g, t, u0[l], u1[l], emax);
     }
-    FxMul<NQ> mul(tab->fxg.d, lane);
+#pragma unroll
+    for (int n = 0; n < 2 * L; ++n)
+      if ((n & 1 ? on1 : on0) && layer(n / 2)) least = fminf(least, fminf(cr[n], cs[n]));
+    // where a quarter of these components are for FP64 sums, the digits would come on top
+    // of sums for most of the element (487, 642 and 1112 us for a field of such elements)
+    uint32_t few = 0;
+    if (__any_sync(0xffffffffu, least < lowd))
+#pragma unroll
+      for (int n = 0; n < 2 * L; ++n) {
+        const bool use = (n & 1 ? on1 : on0) && layer(n / 2);
+        few += __popc(__ballot_sync(0xffffffffu, use && cr[n] < lowd)) +
+               __popc(__ballot_sync(0xffffffffu, use && cs[n] < lowd));
+      }
+    if (lane == 0) col[5 * WPE + warp] = few;
     sync();
+    few = 0;
+#pragma unroll
+    for (int w = 0; w < WPE; ++w) few += col[5 * WPE + w];
+    sums = few > NP / 2;
+  }
+  if (!sums) {
+    FxMul<NQ> mul(tab->fxg.d, lane);
     // ---- the gradient; along t in the exchange's layout: nodes (2t, k0 + l, g)
     int p2 = emax - 1020 - tab->fxg.qd;
 #pragma unroll
@@ -234,11 +257,7 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
         s1[l + h] = fx_double((int64_t)fx_join0(b), p2);
       }
     }
-    float m = INFINITY;
-#pragma unroll
-    for (int n = 0; n < 2 * L; ++n)
-      if ((n & 1 ? on1 : on0) && layer(n / 2)) m = fminf(m, fminf(cr[n], cs[n]));
-    if (__any_sync(0xffffffffu, m < lowd)) {
+    if (__any_sync(0xffffffffu, least < lowd)) {
 #pragma unroll
       for (int n = 0; n < 2 * L; ++n) {
         if (!((n & 1 ? on1 : on0) && layer(n / 2))) continue;
@@ -310,7 +329,7 @@ __global__ void __launch_bounds__(FxGeoShape<NQ>::THREADS, FxGeoShape<NQ>::BLOCK
       uint32_t low = 0;
       if (!zero) {
         const uint32_t dta = __ldg(&tab->fxg.dta[lane]);
-        const float lowdt = fx_slack<NQ>(st) * tab->fxg.lowdt;
+        const float lowdt = slack * tab->fxg.lowdt;
 #pragma unroll
         for (int l = 0; l < L; l += 2) {
           auto sizes = [&](const double *a, const double *b, int m) {
