@@ -241,8 +241,20 @@ __global__ void __launch_bounds__(32 * kFx4Warps, kFx4Blocks)
       if (on0) x[own] = a;
       if (on1) x[own + 1] = b;
       __syncwarp();
-      if (low0) r0 = fx_direct<NQ>(x, tab->kh, i0, j, kk);
-      if (low1) r1 = fx_direct<NQ>(x, tab->kh, i0 + 1, j, kk);
+      if (NQ == 3) {  // 27 nodes: one a lane instead of two on every other (one pass)
+        const int n = lane < NP ? lane : 0, i = n % NQ, jn = n / NQ % NQ, k = n / NQ2;
+        const int owner = ((k >> 1) * 4 + jn) * 4 + (i >> 1) + 2 * (k & 1);
+        const uint32_t m0 = __ballot_sync(0xffffffffu, low0), m1 = __ballot_sync(0xffffffffu, low1);
+        double v = 0.0;
+        if (lane < NP && ((i & 1 ? m1 : m0) >> owner & 1u)) v = fx_direct<NQ>(x, tab->kh, i, jn, k);
+        const double v0 = __shfl_sync(0xffffffffu, v, own & 31);
+        const double v1 = __shfl_sync(0xffffffffu, v, (own + 1) & 31);
+        if (low0) r0 = v0;
+        if (low1) r1 = v1;
+      } else {
+        if (low0) r0 = fx_direct<NQ>(x, tab->kh, i0, j, kk);
+        if (low1) r1 = fx_direct<NQ>(x, tab->kh, i0 + 1, j, kk);
+      }
     }
     if (coef) {
       r0 = ce * r0;
