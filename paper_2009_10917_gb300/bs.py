@@ -114,8 +114,8 @@ _SIGS = {
 
 def operator_mode(mode=-1):
     """bs_operator_mode: bits BS_OP_FUSED, BS_OP_DIRECT (0, the default:
-    unfused, even-odd element kernels); returns the previous mode (-1: query
-    only)."""
+    unfused, the fixed-point element kernels where they serve and even-odd ones
+    elsewhere); returns the previous mode (-1: query only)."""
     return lib().bs_operator_mode(int(mode))
 
 

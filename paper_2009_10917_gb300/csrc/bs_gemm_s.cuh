@@ -11,8 +11,10 @@
 // operands are read by ldmatrix.trans, which takes out the transposes; the
 // loss and Adam with the refreshed bf16 operands are epilogues (their operands
 // loaded ahead of the products), and the two weight gradients share a launch.
-// A training step is five launches.  Sums run over the same 16-wide K blocks
-// in the same order as the large kernel: results are bitwise the same.
+// A training step is five launches.  Products are summed over the same 16-wide K
+// blocks in the same order as in the large kernel, so activations and gradients
+// are bitwise the same; the loss is summed tile by tile and differs from k_mse's
+// in its last bits.
 #pragma once
 
 #include "bs_mlp.cuh"

@@ -633,10 +633,11 @@ int launch_ax_geo_ff(int N, int64_t E, int64_t NL, const int32_t *order, const i
 extern int g_op_fusion;
 
 // Whether a float-float A p runs the FP64 fixed-point kernel (bs_op_fx.cuh): at
-// degrees 6, 7 and 11..15 it is the faster of the two (10M local nodes, with the
-// gather: 160 against 221 us at N = 6, 125 against 216 at N = 7, 289 against 397
-// at N = 11, 173 against 405 at N = 15; N = 5 185 against 187, N = 4 234 against
-// 183, N = 9 359 against 252) and exact to FP64's rounding.
+// degrees 6, 7 and 11..15 it is the faster of the two (10M local nodes, uniform
+// values, with the gather: 164 against 221 us at N = 6, 124 against 216 at N = 7, 290
+// against 397 at N = 11, 164 against 405 at N = 15; N = 5 185 against 187, N = 4 234
+// against 183, N = 9 359 against 252) and the more accurate.  Values spread over e^+-9
+// inside an element make it the slower one (403, 441, 967, 1066 us).
 inline bool ff_takes_fx(int N) { return g_op_evenodd && (N == 6 || N == 7 || N >= 11); }
 // The same on general hexahedra: 519 against 743 us at N = 6, 350 against 754 at N = 7
 // (10M local nodes, uniform values); N = 5 636 against 599.
