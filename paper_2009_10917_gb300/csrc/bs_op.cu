@@ -335,11 +335,14 @@ static bool fx_table(int N, const double *x0, double h, double lambda, OpTab<dou
     return big;
   };
   powers(powers(0.5) < powers(0.0) ? 0.5 : 0.0);
+  // on general hexahedra (2 Nq + 8) 2^-53 of B = the sum of |D|^T |G| |D| |u|: the components
+  // within Nq + 2 of their lines' terms, the entries within Nq + 6 of the fluxes' (the
+  // sizes of the fluxes' own terms, not of the fluxes, make up B)
   double sd, sdt;
   if (!fx_digits(Nq, kh, true, 3, allow, words(t->w, t->a), &s, &t->q, &t->low) ||
       !fx_digits(Nq, [&](int i, int m) { return D[i][m]; }, true, 1, Nq + 2.0,
                  words(tg->d, tg->da), &sd, &tg->qd, &tg->lowd) ||
-      !fx_digits(Nq, M, false, 3, Nq + 2.0,
+      !fx_digits(Nq, M, false, 3, Nq + 6.0,
                  words(tg->dt, tg->dta), &sdt, &tg->qdt, &tg->lowdt))
     return false;
   scaled_kh();
