@@ -205,7 +205,9 @@ __global__ void __launch_bounds__(FxShape16<NQ>::THREADS, FxShape16<NQ>::BLOCKS)
     } else {
 #pragma unroll
       for (int l = 0; l < L; ++l)
-        terms(l, [&](int q, float s) { low |= s < least ? 1u << (8 * l + q) : 0u; });
+        terms(l, [&](int q, float s) {
+          low |= on(q) && layer(l) && s < least ? 1u << (8 * l + q) : 0u;
+        });
     }
     if (__any_sync(0xffffffffu, low)) {
 #pragma unroll
