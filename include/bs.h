@@ -267,7 +267,7 @@ int bs_apply_A_ff(const bs_problem *prob, const double *p, double *Ap, void *str
  *   kernel writes every local value and the gather (BS6) sums every row.  Ap
  *   is bitwise the same either way (a one-copy row sums to +0 + v); p.Ap
  *   differs only by summation order.  Measured slower on GB300
- *   (partial-sector writes into Ap; N = 7 on 48^3: 0.69 vs 0.60 ms per
+ *   (partial-sector writes into Ap; N = 7 on 48^3: 0.75 vs 0.62 ms per
  *   A p).
  *  BS_OP_DIRECT: the element kernels (FP64, FP32, float-float) contract
  *   with the full 1-D stiffness K = D^T W D (3 (N+1) multiply-adds per

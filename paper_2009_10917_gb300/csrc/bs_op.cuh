@@ -25,8 +25,8 @@
 // per-block partial of p.Ap; only the shared nodes' local values go to the
 // N_L buffer, for a gather over the shared rows alone.  The result is
 // bitwise that of the unfused operator (a one-term row sum is +0 + v).
-// Measured slower on GB300 (N = 7 on 48^3: 0.69 vs 0.60 ms per A p, 3.52 vs
-// 3.40 ms with the direct kernel): in the user's global
+// Measured slower on GB300 (N = 7 on 48^3: 0.75 vs 0.62 ms per A p, 3.52 vs
+// 3.39 ms with the direct kernel): in the user's global
 // numbering the single-copy nodes come in runs of N - 1 doubles and the
 // shared rows between them, so both kernels write partial sectors of A p,
 // which costs more than the N_L round trip saved.  Off by default.

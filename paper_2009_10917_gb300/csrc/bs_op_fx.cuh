@@ -53,9 +53,9 @@
 // the tensor pipe is not what bounds it, and the accumulators are wanted in
 // registers at once.
 //
-// Measured (N = 7 on 36^3, 23.9M local nodes): A_L Z p 182 us, the even-odd
+// Measured (N = 7 on 36^3, 23.9M local nodes): A_L Z p 180 us, the even-odd
 // FP64 kernel 1047 us; HBM alone would allow 60 us.  What bounds it now is
-// spread out: issue slots 61%, integer pipe 55%, FP64 pipe 46%, L1 65%, HBM 26%.
+// spread out: issue slots 65%, integer pipe 57%, FP64 pipe 46%, L1 66%, HBM 26%.
 // Conversions by two FP64 additions per node (instead of fx_double) and the
 // weights multiplied node by node took 312 us with the FP64 pipe at 82%.
 // Where every node takes FP64 sums (36^3, A_L u): 1177 us, the direct FP64
@@ -80,7 +80,8 @@ constexpr bool use_fx() {
 }
 
 // Two warps of four layers per element at Nq = 8 (72 registers, 14 elements per
-// SM: 176 us for 46656 elements, A_L Z p alone, against 180 with 80 registers,
+// SM: 176 us for 46656 elements, A_L Z p without the look at each node's terms, against
+// 180 with 80 registers,
 // 190 for one warp of eight layers, 196 for four of two), one warp below (the
 // last warp would idle: Nq = 5, 112 us against 147 for two layers per warp,
 // Nq = 6 139 against 150).

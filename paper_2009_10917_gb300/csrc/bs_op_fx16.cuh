@@ -24,7 +24,7 @@ constexpr bool use_fx16() {
 }
 
 // Two layers a warp, as many elements an SM as leave a thread 80 to 128
-// registers: A_L Z p in ps a node 33, 31, 31, 22, 26, 18, 15, 13 at Nq = 9 .. 16
+// registers: A_L u in ps a node 31, 28, 26, 21, 21, 16, 15, 12 at Nq = 9 .. 16
 // (one layer a warp 38, 34, .., 29, .., 19; FP64 kernels 66, 63, 86 and 99 at Nq = 9,
 // 10, 12 and 16).  The tiles' filling, (Nq / 16)^2, sets most of the difference.
 template <int NQ>

@@ -27,7 +27,7 @@
 namespace bs {
 
 // Three or four warps of two layers per element: 13824, 13824 and 19683 elements at Nq =
-// 6, 7, 8 in 198, 247 and 359 us on uniform values (FP64 kernel 295, 566, 1020; without the
+// 6, 7, 8 in 186, 225 and 312 us on uniform values (FP64 kernel 295, 566, 1020; without the
 // second look at small entries 159, 191, 296), 275, 470 and 1059 where all elements take
 // FP64 sums after all; warps of four layers, or one warp per element, take longer (their
 // registers spill or leave too few warps).  Nq = 5 stays with the FP64 kernel: 225 us against 196, the
